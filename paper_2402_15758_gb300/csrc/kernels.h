@@ -138,12 +138,15 @@ int chain_add_row(ChainPlan* plan, int kind, int wait, const ChainRow& row, char
 cudaError_t chain_launch(const ChainPlan& plan, cudaStream_t s);
 
 // ----------------------------------------------------------------------------
-// fp32 linear (SIMT, exact fp32 FMA order per output)
+// fp32 linear (SIMT, fixed fp32 FMA order per output)
 // ----------------------------------------------------------------------------
 // skip (optional, device): when *skip != 0 at run time the launch does nothing (its
-// output was provided another way, e.g. by the trigram cache).
+// output was provided another way, e.g. by the trigram cache).  W2 (optional, N2 rows):
+// a second weight whose outputs follow W's in Y.  early_w: no kernel of the stream
+// writes the weights, so they may be read before the launch's dependency wait.
 cudaError_t f32_linear(int M, int N, int K, const float* X, int ldx, const float* W, float* Y,
-                       int ldy, int epi, cudaStream_t s, const int* skip = nullptr);
+                       int ldy, int epi, cudaStream_t s, const int* skip = nullptr, const float* W2 = nullptr,
+                       int N2 = 0, bool early_w = false);
 
 // ----------------------------------------------------------------------------
 // attention over the paged KV cache with a per-query ancestor bitmask

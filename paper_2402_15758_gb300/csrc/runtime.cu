@@ -340,11 +340,9 @@ cudaError_t run_lin(chimera_ctx* ctx, const Lin& l) {
   if (l.N == 0 || filtered(ctx, CHIMERA_KIND_LINEAR)) return cudaSuccess;  // N = 0: folded into the previous site
   Scope sc(ctx, CHIMERA_KIND_LINEAR, l.bytes);
   if (l.tc) return tc_linear_launch(l.tp, ctx->stream);
-  cudaError_t e = f32_linear(l.M, l.N, l.K, static_cast<const float*>(l.X), l.ldx, static_cast<const float*>(l.W),
-                             static_cast<float*>(l.Y), l.ldy, l.epi, ctx->stream, l.skip);
-  if (e != cudaSuccess || !l.W2) return e;
-  return f32_linear(l.M, l.N2, l.K, static_cast<const float*>(l.X), l.ldx, static_cast<const float*>(l.W2),
-                    static_cast<float*>(l.Y) + l.N, l.ldy, l.epi, ctx->stream, l.skip);
+  return f32_linear(l.M, l.N, l.K, static_cast<const float*>(l.X), l.ldx, static_cast<const float*>(l.W),
+                    static_cast<float*>(l.Y), l.ldy, l.epi, ctx->stream, l.skip, static_cast<const float*>(l.W2), l.N2,
+                    true);
 }
 
 bool make_lin(chimera_ctx* ctx, Lin* l, int M, int N, int K, const void* X, const void* X_lo, int ldx,

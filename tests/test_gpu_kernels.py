@@ -101,6 +101,26 @@ def test_linear_fp32(M, N, K):
     assert _rel_rows(Y.cpu().numpy(), X.double().numpy() @ W.double().numpy().T) <= 1e-5
 
 
+# one row / few rows / full and ragged 16-row tiles; K below, at and past the 512-wide chunk,
+# with and without 16-byte rows; enough features that a warp takes two
+@pytest.mark.parametrize("M,N,K", [(1, 7, 1), (1, 768, 359), (3, 130, 512), (5, 33, 516), (16, 256, 688),
+                                   (17, 1001, 513), (64, 1300, 1028), (33, 2048, 30)])
+@pytest.mark.parametrize("epi", [0, 1, 2])
+def test_linear_fp32_edges(M, N, K, epi):
+    g = torch.Generator().manual_seed(M * N + K)
+    X = torch.randn(M, K, generator=g)
+    W = torch.randn(N, K, generator=g) * 0.05
+    Y0 = torch.randn(M, N, generator=g)
+    Y = Y0.cuda()
+    pkg.op_linear(X.cuda(), W.cuda(), Y, epi=epi)
+    torch.cuda.synchronize()
+    ref = X.double().numpy() @ W.double().numpy().T
+    ref = {0: ref, 1: co.silu(ref), 2: Y0.double().numpy() + ref}[epi]
+    # fp32 sums of K terms in at most K / 32 + 5 roundings of 2^-24 each, against a row maximum of
+    # at least the sums' own size: 37 * 6e-8 = 2.2e-6 at K = 1028
+    assert _rel_rows(Y.cpu().numpy(), ref) <= 1e-5
+
+
 def _random_tree_anc(n, rng):
     parent = [-1] + [int(rng.integers(0, j)) for j in range(1, n)]
     anc = []
