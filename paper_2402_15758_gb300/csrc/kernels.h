@@ -43,8 +43,43 @@ struct TcLinearParams {
   long long zero_floats;
 };
 
+// The same linear for many rows of split activations, on CTA pairs (linear_pair.cu).
+struct TcPairParams {
+  CUtensorMap tmA, tmA2;  // W, optional W2: box 128 x 64
+  CUtensorMap tmB, tmB2;  // X, X_lo: box TT x 64
+  int M, N;
+  int halves, half_split; // 128-feature halves in all, and those taken from W
+  int TT;                 // tokens per tile (<= 128)
+  int tok_tiles, feat_tiles, kblocks, stages;
+  int width;              // pairs per group: token tiles that share the weight tiles in time
+  uint32_t units;         // of a group: (round of width token tiles, feature tile, K block)
+  int epi, out_f32, vec_red;
+  void* Y;
+  void* Y2;
+  int ldy;
+  float* ws;              // split partials: [grid][2][128 * TT] fp32
+  int* counters;          // [2 * tiles], all zero between launches
+  int* err;
+  unsigned long long wait_ns;
+  const int* skip;
+  float* zero;
+  long long zero_floats;
+};
+struct TcPairPlan {
+  TcPairParams p;
+  int grid = 0;  // 0: not used
+  size_t smem = 0;
+};
+// Fill the plan (arguments already checked by tc_linear_plan): 0, -1 when linear_tc.cu is
+// the better kernel or the shape is out of this one's range, -2 when a tensor map cannot be encoded.
+int tc_pair_plan(TcPairPlan* plan, int M, int N1, int N2, int K, const void* X, const void* X_lo, int ldx, const void* W,
+                 const void* W2, void* Y, void* Y_lo, int ldy, int epi, int out_f32, float* ws, int* counters, int* err,
+                 unsigned long long wait_ns, float* zero, long long zero_floats);
+cudaError_t tc_pair_launch(const TcPairPlan& plan, cudaStream_t s);
+
 struct TcLinearPlan {
   TcLinearParams p;
+  TcPairPlan pair;  // used instead of p when its grid is set
   int grid = 0;
   size_t smem = 0;
   double weight_bytes = 0;  // algorithmic bytes streamed per launch (W once)

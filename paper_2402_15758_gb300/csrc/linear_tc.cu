@@ -56,6 +56,11 @@ constexpr int CTAS_PER_SM = CHIMERA_LIN_CTAS_PER_SM;
 constexpr int PIPE_SMEM = CHIMERA_LIN_PIPE_KB * 1024;
 constexpr int MAX_BN = 256;
 constexpr int MAX_TILES = 8192;
+// Split activations of more than PAIR_ROWS rows go to linear_pair.cu.  Up to 128 rows this
+// kernel reads the weights once as well and starts faster (128 rows, 12288 x 4096: 26.1 us
+// here, 27.9 there); past 128 it would read them once per token tile (136 rows: 41.5, 33.9).
+// One-term activations stay here: a token tile is 256 rows, its work half of a split's.
+constexpr int PAIR_ROWS = 128;
 
 
 // Stream-K partition in 32-bit arithmetic (the host checks units * grid < 2^32).
@@ -542,6 +547,13 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && N % 4 == 0) ? 1 : 0;
   plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 16 * 33 * sizeof(float);
   plan->weight_bytes = 2.0 * N * K;
+  plan->pair.grid = 0;
+  if (X_lo && M > PAIR_ROWS) {
+    const int st = tc_pair_plan(&plan->pair, M, N1, W2 ? N2 : 0, K, X, X_lo, ldx, W, W2, Y, Y_lo, ldy, epi, out_f32, ws,
+                                counters, err, p.wait_ns, zero, p.zero_floats);
+    if (st == -2) return fail("tensor map of the pair kernel");
+    if (st != 0) plan->pair.grid = 0;
+  }
   return 0;
 }
 
@@ -556,6 +568,7 @@ bool g_attr_set[LIN_MAX_DEVICES];
 std::atomic<unsigned long long> g_lin_wait_ns{kDefaultWaitNs};
 
 cudaError_t tc_linear_launch(const TcLinearPlan& plan, cudaStream_t s) {
+  if (plan.pair.grid) return tc_pair_launch(plan.pair, s);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

@@ -370,8 +370,8 @@ bool make_lin(chimera_ctx* ctx, Lin* l, int M, int N, int K, const void* X, cons
     ctx->err = msg;
     return false;
   }
-  l->tp.p.wait_ns = kDefaultWaitNs;  // the timeout hook applies to the stateless entry points only
-  l->tp.p.skip = skip;
+  l->tp.p.wait_ns = l->tp.pair.p.wait_ns = kDefaultWaitNs;  // the timeout hook applies to the stateless entry points only
+  l->tp.p.skip = l->tp.pair.p.skip = skip;
   return true;
 }
 

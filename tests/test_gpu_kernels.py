@@ -78,6 +78,33 @@ def test_linear_bf16_split_operand(M, N, K):
     assert _rel_rows(Y.cpu().numpy(), ref) > 1e-4
 
 
+# the CTA-pair kernel: split activations of more than 128 rows with at least 14 stages per
+# pair.  Ragged token tiles (2 of 80 rows, 3 of 96, 9 in two rounds of 5), an odd number of
+# 128-feature halves, columns that are no multiple of 4, a ragged last K block
+@pytest.mark.parametrize("M,N,K", [(129, 4224, 4096), (256, 2050, 8000), (257, 1000, 12296), (640, 1536, 5000),
+                                   (1100, 1024, 3400)])
+@pytest.mark.parametrize("epi,out_f32", [(0, True), (1, False), (2, True)])
+def test_linear_pair_kernel(M, N, K, epi, out_f32):
+    g = torch.Generator().manual_seed(M + N + K)
+    X32 = torch.randn(M, K, generator=g)
+    hi = X32.to(torch.bfloat16)
+    lo = (X32 - hi.float()).to(torch.bfloat16)
+    W = (torch.randn(N, K, generator=g) * 0.02).to(torch.bfloat16)
+    Y0 = torch.randn(M, N, generator=g).to(torch.float32 if out_f32 else torch.bfloat16)
+    ref = (hi.cuda().double() + lo.cuda().double()) @ W.cuda().double().T
+    ref = {0: ref, 1: ref * torch.sigmoid(ref), 2: Y0.cuda().double() + ref}[epi].cpu().numpy()
+    got = []
+    for _ in range(2):
+        Y = Y0.cuda()
+        pkg.op_linear(hi.cuda(), W.cuda(), Y, epi=epi, out_f32=out_f32, X_lo=lo.cuda())
+        pkg.op_sync()
+        got.append(Y.float().cpu().numpy())
+    # chains of at most 128 truncated fp32 steps (2^-23 each, partly cancelling), or one rounding to bf16
+    assert _rel_rows(got[1], ref) <= (1.6e-5 if out_f32 else 8e-3)
+    if epi != 2:  # stored outputs are summed in a fixed order
+        assert np.array_equal(got[0], got[1])
+
+
 def test_linear_deterministic():
     g = torch.Generator().manual_seed(5)
     X = torch.randn(64, 4096, generator=g).to(torch.bfloat16).cuda()
