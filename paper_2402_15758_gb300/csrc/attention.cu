@@ -18,6 +18,7 @@
 
 #include <mutex>
 
+#include "attention.cuh"
 #include "common.cuh"
 #include "launch.cuh"
 #include "kernels.h"
@@ -48,7 +49,7 @@ constexpr int MAX_SPLITS = 16;
 // thread takes part: first the per-query weights exp(m_s - M) / L into shared memory,
 // then the outputs, 4 dims per item, up to 8 items x 4 splits of loads in flight.
 template <typename T>
-__device__ void combine_splits(const AttnParams& p, const float* wsb, int nq, int hd, int b, int h, T* out,
+__device__ void combine_splits(const AttnParams& p, const float* wsb, int nq, int hd, int row0, int h, T* out,
                                T* out_lo, float* s_w /* [nq][MAX_SPLITS] */) {
   const size_t rec = hd + 4;
   for (int qi = threadIdx.x; qi < nq; qi += blockDim.x) {
@@ -115,7 +116,7 @@ __device__ void combine_splits(const AttnParams& p, const float* wsb, int nq, in
       const int it = it0 + j * nt;
       if (it >= items) continue;
       const int qi = it / c4n, c = (it % c4n) * 4;
-      const size_t o = static_cast<size_t>(b * p.q_rows + qi) * p.ldo + h * hd + c;
+      const size_t o = static_cast<size_t>(row0 + qi) * p.ldo + h * hd + c;
       store_act4(out, out_lo, o, acc[j]);
     }
   }
@@ -133,13 +134,12 @@ __global__ void __launch_bounds__(WARPS * 32) attn_kernel(const AttnParams p) {
   float* Qs = Vs + KT * HD;         // [nq][HD]
   __shared__ int s_last;
 
-  const int s = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  const int s = blockIdx.x, h = blockIdx.y;
+  const QueryBlock qb(p, blockIdx.z);
+  const int b = qb.b, nctx = qb.nctx, nloc = qb.nloc, nq = qb.nq;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nctx = p.n_ctx[b];
-  const int nloc = p.n_local_dev ? p.n_local_dev[b] : p.n_local;
-  const int nq = p.nq_dev ? p.nq_dev[b] : p.nq;
   const int total = nctx + nloc;
-  const int ntiles = (total + KT - 1) / KT;
+  const int ntiles = nq > 0 ? (total + KT - 1) / KT : 0;
   const int tps = (ntiles + p.splits - 1) / p.splits;
   const int t0 = s * tps;
   const int t1 = min(ntiles, t0 + tps);
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_kernel(const AttnParams p) {
 
   for (int idx = threadIdx.x; idx < nq * HD; idx += blockDim.x) {
     const int i = idx / HD, dd = idx % HD;
-    Qs[idx] = q[static_cast<size_t>(b * p.q_rows + i) * p.ldq + h * HD + dd];
+    Qs[idx] = q[static_cast<size_t>(qb.row0 + i) * p.ldq + h * HD + dd];
   }
 
   float m[QPW], l[QPW], acc[QPW][DPL];
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_kernel(const AttnParams p) {
         const float inv = l[qq] > 0.f ? 1.f / l[qq] : 0.f;
 #pragma unroll
         for (int r = 0; r < DPL; ++r)
-          store_act(out, out_lo, static_cast<size_t>(b * p.q_rows + qi) * p.ldo + h * HD + lane + 32 * r,
+          store_act(out, out_lo, static_cast<size_t>(qb.row0 + qi) * p.ldo + h * HD + lane + 32 * r,
                     acc[qq][r] * inv);
       }
     }
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_kernel(const AttnParams p) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  combine_splits(p, wsb, nq, HD, b, h, out, out_lo, sm);  // the K/V tile area is free now
+  combine_splits(p, wsb, nq, HD, qb.row0, h, out, out_lo, sm);  // the K/V tile area is free now
   if (threadIdx.x == 0) p.counters[b * p.H + h] = 0;
 }
 
@@ -280,7 +280,7 @@ cudaError_t launch(const AttnParams& p, cudaStream_t s) {
       attr[dev] = true;
     }
   }
-  dim3 grid(p.splits, p.H, p.B);
+  dim3 grid(p.splits, p.H, p.B * std::max(1, p.q_blocks));
   launch_pdl(attn_kernel<TKV, T, HD>, dim3(grid), dim3(WARPS * 32), smem, s, p);
   return cudaGetLastError();
 }
@@ -301,6 +301,9 @@ int attn_pick_splits(int dtype, int hd, int planes, int B, int H, int want) {
 cudaError_t attention(const AttnParams& p, int dtype, cudaStream_t s) {
   if (p.nq_max > WARPS * QPW || p.n_local > 64 || p.splits > MAX_SPLITS || p.splits < 1) return cudaErrorInvalidValue;
   if (p.planes != 2 && !(p.planes == 4 && dtype == 1)) return cudaErrorInvalidValue;
+  // blocks of prompt rows: device row counts, no fused projections, one split per block
+  if (p.q_blocks > 1 && (p.qkv || !p.nq_dev || !p.n_local_dev || p.q_local0 != 0 || p.nq != 64 || p.n_local != 64 || p.splits != 1))
+    return cudaErrorInvalidValue;
   if (dtype == 0) {
     if (p.qkv) return cudaErrorInvalidValue;
     if (p.hd == 64) return launch<float, float, 64>(p, s);

@@ -27,6 +27,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "attention.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   float* s_lh = s_xm + 4 * NQ;       // [2 halves][64] partial row sums
   volatile int* abort = s_abort;
 
-  const int s = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  const int s = blockIdx.x, h = blockIdx.y;
   const int S = gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   bf16* pool = static_cast<bf16*>(const_cast<void*>(p.pool)) + static_cast<size_t>(p.layer) * p.pool_layer_stride;
@@ -198,7 +199,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   if (warp == MMA_WARP) tmem_alloc(tmem_slot, TMEM_COLS);
 
   if (!p.prewait_kv) pdl_wait();
-  const int nctx = p.n_ctx[b];
+  const QueryBlock qb(p, blockIdx.z);  // (early reads: n_ctx; the device counts are used by prompt chunks only)
+  const int b = qb.b, nctx = qb.nctx;
   // Local mode (fused projections, local rows starting at row 0: verify, prefill, plain
   // decoding, the draft's first sub-step): every local row is written by this launch,
   // so the local rows form one extra tile that the CTA owning it builds in shared
@@ -207,7 +209,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   // (so it goes to the CTA with the fewest committed tiles) and that CTA's first tile
   // (stage 0, free at start).  Otherwise the tiles cover slots [0, nctx + n_local).
   const bool lmode = p.qkv != nullptr && p.q_local0 == 0;
-  const int ntiles = lmode ? (nctx + KT - 1) / KT : (nctx + p.n_local + KT - 1) / KT;  // tiles of the pool
+  // tiles of the pool (a block of prompt rows past its sequence's last row has none)
+  const int ntiles = lmode              ? (nctx + KT - 1) / KT
+                     : p.q_blocks <= 1 ? (nctx + p.n_local + KT - 1) / KT
+                     : qb.nq > 0       ? (nctx + qb.nloc + KT - 1) / KT
+                                       : 0;
   const int T = ntiles + (lmode ? 1 : 0);
   const int tps = (T + S - 1) / S;
   const int v0 = min(T, s * tps), v1 = min(T, v0 + tps);
@@ -278,8 +284,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   }
   pdl_trigger();
 
-  const int nloc = min(p.n_local_dev ? p.n_local_dev[b] : p.n_local, p.n_local);
-  const int nq = p.nq_dev ? p.nq_dev[b] : p.nq;
+  const int nloc = p.q_blocks > 1 ? qb.nloc : min(p.n_local_dev ? p.n_local_dev[b] : p.n_local, p.n_local);
+  const int nq = p.q_blocks > 1 ? qb.nq : p.nq_dev ? p.nq_dev[b] : p.nq;
   const int total = nctx + nloc;
   const int dm = p.H * HD;
 
@@ -288,8 +294,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     const int r = it >> 3, j = it & 7;  // row, 8-dim chunk j of the first half (dims 8j.., 64 + 8j..)
     float lo_half[8], hi_half[8];
     if (r < nq) {
-      const float* src = p.qkv ? p.qkv + static_cast<size_t>(b * p.q_rows + r) * p.ldqkv + h * HD + 8 * j
-                               : p.q + static_cast<size_t>(b * p.q_rows + r) * p.ldq + h * HD + 8 * j;
+      const float* src = p.qkv ? p.qkv + static_cast<size_t>(qb.row0 + r) * p.ldqkv + h * HD + 8 * j
+                               : p.q + static_cast<size_t>(qb.row0 + r) * p.ldq + h * HD + 8 * j;
       const float4 a0 = *reinterpret_cast<const float4*>(src), a1 = *reinterpret_cast<const float4*>(src + 4);
       const float4 b0 = *reinterpret_cast<const float4*>(src + HD / 2),
                    b1 = *reinterpret_cast<const float4*>(src + HD / 2 + 4);
@@ -810,7 +816,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
       }
     }
-    const size_t o_idx = static_cast<size_t>(b * p.q_rows + q0 + rl) * p.ldo + h * HD + c;
+    const size_t o_idx = static_cast<size_t>(qb.row0 + q0 + rl) * p.ldo + h * HD + c;
     store_act4(out, out_lo, o_idx, acc);
   }
 }
@@ -865,7 +871,7 @@ cudaError_t launch_tc(const AttnParams& p, cudaStream_t s) {
     ++na;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.splits, p.H, p.B);
+  cfg.gridDim = dim3(p.splits, p.H, p.B * std::max(1, p.q_blocks));
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = tc_smem<SPLIT>();
   cfg.stream = s;

@@ -212,6 +212,11 @@ struct AttnParams {
   float* ws;              // [B][H][splits][nq_max][hd + 4] (output, max, sum, pad)
   int* counters;          // [B][H], zero between launches
   int nq_max;
+  // Prompt rows (qkv null): blocks of 64 query rows per sequence, 0 meaning one.  Block j
+  // takes rows 64 j .. of the sequence's query rows, nq, n_local and their device
+  // counts covering all of them (nq and n_local then per block: 64); its context is the n_ctx
+  // committed rows and the 64 j local rows before it.
+  int q_blocks;
   // Fused RoPE + KV write (bf16 models, head_dim 128).  With qkv set, the queries and
   // the nq fresh local rows come from the fp32 projections: row (b * q_rows + i) holds
   // q at column h*hd, k at H*hd + h*hd, v at 2*H*hd + h*hd.  Query / fresh row i sits at

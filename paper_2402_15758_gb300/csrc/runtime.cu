@@ -19,7 +19,13 @@ using namespace chimera;
 
 namespace {
 
-constexpr int CHUNK = 64;        // prefill rows per sequence per pass (one 64-bit mask)
+constexpr int CHUNK = 64;        // granule of prompt chunks: a query block (one 64-bit mask)
+// Rows of a prefill pass over all sequences.  A pass streams every weight once, so its
+// linears are bound by HBM up to about 128 rows and by the tensor cores from there on:
+// 12288 x 4096 runs at 0.64 PFLOP/s with 64 rows, 1.24 with 256, 1.63 with 1024 and no
+// faster with 2048.  A 600-token prompt of the 4096-wide model: 34.9 ms in passes of 64
+// rows, 14.6 ms in one pass of 640.
+constexpr int PREFILL_ROWS = 1024;
 constexpr int LOG_CAP = 4096;    // per-step accepted-count log
 constexpr int MAX_KMAX = 8;
 constexpr int CHAIN_BAR_INTS = 16;     // >= CHAIN_MAX_STEPS + 1 counters per chain launch
@@ -202,6 +208,8 @@ struct chimera_ctx {
 
   // activations
   int R = 0;
+  int prefill_rows = 0;  // rows of a prefill pass over all sequences (capacity)
+  int chunk = CHUNK;     // prefill rows per sequence per pass, a multiple of CHUNK
   float* x = nullptr;
   // GEMM operands in the model dtype; *_lo = the bf16 rounding residuals (split mode)
   void *xn = nullptr, *xn_lo = nullptr, *ao = nullptr, *ao_lo = nullptr, *hf = nullptr, *hf_lo = nullptr;
@@ -413,7 +421,7 @@ int att_splits(const chimera_ctx* ctx, int B, int nq, int n_keys) {
 cudaError_t run_attention(chimera_ctx* ctx, bool draft_pool, int layer, int nq, const int* nq_dev, int q_local0,
                           int n_local, const int* n_local_dev, const unsigned long long* anc, int q_rows, int splits,
                           int nq_max, double bytes, const float* qkv = nullptr, int pos_base = 0,
-                          const int* pos_off = nullptr) {
+                          const int* pos_off = nullptr, int q_blocks = 0) {
   if (filtered(ctx, CHIMERA_KIND_ATTENTION)) return cudaSuccess;
   if (qkv && !ctx->filter_kind &&
       !(ctx->dtype == 1 && (ctx->last_kind == CHIMERA_KIND_LINEAR || ctx->last_kind == CHIMERA_KIND_CHAIN))) {
@@ -460,6 +468,7 @@ cudaError_t run_attention(chimera_ctx* ctx, bool draft_pool, int layer, int nq, 
   p.ws = ctx->att_ws;
   p.counters = ctx->att_cnt;
   p.nq_max = nq_max;
+  p.q_blocks = q_blocks;
   if (attn_ws_floats(p.B, p.H, splits, nq_max, p.hd) > ctx->att_ws_floats) return cudaErrorInvalidValue;
   return attention(p, ctx->dtype, ctx->stream);
 }
@@ -573,13 +582,14 @@ cudaError_t enqueue_layer(chimera_ctx* ctx, int l, const Lin* lin, int rows, int
   const bool z = !ctx->tc_zero;
   RUN(run_norm(ctx, ctx->x, w.attn_norm, rows, (z || l == 0) ? ctx->qkv : nullptr, 3 * d));
   RUN(run_lin(ctx, lin[0]));
-  if (attn_fuses_rope(ctx->dtype, ctx->hd)) {
+  const int blocks = (rows_per_seq + CHUNK - 1) / CHUNK, nq = std::min(rows_per_seq, CHUNK);
+  if (blocks == 1 && attn_fuses_rope(ctx->dtype, ctx->hd)) {
     RUN(run_attention(ctx, false, l, rows_per_seq, valid, 0, rows_per_seq, valid, anc, rows_per_seq, splits,
                       rows_per_seq, kv_bytes, ctx->qkv, 0, pos_off));
-  } else {
+  } else {  // several blocks of prompt rows read one another's keys: RoPE and the KV write come first
     RUN(run_rope(ctx, false, l, ctx->qkv, 3 * d, 0, d, 2 * d, rows_per_seq, valid, 0, 0, 0, pos_off));
-    RUN(run_attention(ctx, false, l, rows_per_seq, valid, 0, rows_per_seq, valid, anc, rows_per_seq, splits,
-                      rows_per_seq, kv_bytes));
+    RUN(run_attention(ctx, false, l, nq, valid, 0, nq, valid, anc, rows_per_seq, splits, nq, kv_bytes, nullptr, 0,
+                      nullptr, blocks));
   }
   RUN(run_lin(ctx, lin[1]));
   RUN(run_norm(ctx, ctx->x, w.ffn_norm, rows, z ? ctx->gu : nullptr, 2 * ctx->F));
@@ -968,7 +978,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
   if (!make_lin(ctx, &ctx->ar_lm, B, V, d, ctx->hfin, ctx->hfin_lo, d, ctx->lm_head, ctx->logits, nullptr, V, ACC,
                 f32))
     return false;
-  if (!layer_plans(ctx->pre, B * CHUNK)) return false;
+  if (!layer_plans(ctx->pre, B * ctx->chunk)) return false;
   if (!make_lin(ctx, &ctx->ver_lm, B * N, V, d, ctx->hfin, ctx->hfin_lo, d, ctx->lm_head, ctx->logits, nullptr, V,
                 ACC, f32))
     return false;
@@ -976,7 +986,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
                 ACC, f32))
     return false;
   const void* dl_kv = eoff(ctx, const_cast<void*>(ctx->draft.wqkv), static_cast<size_t>(d) * d);
-  if (!make_lin(ctx, &ctx->pre_dkv, B * CHUNK, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, ACC, f32))
+  if (!make_lin(ctx, &ctx->pre_dkv, B * ctx->chunk, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, ACC, f32))
     return false;
   if (!make_lin(ctx, &ctx->commit_kv, B * ctx->D1, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, ACC,
                 f32))
@@ -1008,7 +1018,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
                   ctx->hlog + static_cast<size_t>(k) * B * V, nullptr, V, ACC, f32))
       return false;
   ctx->att_splits_ver = att_splits(ctx, B, N, ctx->plan_keys + N);
-  ctx->att_splits_pre = att_splits(ctx, B, CHUNK, ctx->plan_keys);
+  ctx->att_splits_pre = ctx->chunk > CHUNK ? 1 : att_splits(ctx, B, CHUNK, ctx->plan_keys);
   ctx->att_splits_draft = att_splits(ctx, B, 1, ctx->plan_keys);
   ctx->att_splits_ar = att_splits(ctx, B, 1, ctx->plan_keys + 1);
   if (ctx->use_chain && !build_chains(ctx, B)) return false;
@@ -1254,8 +1264,11 @@ chimera_status chimera_init(const chimera_config* cfg, const chimera_weights* w,
   ctx->NB = B * ctx->max_pages;
   ctx->kv_layer_stride = static_cast<long long>(ctx->NB) * ctx->H * ctx->kv_planes * 16 * ctx->hd;
   ctx->max_pos = ctx->cap + 64;
-  ctx->R = B * std::max(N, CHUNK);
-  const int Rc = B * std::max(CHUNK, ctx->D1);
+  ctx->prefill_rows = B * CHUNK;
+  if (ctx->prefill_rows < PREFILL_ROWS)
+    ctx->prefill_rows = std::min(PREFILL_ROWS, B * ((ctx->cap + CHUNK - 1) / CHUNK * CHUNK));
+  ctx->R = std::max(B * N, ctx->prefill_rows);
+  const int Rc = std::max(ctx->prefill_rows, B * ctx->D1);
   bool ok = true;
   const size_t Rx = static_cast<size_t>(std::max(ctx->R, Rc));
   const bool sp = ctx->split != 0;
@@ -1463,6 +1476,10 @@ chimera_status chimera_prefill(chimera_ctx* ctx, int batch, const int32_t* token
   }
   ctx->batch = batch;
   ctx->plan_keys = max_len;
+  // as few passes as the workspace allows, of equal length
+  const int most = std::max(CHUNK, ctx->prefill_rows / batch / CHUNK * CHUNK);
+  const int passes = (max_len + most - 1) / most;
+  ctx->chunk = ((max_len + passes - 1) / passes + CHUNK - 1) / CHUNK * CHUNK;
   if (!build_plans(ctx, batch)) return CHIMERA_EINVAL;
   for (int b = 0; b < batch; ++b) {
     chimera_status st = ensure_blocks(ctx, b, lens[b] + need);
@@ -1487,30 +1504,30 @@ chimera_status chimera_prefill(chimera_ctx* ctx, int batch, const int32_t* token
     CK(cudaStreamSynchronize(s));
   }
   ctx->host_n.assign(batch, 0);
-  const int d = ctx->d, B = batch;
-  const int chunks = (max_len + CHUNK - 1) / CHUNK;
+  const int d = ctx->d, B = batch, C = ctx->chunk;
+  const int chunks = (max_len + C - 1) / C;
   const void* dl_norm = ctx->draft.attn_norm;
   for (int cidx = 0; cidx < chunks; ++cidx) {
     int* hv = ctx->h_stage;
     for (int b = 0; b < B; ++b) {
-      const int v = std::max(0, std::min(CHUNK, lens[b] - cidx * CHUNK));
+      const int v = std::max(0, std::min(C, lens[b] - cidx * C));
       hv[b] = v;
-      const int li = lens[b] - 1 - cidx * CHUNK;
-      hv[64 + b] = (li >= 0 && li < CHUNK) ? li : -1;
+      const int li = lens[b] - 1 - cidx * C;
+      hv[64 + b] = (li >= 0 && li < C) ? li : -1;
     }
     CK(cudaMemcpyAsync(ctx->d_valid, hv, B * sizeof(int), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(ctx->d_last, hv + 64, B * sizeof(int), cudaMemcpyHostToDevice, s));
-    CK(embed(ctx->dtype, ctx->embed, d, ctx->V, ctx->x, B * CHUNK, CHUNK, nullptr, ctx->d_tok, ctx->tok_stride, ctx->d_n,
+    CK(embed(ctx->dtype, ctx->embed, d, ctx->V, ctx->x, B * C, C, nullptr, ctx->d_tok, ctx->tok_stride, ctx->d_n,
              ctx->d_valid, ctx->d_err, s));
     for (int l = 0; l < ctx->L; ++l)
-      CK(enqueue_layer(ctx, l, &ctx->pre[5 * l], B * CHUNK, CHUNK, ctx->d_valid, nullptr, ctx->d_chain,
+      CK(enqueue_layer(ctx, l, &ctx->pre[5 * l], B * C, C, ctx->d_valid, nullptr, ctx->d_chain,
                        ctx->att_splits_pre, 0));
-    CK(run_final_norm(ctx, B * CHUNK, false));
+    CK(run_final_norm(ctx, B * C, false));
     // draft-layer K/V of the chunk's H_LLM rows
-    CK(run_norm(ctx, ctx->hfin32, dl_norm, B * CHUNK, ctx->kvtmp, 2 * d));
+    CK(run_norm(ctx, ctx->hfin32, dl_norm, B * C, ctx->kvtmp, 2 * d));
     CK(run_lin(ctx, ctx->pre_dkv));
-    CK(run_rope(ctx, true, 0, ctx->kvtmp, 2 * d, -1, 0, d, CHUNK, ctx->d_valid, 0, 0, 0, nullptr));
-    CK(launch_prefill_advance(ctx->dtype, ctx->hfin32, d, CHUNK, ctx->d_valid, ctx->d_last, ctx->d_n, ctx->headin,
+    CK(run_rope(ctx, true, 0, ctx->kvtmp, 2 * d, -1, 0, d, C, ctx->d_valid, 0, 0, 0, nullptr));
+    CK(launch_prefill_advance(ctx->dtype, ctx->hfin32, d, C, ctx->d_valid, ctx->d_last, ctx->d_n, ctx->headin,
                               ctx->headin_lo, B, s));
     CK(cudaStreamSynchronize(s));  // the staging buffer is reused by the next chunk
   }

@@ -111,8 +111,8 @@ __global__ void rope_kv_kernel(const RopeKvParams p) {
   const int nvalid = p.valid ? p.valid[b] + p.valid_plus : p.rows_per_seq;
   const bool write_kv = i < nvalid;
   const int half = p.hd / 2;
-  if (pos < 0 || pos >= p.max_pos) {
-    if (threadIdx.x == 0) atomicOr(p.err, ERR_CAPACITY);
+  if (pos < 0 || pos >= p.max_pos) {  // rows past the valid ones may lie past the table: unused
+    if (write_kv && threadIdx.x == 0) atomicOr(p.err, ERR_CAPACITY);
     pos = 0;
   }
   int page = -1;

@@ -402,3 +402,27 @@ def test_bf16_ar_steps_match_oracle(name, fused):
     assert ctx.read("n").tolist() == [len(s) - 1 for s in seqs]
     ctx.close()
     print(f"{name} AR: 5 steps x {B} seqs, near-tie flags {flags}")
+
+
+# prompts of several 64-row query blocks per pass, ragged (a sequence that ends blocks before
+# the others), and of more rows than one pass takes
+@pytest.mark.parametrize("name,lens", [("tiny", [200]), ("tiny", [7, 130, 64]), ("mini", [65, 300, 64]), ("mini", [1100])])
+def test_prefill_chunks(name, lens):
+    cfg, w_cpu, w_dev = _setup(name)
+    tol = tol_of(cfg)
+    W = co.OracleWeights(w_cpu)
+    rng = np.random.default_rng(len(lens))
+    prompts = [rng.integers(0, cfg["vocab"], n).tolist() for n in lens]
+    cap = max(lens) + 160
+    ctx = pkg.Chimera(cfg, w_dev, max_batch=len(lens), max_seq_len=cap)
+    ctx.prefill(prompts)
+    logits = ctx.read("prefill_logits")
+    assert ctx.read("n").tolist() == lens
+    for b, x in enumerate(prompts):
+        st = co.prefill(W, cfg, x, cap)
+        assert rel_rows(logits[b], st.prefill_logits) <= tol
+        for layer in (0, cfg["n_layers"] - 1, -1):
+            k, v = ctx.read_kv(layer, b, 0, len(x))
+            rk = st.dK[:len(x)] if layer < 0 else st.K[layer, :len(x)]
+            rv = st.dV[:len(x)] if layer < 0 else st.V[layer, :len(x)]
+            assert rel_rows(k, rk) <= tol and rel_rows(v, rv) <= tol, (b, layer)
