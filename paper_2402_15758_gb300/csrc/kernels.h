@@ -246,6 +246,10 @@ int attn_pick_splits(int dtype, int hd, int planes, int B, int H, int want);
 // [outer][pitch_elems] with an inner extent of `inner` elements; 0 on success.
 int encode_2d_bf16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_elems,
                    uint32_t box_inner, uint32_t box_outer);
+// 5D bf16 tensor map (128-byte swizzle, zero fill out of bounds), strides of dimensions
+// 1..4 in bytes; 0 on success.
+int encode_5d_bf16(CUtensorMap* map, const void* base, const uint64_t (&dims)[5], const uint64_t (&strides)[4],
+                   const uint32_t (&box)[5]);
 // Tensor-core tree attention (bf16 planes, head_dim 128; splits <= 8 form one cluster).
 cudaError_t attention_tc(const AttnParams& p, cudaStream_t s);
 int attention_tc_splits(int planes, int BH, int want);

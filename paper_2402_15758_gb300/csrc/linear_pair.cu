@@ -92,20 +92,23 @@ __device__ __forceinline__ void tma_load_2d_pair_hint(void* smem_dst, const CUte
 }
 // D (both CTAs' tensor memory) (+)= A . B^T with 128 rows of A and N / 2 rows of B in each CTA.
 __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                 uint32_t accumulate) {
+                                                 uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected)
       : "memory");
 }
 // Arrive on the barrier at this offset in both CTAs once every MMA issued so far is done.
-__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar, uint32_t elected) {
   asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %2, 0;\n\t"
+      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
           smem_u32(bar)),
-      "h"(static_cast<uint16_t>(3))
+      "h"(static_cast<uint16_t>(3)), "r"(elected)
       : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
@@ -281,45 +284,53 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
   } else if (warp == 1) {
     pdl_wait();
     pdl_trigger();
-    if (lane == 0 && !rank) {
-      // ---------------- MMA issuer of the pair ----------------
+    __syncwarp();
+    if (!rank) {
+      // ---------------- MMA issuer of the pair (the whole warp, one elected lane issues) ----------------
+      const uint32_t elected = elect_one();
       const uint32_t n = 2 * p.TT;
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
+      const uint64_t desc0 = sw128_desc(smem_u32(smem));
       int stage = 0, buf = 0;
       uint32_t phase = 0, aphase = 0;
-      for (uint32_t u = u_begin; u < u_end && !*abort;) {
+      bool ok = true;
+      for (uint32_t u = u_begin; ok && u < u_end;) {
         const uint32_t tile_end = min(u_end, (u / KB + 1) * KB);
         const uint32_t seg_end = min(tile_end, u + SEG_UNITS);
-        if (!mbar_wait(&tempty[buf], aphase ^ 1u, abort, p.wait_ns)) break;
+        ok = mbar_wait_warp(&tempty[buf], aphase ^ 1u, abort, p.wait_ns);
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * 256;
-        bool first = true;
-        for (; u < seg_end; ++u) {
-          if (!mbar_wait(&full[stage], phase, abort, p.wait_ns)) break;
+        uint32_t acc = 0;
+        for (; ok && u < seg_end; ++u) {
+          ok = mbar_wait_warp(&full[stage], phase, abort, p.wait_ns);
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * stage_bytes);
+          const uint64_t da = desc0 + static_cast<uint64_t>((stage * stage_bytes) >> 4);
+          const uint64_t db = da + static_cast<uint64_t>(A_BYTES >> 4);
 #pragma unroll
           for (int a = 0; a < BKA; ++a)
 #pragma unroll
-            for (int k = 0; k < ATOM / UK; ++k)
-              tc_mma_bf16_pair(d_tmem, sw128_desc(sa + a * A_ATOM + k * 32), sw128_desc(sa + A_BYTES + a * b_atom + k * 32),
-                               idesc, (first && a == 0 && k == 0) ? 0u : 1u);
-          first = false;
-          tc_commit_pair(&empty[stage]);
+            for (int k = 0; k < ATOM / UK; ++k) {
+              tc_mma_bf16_pair(d_tmem, da + static_cast<uint64_t>((a * A_ATOM + k * 32) >> 4),
+                               db + static_cast<uint64_t>((a * b_atom + k * 32) >> 4), idesc, acc, elected);
+              acc = 1;
+            }
+          tc_commit_pair(&empty[stage], elected);
           if (++stage == p.stages) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        tc_commit_pair(&tfull[buf]);
+        if (ok) tc_commit_pair(&tfull[buf], elected);
         buf ^= 1;
         if (buf == 0) aphase ^= 1u;
       }
-      if (*abort) {  // every MMA issued so far must complete before tensor memory is released
-        tc_commit_pair(drain);
+      if (!ok) {  // every MMA issued so far must complete before tensor memory is released
+        tc_commit_pair(drain, elected);
         mbar_wait_plain(drain, 0, 200000000ull);
       }
     }
+    __syncwarp();
   } else {
     // ---------------- epilogue ----------------
     pdl_wait();  // Y, the workspace and the counters are shared with earlier kernels

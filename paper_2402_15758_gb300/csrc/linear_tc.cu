@@ -5,8 +5,13 @@
 // Swap-AB: the weight tile (128 output features x 64 K) is the MMA's A operand
 // (UMMA M = 128) and the token tile (BN rows x 64 K, BN = 16..256) is its B operand,
 // so the skinny token dimension of the draft (1..8 rows) and of the tree verify
-// (16..256 rows) becomes the MMA N.  At these sizes the kernel is bound by streaming
-// W from HBM once.
+// (16..128 rows) becomes the MMA N.  At these sizes the kernel is bound by streaming
+// W from HBM once.  With X = hi + lo (BN <= 128) the lo rows follow the hi rows in B, one
+// MMA with N = 2 BN multiplies the weights with both, and the epilogue adds the two
+// halves of the columns: half the MMAs, the weight tile read from shared memory once, and
+// each half's fp32 accumulation half as many (truncating) steps long.  Measured (GB300, 64
+// rows, with the MMAs issued by a converged warp): 12288 x 4096 20.2 -> 18.4 us, 22016 x 4096
+// 32.1 -> 29.7 (6.07 TB/s), 4096 x 11008 18.6 -> 17.0; error against 64 bits 6.9e-6 -> 3.3e-6.
 //
 // Work split: stream-K.  The (feature tile, token tile, K block) units are cut into
 // gridDim.x equal contiguous ranges (one persistent CTA per SM), so every SM streams
@@ -142,8 +147,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
                                              ~static_cast<uintptr_t>(1023));
   const int a_atom = BM * ATOM * 2;     // one 128 x 64 weight box
   const int b_atom = p.BN * ATOM * 2;  // one BN x 64 activation box
-  const int b_bytes = b_atom * BKA;
-  const int stage_bytes = a_atom * BKA + (p.has_lo ? 2 : 1) * b_bytes;
+  const int terms = p.has_lo ? 2 : 1;
+  const int b_step = terms * b_atom;   // an atom's hi rows, then its lo rows
+  const int stage_bytes = a_atom * BKA + b_step * BKA;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes);
   uint64_t* empty = full + MAX_STAGES;
   uint64_t* tfull = empty + MAX_STAGES;
@@ -215,8 +221,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
         const int tt = t % p.tok_tiles;
 #pragma unroll
         for (int a = 0; a < BKA; ++a) {
-          tma_load_2d(sb + a * b_atom, &p.tmB, kb * BK + a * ATOM, tt * p.BN, bar);
-          if (p.has_lo) tma_load_2d(sb + b_bytes + a * b_atom, &p.tmB2, kb * BK + a * ATOM, tt * p.BN, bar);
+          tma_load_2d(sb + a * b_step, &p.tmB, kb * BK + a * ATOM, tt * p.BN, bar);
+          if (p.has_lo) tma_load_2d(sb + a * b_step + b_atom, &p.tmB2, kb * BK + a * ATOM, tt * p.BN, bar);
         }
       };
       // The weights do not depend on earlier kernels: request the first stages' weight
@@ -261,52 +267,53 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
   } else if (warp == 1) {
     pdl_wait();
     pdl_trigger();
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = idesc_bf16_m128(p.BN);
-      int stage = 0;
-      uint32_t phase = 0;
-      int buf = 0;
-      uint32_t aphase = 0;
-      for (uint32_t u = u_begin; u < u_end && !*abort;) {
-        const int t = static_cast<int>(u / KB);
-        const uint32_t seg_end = min(u_end, static_cast<uint32_t>(t + 1) * KB);
-        if (!mbar_wait(&tempty[buf], aphase ^ 1u, abort, p.wait_ns)) break;
+    // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+    __syncwarp();
+    const uint32_t elected = elect_one();
+    const uint32_t idesc = idesc_bf16_m128(terms * p.BN);
+    const uint64_t desc0 = sw128_desc(smem_u32(smem));
+    int stage = 0;
+    uint32_t phase = 0;
+    int buf = 0;
+    uint32_t aphase = 0;
+    bool ok = true;
+    for (uint32_t u = u_begin; ok && u < u_end;) {
+      const uint32_t seg_end = min(u_end, (u / KB + 1) * KB);
+      ok = mbar_wait_warp(&tempty[buf], aphase ^ 1u, abort, p.wait_ns);
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + buf * p.acc_stride;
+      uint32_t acc = 0;
+      for (; ok && u < seg_end; ++u) {
+        ok = mbar_wait_warp(&full[stage], phase, abort, p.wait_ns);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * p.acc_stride;
-        bool first = true;
-        for (; u < seg_end; ++u) {
-          if (!mbar_wait(&full[stage], phase, abort, p.wait_ns)) break;
-          tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * stage_bytes);
-          const uint32_t sb = sa + a_atom * BKA;
+        const uint64_t da = desc0 + static_cast<uint64_t>((stage * stage_bytes) >> 4);
+        const uint64_t db = da + static_cast<uint64_t>((a_atom * BKA) >> 4);
 #pragma unroll
-          for (int a = 0; a < BKA; ++a) {
+        for (int a = 0; a < BKA; ++a) {
 #pragma unroll
-            for (int k = 0; k < ATOM / UK; ++k) {
-              const uint64_t adesc = sw128_desc(sa + a * a_atom + k * 32);
-              tc_mma_bf16(d_tmem, adesc, sw128_desc(sb + a * b_atom + k * 32), idesc,
-                          (first && a == 0 && k == 0) ? 0u : 1u);
-              if (p.has_lo) tc_mma_bf16(d_tmem, adesc, sw128_desc(sb + b_bytes + a * b_atom + k * 32), idesc, 1u);
-            }
-          }
-          first = false;
-          tc_commit(&empty[stage]);
-          if (++stage == p.stages) {
-            stage = 0;
-            phase ^= 1u;
+          for (int k = 0; k < ATOM / UK; ++k) {  // 32 bytes per K step
+            tc_mma_bf16(d_tmem, da + static_cast<uint64_t>((a * a_atom + k * 32) >> 4),
+                        db + static_cast<uint64_t>((a * b_step + k * 32) >> 4), idesc, acc, elected);
+            acc = 1;
           }
         }
-        tc_commit(&tfull[buf]);
-        buf ^= 1;
-        if (buf == 0) aphase ^= 1u;
+        tc_commit(&empty[stage], elected);
+        if (++stage == p.stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
-      if (*abort) {
-        // every MMA issued so far must complete before TMEM is released
-        tc_commit(drain);
-        mbar_wait_plain(drain, 0, 200000000ull);
-      }
+      if (ok) tc_commit(&tfull[buf], elected);
+      buf ^= 1;
+      if (buf == 0) aphase ^= 1u;
     }
+    if (!ok) {
+      // every MMA issued so far must complete before TMEM is released
+      tc_commit(drain, elected);
+      mbar_wait_plain(drain, 0, 200000000ull);
+    }
+    __syncwarp();
   } else {
     // ---------------- epilogue (warps 2..5, TMEM lanes 32*(warp%4) ..) ----------------
     pdl_wait();  // Y, the split workspace and the counters are shared with earlier kernels
@@ -319,6 +326,16 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
     }
     const int q = warp & 3;
     const int row = q * 32 + lane;
+    // 16 token columns of this lane's feature: with a split, the hi and the lo products
+    auto load16 = [&](uint32_t taddr, float (&v)[16]) {
+      tmem_ld_16(taddr, v);
+      if (p.has_lo) {
+        float lo[16];
+        tmem_ld_16(taddr + p.BN, lo);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += lo[j];
+      }
+    };
     int buf = 0;
     uint32_t aphase = 0;
     for (uint32_t u = u_begin; u < u_end;) {
@@ -339,7 +356,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       if (nparts == 1 || p.epi == EPI_RESID) {
         for (int c0 = 0; c0 < p.BN; c0 += 16) {
           float v[16];
-          tmem_ld_16(tbase + c0, v);
+          load16(tbase + c0, v);
           if (p.vec_red)
             epi_red16(p, m0 + c0, ft * BM + q * 32, lane, v, s_red + q * 16 * 33);
           else
@@ -352,7 +369,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
         float* wsp = p.ws + static_cast<size_t>(my_slot) * BM * p.BN;
         for (int c0 = 0; c0 < p.BN; c0 += 16) {
           float v[16];
-          tmem_ld_16(tbase + c0, v);
+          load16(tbase + c0, v);
 #pragma unroll
           for (int j = 0; j < 16; ++j) __stcg(&wsp[(c0 + j) * BM + row], v[j]);
         }
@@ -454,6 +471,24 @@ int encode_2d_bf16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t 
   return r == CUDA_SUCCESS ? 0 : -2;
 }
 
+int encode_5d_bf16(CUtensorMap* map, const void* base, const uint64_t (&dims)[5], const uint64_t (&strides)[4],
+                   const uint32_t (&box)[5]) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return -1;
+  cuuint64_t gd[5], gs[4];
+  cuuint32_t bx[5], es[5];
+  for (int i = 0; i < 5; ++i) {
+    gd[i] = dims[i];
+    bx[i] = box[i];
+    es[i] = 1;
+    if (i < 4) gs[i] = strides[i];
+  }
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), gd, gs, bx, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? 0 : -2;
+}
+
 namespace {
 
 uint32_t pow2ceil(uint32_t v) {
@@ -533,10 +568,10 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   p.counters = counters;
   p.err = err;
   p.wait_ns = g_lin_wait_ns.load();
-  p.acc_stride = pow2ceil(static_cast<uint32_t>(p.BN));
+  p.acc_stride = pow2ceil(static_cast<uint32_t>((p.has_lo ? 2 : 1) * p.BN));
   p.tmem_cols = pow2ceil(2 * p.acc_stride);
   if (p.tmem_cols < 32) p.tmem_cols = 32;
-  if (p.tmem_cols > 512) return fail("accumulators exceed tensor memory");
+  if (p.tmem_cols > 512 || (p.has_lo && p.BN > 128)) return fail("accumulators exceed tensor memory");
   if (encode_2d_bf16(&p.tmA, W, K, N1, K, ATOM, BM) != 0) return fail("tensor map of W");
   if (W2 && encode_2d_bf16(&p.tmA2, W2, K, N2, K, ATOM, BM) != 0) return fail("tensor map of W2");
   if (encode_2d_bf16(&p.tmB, X, K, M, ldx, ATOM, p.BN) != 0) return fail("tensor map of X");
