@@ -12,16 +12,32 @@
 // values, probabilities); each product takes hi*hi + lo*hi + hi*lo, so the result
 // matches fp32 arithmetic to ~2^-16.  Q, K and V tiles sit in shared memory in the
 // K-major 128-byte-swizzled layout (V is read MN-major by the PV product); P is written
-// by the softmax warps in the same layout.  Two S accumulators in tensor memory let the
-// QK product of tile t+1 overlap the softmax of tile t.  The running max is only raised
-// (and O rescaled) when a row's maximum grows by more than a factor ~e^8 (keeping P, l
-// and O finite in fp32); the final normalisation uses the same max, so the result is
-// exact.  Scores and maxima are kept in base-2 units (scaled by log2 e).
+// by the softmax warps in the same layout.  The running max is only raised (and O
+// rescaled) when a row's maximum grows by more than a factor ~e^8 (keeping P, l and O
+// finite in fp32); the final normalisation uses the same max, so the result is exact.
+// Scores and maxima are kept in base-2 units (scaled by log2 e).
 //
-// Warps: 0..7 softmax + epilogue (warp w: tensor-memory lanes 32 (w % 4).., rows
-// 16 (w % 4) .. + 15, keys / output columns of half w / 4), 8 loads the KV tiles (one thread issues TMA copies of 16-row page boxes into
-// two-stage rings for K and for V, 128-byte swizzle applied by the copy engine), 9
-// issues the MMAs and owns the tensor-memory allocation.
+// A tile's chain (QK product, softmax, PV product and the barriers between them) is
+// longer than its K and V take to stream in, so the even and the odd tiles of a CTA are
+// two independent softmax streams: each has its own four warps, S accumulator, P buffer,
+// running max and sum, and O accumulator, and nothing passes between them until the
+// merge, which takes 2 S partials per row instead of S.
+//
+// What bounds it (GB300, split planes, 4 splits of 32 heads): at a 16384-row context the K
+// and V stream (91.5 us, 5.9 TB/s; 75 us with the loads left out), at a 1000-row one the
+// latency of the prologue and of the merge (15.5 us, of which about 9 do not depend on
+// the context).  Before: 128.4 and 18.1 us, bound by the MMA issue: one lane moved the
+// operands of 36 small MMAs a tile to uniform registers (54 cycles each).  Also
+// measured: both streams in one, eight warps sharing a tile and its row maxima (2 % slower
+// then); K in 2 KB boxes and an L2 prefetch three tiles ahead (108.9 us, without the
+// prefetch 95.8); QK products of 32 keys, to allow boxes of a page with its rows together
+// (8 us slower).
+//
+// Warps: 0..7 softmax + epilogue (warp w: stream w / 4, tensor-memory lanes 32 (w % 4)..,
+// rows 16 (w % 4) .. + 15; a warp whose rows are all past nq only keeps the barriers
+// going), 8 loads the KV tiles (TMA copies of 16-row page boxes into two-stage rings for
+// K and for V, 128-byte swizzle applied by the copy engine), 9 issues the MMAs and owns
+// the tensor-memory allocation.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -37,16 +53,19 @@ namespace {
 constexpr int HD = 128;
 constexpr int KT = 64;                      // keys per tile
 constexpr int NQ = 64;                      // query rows (UMMA M)
-constexpr int SOFT_WARPS = 8, LOAD_WARPS = 1;  // softmax: warps w and w + 4 share rows, split keys
+constexpr int SOFT_WARPS = 8, LOAD_WARPS = 1;  // softmax: warps w and w + 4 share rows, w / 4 = tile parity
+constexpr int STREAM_WARPS = SOFT_WARPS / 2;
 constexpr int THREADS = (SOFT_WARPS + LOAD_WARPS + 1) * 32;
 constexpr int MMA_WARP = SOFT_WARPS + LOAD_WARPS;
 constexpr int ATOM_ROWS64 = 64 * 128;       // bytes of one 64-row x 128-byte swizzle atom column
+constexpr int GROUP = 8 * 128;              // 8 rows x 64 dims: one swizzle atom
 constexpr int TILE64 = 2 * ATOM_ROWS64;     // 64 rows x 128 bf16 (two atoms): 16 KB
 constexpr int STAGES = 2;
-constexpr int L2_AHEAD = 3;                 // tiles requested into L2 beyond the newest ring load
 constexpr int PAGE_CACHE = 1024;
 constexpr float RESCALE_LOG2 = 11.5f;        // raise the running max when it grows by > 2^11.5 (~e^8)
-constexpr uint32_t TMEM_COLS = 256;          // S[2] (64 cols each) + O (128 cols)
+constexpr uint32_t TMEM_COLS = 512;          // S[2] (64 cols each), O[2] (128 cols each)
+constexpr uint32_t O_COL = 128;
+constexpr int MAX_PARTS = 16;                // partials of a row: 2 streams x 8 splits
 constexpr int PREC = HD + 4;                 // partial record (o[128], m, l, pad)
 
 // Byte offset of 16-byte chunk c (0..7) of row r inside a 128-byte-swizzled atom column.
@@ -98,11 +117,12 @@ __device__ __forceinline__ void tmem_wait_ld16(uint32_t (&r)[16]) {
                :
                : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld32(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :
-               : "memory");
+// Four 16-column pieces of a 128-column row: lanes 0..15 columns 0..63, 16..31 columns 64..127.
+__device__ __forceinline__ void tmem_ld_row(uint32_t taddr, uint32_t (&r)[4][16]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) tmem_ld16x2<64>(taddr + 16 * c, r[c]);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) tmem_wait_ld16(r[c]);
 }
 // 2^x on the special-function unit (inputs here are <= 0; results below 2^-126 flush to 0)
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -115,8 +135,8 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
-// Kernel arguments: the tensor map of the pool viewed as [pool_rows][hd] bf16 (box
-// 64 dims x 16 rows) and the attention parameters.
+// Kernel arguments: the tensor map of the pool viewed as [8-row group][plane][dim half][8
+// rows][64 dims] (box: the planes of K, or of V, of one page) and the attention parameters.
 struct TcArgs {
   CUtensorMap kv_map;
   AttnParams p;
@@ -149,7 +169,13 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   const AttnParams& p = args.p;
   constexpr int NP = SPLIT ? 4 : 2;
   constexpr int KP = NP / 2;                 // planes of K (and of V): hi (, lo)
-  constexpr int HALF_BYTES = KP * TILE64;   // one stage of K or of V
+  constexpr int HALF_BYTES = KP * TILE64;   // one stage of K or of V:
+  // [page][8-row group][plane][dim half][8 rows][128 B]: one box per page, and the groups of
+  // a plane and dim half lie at one stride (ROW_STRIDE) over the whole tile, as the
+  // descriptors need
+  constexpr int ROW_STRIDE = 2 * KP * GROUP;
+  constexpr int PAGE_BYTES = 2 * ROW_STRIDE;
+  constexpr int PLANE_STRIDE = 2 * GROUP;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* q_hi = smem;                     // 64 x 128 (two atoms)
@@ -157,23 +183,20 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   uint8_t* p_buf = q_lo + TILE64;           // [2 buffers][hi, lo] 64 x 64 (one atom each, 8 KB)
   uint8_t* kbuf = p_buf + 4 * (NQ * 128);   // [STAGES][KP planes] 64 keys x 128 dims
   uint8_t* vbuf = kbuf + STAGES * HALF_BYTES;
-  float* part = reinterpret_cast<float*>(kbuf);  // [64][PREC], reuses the KV stages after the loop
+  float* part = reinterpret_cast<float*>(smem);  // partial records, over the Q, P, K and V tiles after the loop
   uint64_t* bars = reinterpret_cast<uint64_t*>(vbuf + STAGES * HALF_BYTES);
   uint64_t* k_full = bars;           // [2] count 1 + transaction bytes (TMA)
   uint64_t* v_full = bars + 2;       // [2] count 1 + transaction bytes (TMA)
   uint64_t* k_empty = bars + 4;      // [2] tcgen05.commit after QK
   uint64_t* v_empty = bars + 6;      // [2] tcgen05.commit after PV
   uint64_t* s_full = bars + 8;       // [2] tcgen05.commit
-  uint64_t* s_free = bars + 10;      // [2] count 4 (softmax warps)
+  uint64_t* s_free = bars + 10;      // [2] count 4 (the stream's softmax warps)
   uint64_t* p_full = bars + 12;      // [2] count 4
   uint64_t* pv_done = bars + 14;     // [2] tcgen05.commit
   uint64_t* o_done = bars + 16;      // tcgen05.commit
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_pages = s_abort + 2;        // [PAGE_CACHE]
-  float* s_stat = reinterpret_cast<float*>(s_pages + PAGE_CACHE);  // [64][2] final (m, l)
-  float* s_xm = s_stat + 2 * NQ;     // [2 tiles][2 halves][64] tile maxima of the key halves
-  float* s_lh = s_xm + 4 * NQ;       // [2 halves][64] partial row sums
   volatile int* abort = s_abort;
 
   const int s = blockIdx.x, h = blockIdx.y;
@@ -188,8 +211,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       mbar_init(&k_empty[i], 1);
       mbar_init(&v_empty[i], 1);
       mbar_init(&s_full[i], 1);
-      mbar_init(&s_free[i], SOFT_WARPS);
-      mbar_init(&p_full[i], SOFT_WARPS);
+      mbar_init(&s_free[i], STREAM_WARPS);
+      mbar_init(&p_full[i], STREAM_WARPS);
       mbar_init(&pv_done[i], 1);
     }
     mbar_init(o_done, 1);
@@ -231,39 +254,24 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // ---- KV staging (the loader warp, all lanes together): K or V of tile t into stage st
-  // as 4 pages x KP planes x 2 swizzle atoms of 16 rows, one box per lane; pages at or
-  // past kend are requested out of bounds (zero fill). One thread issues a box only every
-  // ~70 ns, so the 8 KP boxes of a half go out from as many lanes at once. ----
-  const long long rows_per_layer = p.pool_layer_stride / HD;
+  // ---- KV staging (the loader warp, all lanes together): K or V of tile t into stage st,
+  // a page's planes and dim halves as one box per lane (4 or 8 KB); pages at or past kend
+  // are requested out of bounds (zero fill). ----
+  const int groups_per_layer = static_cast<int>(p.pool_layer_stride / (16 * HD));  // 16-row planes
   auto issue_half = [&](int t, int st, int kend, bool is_v) {
     uint64_t* bar = is_v ? &v_full[st] : &k_full[st];
     if (lane == 0) mbar_arrive_expect_tx(bar, static_cast<uint32_t>(HALF_BYTES));
     __syncwarp();
-    if (lane < 8 * KP) {
-      const int u = lane / (2 * KP), plane = (lane >> 1) % KP, a = lane & 1;
-      const int kg = t * KT + u * 16;
-      long long y = p.pool_rows;  // out of bounds
+    if (lane < 4) {
+      const int kg = t * KT + lane * 16;
+      int y = static_cast<int>(p.pool_rows / 16);  // out of bounds
       if (kg < kend) {
-        const int page = cached ? s_pages[(t - t0) * 4 + u] : p.page_table[b * p.max_pages + t * 4 + u];
-        y = static_cast<long long>(p.layer) * rows_per_layer +
-            ((static_cast<long long>(page) * p.H + h) * NP + (is_v ? KP : 0) + plane) * 16;
+        const int page = cached ? s_pages[(t - t0) * 4 + lane] : p.page_table[b * p.max_pages + t * 4 + lane];
+        y = p.layer * groups_per_layer + (page * p.H + h) * NP + (is_v ? KP : 0);
       }
-      uint8_t* base = (is_v ? vbuf : kbuf) + st * HALF_BYTES;
-      tma_load_2d(base + plane * TILE64 + a * ATOM_ROWS64 + u * 16 * 128, &args.kv_map, a * 64,
-                  static_cast<int>(y), bar);
+      tma_load_5d((is_v ? vbuf : kbuf) + st * HALF_BYTES + lane * PAGE_BYTES, &args.kv_map, 0, 0, 0, y, 0, bar);
     }
   };
-
-  // L2 prefetch of tile t's page-planes (NP x 4 KB, contiguous per page), one page per lane
-  auto prefetch_tile = [&](int t, int kend) {
-    if (lane < 4 && t * KT + lane * 16 < kend) {
-      const int page = cached ? s_pages[(t - t0) * 4 + lane] : p.page_table[b * p.max_pages + t * 4 + lane];
-      const bf16* src = pool + (static_cast<size_t>(page) * p.H + h) * NP * 16 * HD;
-      prefetch_l2_bulk(src, NP * 16 * HD * 2);
-    }
-  };
-  int pf = 0;  // tiles [0, pf) of the range were requested into L2
 
   int pre = 0;  // leading tiles (K and V) requested before the dependency wait
   if (p.prewait_kv) {
@@ -277,8 +285,6 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         issue_half(t0 + pre, (hl + pre) & 1, nctx, true);
         ++pre;
       }
-      for (; pf < t1 - t0 && pf < STAGES + L2_AHEAD && (lmode || (t0 + pf + 1) * KT <= nctx); ++pf)
-        if (pf >= pre) prefetch_tile(t0 + pf, nctx);
     }
     pdl_wait();
   }
@@ -384,9 +390,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           }
         }
       }
-      // stage 0: row i, dims j .. j + 3 (atom 0) and 64 + j .. (atom 1): half of chunk j / 8
-      const uint32_t o0 = swz(i, j >> 3) + ((j & 7) << 1);
-      const uint32_t o1 = ATOM_ROWS64 + o0;
+      // stage 0: row i, dims j .. j + 3 (half 0) and 64 + j .. (half 1): half of chunk j / 8
+      const uint32_t o0 = (i >> 3) * ROW_STRIDE + swz(i & 7, j >> 3) + ((j & 7) << 1);
+      const uint32_t o1 = GROUP + o0;
       uint8_t* kt = kbuf;
       uint8_t* vt = vbuf;
       *reinterpret_cast<uint2*>(kt + o0) = kh0;
@@ -394,10 +400,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       *reinterpret_cast<uint2*>(vt + o0) = vh0;
       *reinterpret_cast<uint2*>(vt + o1) = vh1;
       if (SPLIT) {
-        *reinterpret_cast<uint2*>(kt + TILE64 + o0) = kl0;
-        *reinterpret_cast<uint2*>(kt + TILE64 + o1) = kl1;
-        *reinterpret_cast<uint2*>(vt + TILE64 + o0) = vl0;
-        *reinterpret_cast<uint2*>(vt + TILE64 + o1) = vl1;
+        *reinterpret_cast<uint2*>(kt + PLANE_STRIDE + o0) = kl0;
+        *reinterpret_cast<uint2*>(kt + PLANE_STRIDE + o1) = kl1;
+        *reinterpret_cast<uint2*>(vt + PLANE_STRIDE + o0) = vl0;
+        *reinterpret_cast<uint2*>(vt + PLANE_STRIDE + o1) = vl1;
       }
     }
   }
@@ -450,6 +456,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     mbar_arrive(&v_full[0]);
   }
 
+  // softmax state of this lane's row (softmax warps)
+  const int strm = (warp >> 2) & 1, quad = warp & 3, sub = lane >> 4;
+  const int r = quad * 16 + (lane & 15);
+  const uint32_t tlane = static_cast<uint32_t>(quad * 32) << 16;
+  float m_used = -INFINITY, l = 0.f;
+
   if (warp == SOFT_WARPS) {
     // ---------------- KV loader (the whole warp; lane 0 polls and decides) ----------------
     if (!p.prewait_kv && lane == 0) prefetch_tensormap(&args.kv_map);
@@ -466,7 +478,6 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
                                                 (nk < STAGES || mbar_test(&k_empty[nk & 1], ((nk - STAGES) >> 1) & 1))) ? 1 : 0, 0);
       if (kgo) {
         issue_half(t0 + nk - hl, nk & 1, kend, false);
-        for (pf = max(pf, nk - hl + 1); pf < t1 - t0 && pf <= nk - hl + L2_AHEAD; ++pf) prefetch_tile(t0 + pf, kend);
         ++nk;
         moved = true;
       }
@@ -494,69 +505,71 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     }
     __syncwarp();
   } else if (warp == MMA_WARP) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0 && nt > 0) {
+    // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+    const int ntu = __shfl_sync(0xffffffffu, nt, 0);
+    if (ntu > 0) {
+      const uint32_t elected = elect_one();
       const uint32_t id_qk = idesc_f16(NQ, KT, false);
       const uint32_t id_pv = idesc_f16(NQ, HD, true);
-      const uint32_t qh = smem_u32(q_hi), ql = smem_u32(q_lo);
-      // descriptors are precomputed once; advancing a K-major operand by b bytes adds
-      // b >> 4 to its start-address field (all operands lie below 256 KB of shared memory)
-      const uint64_t dq_h = desc_sw128(qh, 16, 1024), dq_l = desc_sw128(ql, 16, 1024);
-      uint64_t dk_h[STAGES], dv_h[STAGES], dp_h[2];
-#pragma unroll
-      for (int st = 0; st < STAGES; ++st) {
-        dk_h[st] = desc_sw128(smem_u32(kbuf + st * HALF_BYTES), 16, 1024);
-        // V as MN-major B: 64-dim atoms 8 KB apart (leading), 8-key groups 1 KB apart
-        dv_h[st] = desc_sw128(smem_u32(vbuf + st * HALF_BYTES), ATOM_ROWS64, 1024);
-      }
-#pragma unroll
-      for (int pb = 0; pb < 2; ++pb) dp_h[pb] = desc_sw128(smem_u32(p_buf + (2 * pb) * (NQ * 128)), 16, 1024);
-      constexpr uint64_t LO_OFS = TILE64 >> 4;        // hi plane -> lo plane (16 KB)
+      // descriptors are made once; advancing an operand by b bytes adds b >> 4 to its
+      // start-address field (all operands lie below 256 KB of shared memory)
+      const uint64_t dq_h = desc_sw128(smem_u32(q_hi), 16, 1024), dq_l = desc_sw128(smem_u32(q_lo), 16, 1024);
+      const uint64_t dp = desc_sw128(smem_u32(p_buf), 16, 1024);
+      const uint64_t dk = desc_sw128(smem_u32(kbuf), 16, ROW_STRIDE);
+      // V as MN-major B: 64-dim atoms GROUP apart (leading), 8-key groups ROW_STRIDE apart
+      const uint64_t dv = desc_sw128(smem_u32(vbuf), GROUP, ROW_STRIDE);
+      constexpr uint64_t LO_OFS = PLANE_STRIDE >> 4;  // hi plane -> lo plane
       constexpr uint64_t P_LO_OFS = (NQ * 128) >> 4;  // P hi -> P lo (8 KB)
-      auto pv = [&](int i) {  // O += P_i V_i
-        const int st = i & 1;
-        const uint32_t o_t = tmem + 128;
+      auto pv = [&](int i) {  // O[i & 1] += P_i V_i
+        const uint32_t st = i & 1;
+        const uint32_t o_t = tmem + O_COL + st * 128;
+        const uint64_t a0 = dp + static_cast<uint64_t>(st * (2 * NQ * 128 >> 4));
+        const uint64_t b0 = dv + static_cast<uint64_t>(st * (HALF_BYTES >> 4));
+        uint32_t acc = i > 1 ? 1u : 0u;
 #pragma unroll
         for (int ks = 0; ks < KT / 16; ++ks) {
-          const uint64_t a_h = dp_h[st] + static_cast<uint64_t>(ks * 2);  // 32 bytes per K step
-          const uint64_t b_h = dv_h[st] + static_cast<uint64_t>(ks * 128);  // 16 keys = 2 KB
-          tc_mma_bf16(o_t, a_h, b_h, id_pv, (i > 0 || ks > 0) ? 1u : 0u);
-          tc_mma_bf16(o_t, a_h + P_LO_OFS, b_h, id_pv, 1u);
-          if (SPLIT) tc_mma_bf16(o_t, a_h, b_h + LO_OFS, id_pv, 1u);
+          const uint64_t a_h = a0 + static_cast<uint64_t>(ks * 2);                   // 32 bytes per K step
+          const uint64_t b_h = b0 + static_cast<uint64_t>(ks * (PAGE_BYTES >> 4));  // 16 keys: a page
+          tc_mma_bf16(o_t, a_h, b_h, id_pv, acc, elected);
+          acc = 1;
+          tc_mma_bf16(o_t, a_h + P_LO_OFS, b_h, id_pv, 1u, elected);
+          if (SPLIT) tc_mma_bf16(o_t, a_h, b_h + LO_OFS, id_pv, 1u, elected);
         }
-        tc_commit(&pv_done[i & 1]);
-        tc_commit(&v_empty[st]);
+        tc_commit(&pv_done[st], elected);
+        tc_commit(&v_empty[st], elected);
       };
       auto qk = [&](int i) {  // S_i = Q K_i^T into S buffer i & 1
-        const int st = i & 1;
+        const uint32_t st = i & 1;
         const uint32_t s_t = tmem + st * 64;
+        const uint64_t b0 = dk + static_cast<uint64_t>(st * (HALF_BYTES >> 4));
 #pragma unroll
         for (int ks = 0; ks < HD / 16; ++ks) {
-          const uint64_t off = static_cast<uint64_t>(((ks >> 2) * ATOM_ROWS64 + (ks & 3) * 32) >> 4);
-          const uint64_t b_h = dk_h[st] + off;
-          tc_mma_bf16(s_t, dq_h + off, b_h, id_qk, ks > 0 ? 1u : 0u);
-          tc_mma_bf16(s_t, dq_l + off, b_h, id_qk, 1u);
-          if (SPLIT) tc_mma_bf16(s_t, dq_h + off, b_h + LO_OFS, id_qk, 1u);
+          const uint64_t a_ofs = static_cast<uint64_t>(((ks >> 2) * ATOM_ROWS64 + (ks & 3) * 32) >> 4);
+          const uint64_t b_h = b0 + static_cast<uint64_t>(((ks >> 2) * GROUP + (ks & 3) * 32) >> 4);
+          tc_mma_bf16(s_t, dq_h + a_ofs, b_h, id_qk, ks > 0 ? 1u : 0u, elected);
+          tc_mma_bf16(s_t, dq_l + a_ofs, b_h, id_qk, 1u, elected);
+          if (SPLIT) tc_mma_bf16(s_t, dq_h + a_ofs, b_h + LO_OFS, id_qk, 1u, elected);
         }
-        tc_commit(&s_full[st]);
-        tc_commit(&k_empty[st]);
+        tc_commit(&s_full[st], elected);
+        tc_commit(&k_empty[st], elected);
       };
-      // issue whichever product is ready: PV(np) when P and V of tile np are in, QK(nq)
-      // when K is in, its S buffer is free and it runs at most one tile ahead of the PV
-      // products (so no barrier is ever two phases ahead of its waiter)
+      // issue whichever product is ready: PV(npv) when P and V of tile npv are in, QK(nqk)
+      // when K is in and the softmax of tile nqk - 2 has read its S buffer (so no barrier is
+      // ever two phases ahead of its waiter)
       int nqk = 0, npv = 0;
       uint64_t last_progress = global_timer_ns();
-      while (npv < nt && !*abort) {
+      while (npv < ntu) {
         bool moved = false;
-        if (npv < nqk && mbar_test(&p_full[npv & 1], (npv >> 1) & 1) &&
-            mbar_test(&v_full[npv & 1], (npv >> 1) & 1)) {
+        if (npv < nqk && __all_sync(0xffffffffu, mbar_test(&p_full[npv & 1], (npv >> 1) & 1) &&
+                                                     mbar_test(&v_full[npv & 1], (npv >> 1) & 1))) {
           tc_fence_after();
           pv(npv);
           ++npv;
           moved = true;
         }
-        if (nqk < nt && nqk <= npv + 1 && mbar_test(&k_full[nqk & 1], (nqk >> 1) & 1) &&
-            (nqk < 2 || mbar_test(&s_free[nqk & 1], ((nqk - 2) >> 1) & 1))) {
+        if (nqk < ntu &&
+            __all_sync(0xffffffffu, mbar_test(&k_full[nqk & 1], (nqk >> 1) & 1) &&
+                                        (nqk < 2 || mbar_test(&s_free[nqk & 1], ((nqk - 2) >> 1) & 1)))) {
           tc_fence_after();
           qk(nqk);
           ++nqk;
@@ -564,162 +577,139 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         }
         if (moved) {
           last_progress = global_timer_ns();
-        } else if (global_timer_ns() - last_progress > 2000000000ull) {
-          *abort = 1;
+        } else {
+          const bool late = global_timer_ns() - last_progress > 2000000000ull;
+          if (late) *abort = 1;
+          if (__any_sync(0xffffffffu, late || *abort)) break;
         }
       }
-      tc_commit(o_done);  // all MMAs issued by this thread, including any after an abort
+      tc_commit(o_done, elected);  // all MMAs issued by this lane, including any after an abort
       // tensor memory and the KV stages are released only after every MMA completed
       mbar_wait_plain(o_done, 0, 200000000ull);
     }
   } else {
     // ---------------- softmax (warps 0..7) ----------------
-    // Warps w and w + 4 own the 16 rows of TMEM sub-partition w % 4 and the key halves
-    // 0 / 1 of every tile; within a warp, lanes l and l + 16 share row l % 16 and take
-    // 16 keys each (the 16x32bx2 access shape), so every lane works. The two lanes of a
-    // row combine by a shuffle, the warp pair through shared memory (named barrier
-    // 1 + w % 4). After a timeout the loop keeps running (without work) so both warps of
-    // a pair still meet at every barrier.
-    const int half = warp >> 2, quad = warp & 3, sub = lane >> 4;
-    const int r = quad * 16 + (lane & 15);
+    // Warp w owns the 16 rows of TMEM sub-partition w % 4 in every second tile (w / 4: even
+    // or odd); lanes l and l + 16 share row l % 16 and take 32 keys each (the 16x32bx2
+    // access shape) and combine by a shuffle.
+    const bool any = quad * 16 < nq;
     const bool live = r < nq;
-    const int kofs = 32 * half + 16 * sub;  // this lane's first key within a tile
     const unsigned long long anc = live ? p.anc[p.q_local0 + r] : 0ull;
     const float scale2 = p.scale * 1.4426950408889634f;  // softmax in base 2: exp(x) = 2^(x log2 e)
-    const uint32_t tlane = static_cast<uint32_t>(quad * 32) << 16;
-    float m_used = -INFINITY, l = 0.f;
-    bool dead = false;
-    for (int i = 0; i < nt; ++i) {
-      const int sb = i & 1;
+    uint8_t* ph = p_buf + (2 * strm) * (NQ * 128);
+    uint8_t* pl = ph + NQ * 128;
+    for (int i = strm; i < nt; i += 2) {
       const bool loc = hl && i == 0;
       const int t = t0 + i - hl;
-      bool ok = !dead && mbar_wait(&s_full[sb], (i >> 1) & 1, abort);
-      dead = !__all_sync(0xffffffffu, ok);
+      if (!__all_sync(0xffffffffu, mbar_wait(&s_full[strm], (i >> 1) & 1, abort))) break;
       tc_fence_after();
-      float sv[16];
-      if (!dead) {
-        uint32_t rr[16];
-        tmem_ld16x2<16>(tmem + tlane + sb * 64 + half * 32, rr);
-        tmem_wait_ld16(rr);
+      float sv[32];
+      if (any) {
+        uint32_t ra[16], rb[16];
+        tmem_ld16x2<32>(tmem + tlane + strm * 64, ra);
+        tmem_ld16x2<32>(tmem + tlane + strm * 64 + 16, rb);
+        tmem_wait_ld16(ra);
+        tmem_wait_ld16(rb);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) sv[j] = __uint_as_float(rr[j]);
+        for (int j = 0; j < 16; ++j) {
+          sv[j] = __uint_as_float(ra[j]);
+          sv[16 + j] = __uint_as_float(rb[j]);
+        }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0 && !dead) mbar_arrive(&s_free[sb]);
-      // visibility of this lane's 16 keys (bit j: key kofs + j of the tile): the local
-      // tile's keys are local rows (ancestor mask), a pool tile's keys are slots 64 t ..
-      uint32_t vbits = 0u;
-      if (live) {
-        unsigned long long vis;
-        if (loc) {
-          vis = anc & (nloc >= 64 ? ~0ull : ((1ull << nloc) - 1ull));
-        } else {
-          const int base = t * KT;
-          const int nc = nctx - base, nv = total - base, off = base - nctx;
-          const unsigned long long cm = nc >= 64 ? ~0ull : (nc <= 0 ? 0ull : ((1ull << nc) - 1ull));
-          const unsigned long long lm =
-              lmode ? 0ull : (off >= 0 ? (off < 64 ? (anc >> off) : 0ull) : (-off < 64 ? (anc << -off) : 0ull));
-          const unsigned long long vm = nv >= 64 ? ~0ull : (nv <= 0 ? 0ull : ((1ull << nv) - 1ull));
-          vis = (cm | lm) & vm;
-        }
-        vbits = static_cast<uint32_t>(vis >> kofs) & 0xFFFFu;
-      }
-      float ta = -INFINITY, tb = -INFINITY;  // two chains of maxima
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        sv[j] = (!dead && ((vbits >> j) & 1u)) ? sv[j] * scale2 : -INFINITY;
-        if (j & 1)
-          tb = fmaxf(tb, sv[j]);
-        else
-          ta = fmaxf(ta, sv[j]);
-      }
-      // the row's maximum over its 64 keys: the other lane of the row, then the pair warp
-      float tmax = fmaxf(ta, tb);
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-      if (sub == 0) s_xm[(sb * 2 + half) * NQ + r] = tmax;
-      named_bar(1 + quad, 64);
-      tmax = fmaxf(tmax, s_xm[(sb * 2 + (half ^ 1)) * NQ + r]);
-      // this tile's P buffer was read by the PV product of tile i - 2
+      if (lane == 0) mbar_arrive(&s_free[strm]);
+      // this stream's P buffer and O accumulator were used by the PV product of tile i - 2
       if (i >= 2) {
-        ok = !dead && mbar_wait(&pv_done[i & 1], ((i - 2) >> 1) & 1, abort);
-        dead = !__all_sync(0xffffffffu, ok);
+        if (!__all_sync(0xffffffffu, mbar_wait(&pv_done[strm], ((i - 2) >> 1) & 1, abort))) break;
         tc_fence_after();
       }
-      // m moves only when the tile's maximum exceeds it by more than 2^RESCALE_LOG2; O then
-      // holds products of earlier tiles exactly when m was already finite. Both decisions
-      // depend only on the row's shared maxima, so all four lanes of a row agree.
-      const bool raise = tmax > m_used + RESCALE_LOG2 || (m_used == -INFINITY && tmax > -INFINITY);
-      const bool rescale = raise && m_used != -INFINITY;
-      float corr = 1.f;
-      if (raise) {
-        corr = rescale ? exp2f(m_used - tmax) : 0.f;
-        m_used = tmax;
-      }
-      if (!dead && i > 0 && __any_sync(0xffffffffu, rescale)) {
-        // O holds the products up to tile i - 1: wait for the last one before rescaling
-        ok = mbar_wait(&pv_done[(i - 1) & 1], ((i - 1) >> 1) & 1, abort);
-        dead = !__all_sync(0xffffffffu, ok);
-        tc_fence_after();
-        if (!dead) {
-          // this warp's 64 columns of its O rows (lanes 0..15: the first 32, lanes
-          // 16..31: the last 32); factor 1 for rows that kept m
-          const float f = rescale ? corr : 1.f;
-          const uint32_t oa = tmem + tlane + 128 + half * 64;
-          uint32_t rr[32];
-          tmem_ld16x2<32>(oa, rr);
-          tmem_ld16x2<32>(oa + 16, rr + 16);
-          tmem_wait_ld32(rr);
+      if (any) {
+        // visibility of this lane's 32 keys (bit j: key 32 sub + j of the tile): the local
+        // tile's keys are local rows (ancestor mask), a pool tile's keys are slots 64 t ..
+        uint32_t vbits = 0u;
+        if (live) {
+          unsigned long long vis;
+          if (loc) {
+            vis = anc & (nloc >= 64 ? ~0ull : ((1ull << nloc) - 1ull));
+          } else {
+            const int base = t * KT;
+            const int nc = nctx - base, nv = total - base, off = base - nctx;
+            const unsigned long long cm = nc >= 64 ? ~0ull : (nc <= 0 ? 0ull : ((1ull << nc) - 1ull));
+            const unsigned long long lm =
+                lmode ? 0ull : (off >= 0 ? (off < 64 ? (anc >> off) : 0ull) : (-off < 64 ? (anc << -off) : 0ull));
+            const unsigned long long vm = nv >= 64 ? ~0ull : (nv <= 0 ? 0ull : ((1ull << nv) - 1ull));
+            vis = (cm | lm) & vm;
+          }
+          vbits = static_cast<uint32_t>(vis >> (32 * sub));
+        }
+        if (__any_sync(0xffffffffu, vbits != 0xffffffffu)) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) rr[j] = __float_as_uint(__uint_as_float(rr[j]) * f);
-          tmem_st16x2<32>(oa, rr);
-          tmem_st16x2<32>(oa + 16, rr + 16);
+          for (int j = 0; j < 32; ++j)
+            if (!((vbits >> j) & 1u)) sv[j] = -INFINITY;
+        }
+        float t4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};  // four chains of maxima
+#pragma unroll
+        for (int j = 0; j < 32; ++j) t4[j & 3] = fmaxf(t4[j & 3], sv[j]);
+        float tmax = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16)) * scale2;  // over the row's 64 keys
+        // m moves only when the tile's maximum exceeds it by more than 2^RESCALE_LOG2; O then
+        // holds products of earlier tiles exactly when m was already finite.  Both lanes of a
+        // row decide alike.
+        const bool raise = tmax > m_used + RESCALE_LOG2 || (m_used == -INFINITY && tmax > -INFINITY);
+        const bool rescale = raise && m_used != -INFINITY;
+        float corr = 1.f;
+        if (raise) {
+          corr = rescale ? exp2f(m_used - tmax) : 0.f;
+          m_used = tmax;
+        }
+        if (__any_sync(0xffffffffu, rescale)) {  // factor 1 for rows that kept m
+          const float f = rescale ? corr : 1.f;
+          const uint32_t oa = tmem + tlane + O_COL + strm * 128;
+          uint32_t rr[4][16];
+          tmem_ld_row(oa, rr);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) rr[c][j] = __float_as_uint(__uint_as_float(rr[c][j]) * f);
+            tmem_st16x2<64>(oa + 16 * c, rr[c]);
+          }
           tmem_wait_st();
         }
-      }
-      l *= corr;
-      // P = 2^(S - m), two-term split into the swizzled P tile (this lane's 2 chunks)
-      uint8_t* ph = p_buf + (2 * sb) * (NQ * 128);
-      uint8_t* pl = ph + NQ * 128;
-      float ra = 0.f, rb = 0.f;
+        l *= corr;
+        // P = 2^(S - m), two-term split into the swizzled P tile (this lane's 4 chunks of 8);
+        // a row with no visible key yet has m = -inf and scores -inf: P = 0
+        const float mm = m_used == -INFINITY ? 0.f : m_used;
+        float l4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float pv8[8];
+        for (int c = 0; c < 4; ++c) {
+          float e[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float x = sv[8 * c + e];
-          pv8[e] = (x == -INFINITY) ? 0.f : ex2_approx(x - m_used);
-          if (e & 1)
-            rb += pv8[e];
-          else
-            ra += pv8[e];
+          for (int j = 0; j < 8; ++j) {
+            e[j] = ex2_approx(fmaf(sv[8 * c + j], scale2, -mm));
+            l4[j & 3] += e[j];
+          }
+          uint4 hh, ll;
+          split_pair(e[0], e[1], hh.x, ll.x);
+          split_pair(e[2], e[3], hh.y, ll.y);
+          split_pair(e[4], e[5], hh.z, ll.z);
+          split_pair(e[6], e[7], hh.w, ll.w);
+          *reinterpret_cast<uint4*>(ph + swz(r, 4 * sub + c)) = hh;
+          *reinterpret_cast<uint4*>(pl + swz(r, 4 * sub + c)) = ll;
         }
-        uint4 hh, ll;
-        split_pair(pv8[0], pv8[1], hh.x, ll.x);
-        split_pair(pv8[2], pv8[3], hh.y, ll.y);
-        split_pair(pv8[4], pv8[5], hh.z, ll.z);
-        split_pair(pv8[6], pv8[7], hh.w, ll.w);
-        if (!dead) {
-          *reinterpret_cast<uint4*>(ph + swz(r, kofs / 8 + c)) = hh;
-          *reinterpret_cast<uint4*>(pl + swz(r, kofs / 8 + c)) = ll;
-        }
+        l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+        fence_async_smem();
       }
-      l += ra + rb;
-      fence_async_smem();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0 && !dead) mbar_arrive(&p_full[sb]);
+      if (lane == 0) mbar_arrive(&p_full[strm]);
     }
-    l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's sum over this warp's key half
-    if (sub == 0) {
-      if (half == 0) s_stat[2 * r] = m_used;
-      s_lh[half * NQ + r] = l;
-    }
+    l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's sum over the stream's tiles
   }
 
-  // ---- epilogue: every CTA pushes its partial rows (O, m, l) to the cluster CTA that
+  // ---- epilogue: every stream pushes its partial rows (O, m, l) to the cluster CTA that
   // finishes them (rows [r * ceil(nq / S), ...) belong to rank r); the receive buffer
-  // reuses the KV rings, so the pushes start once every CTA of the cluster is past its
+  // reuses the tiles, so the pushes start once every CTA of the cluster is past its
   // main loop (split cluster barrier) ----
   if (warp < SOFT_WARPS) {
     if (nt > 0) {
@@ -728,46 +718,36 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     }
     __syncwarp();
   }
-  __syncthreads();  // this CTA's rings are idle: every load landed and every MMA completed
+  __syncthreads();  // this CTA's tiles are idle: every load landed and every MMA completed
   __syncwarp();
   if (S > 1) cluster_arrive();
   const int rpc = (nq + S - 1) / S;
-  float* recv = part;                     // [S][rpc][PREC], S * rpc <= NQ + 7 rows (37.5 KB)
-  float* s_w = part + (NQ + 8) * PREC;    // [rpc][8] merge weights, past the receive slots
+  float* recv = part;                         // [2 S][rpc][PREC], S * rpc <= NQ + 7 rows (75 KB)
+  float* s_w = part + 2 * (NQ + 8) * PREC;    // [rpc][MAX_PARTS] merge weights, past the receive slots
   {
-    const bool soft = warp < SOFT_WARPS;
-    const int half = (warp >> 2) & 1, sub = lane >> 4;
-    const int r = (warp & 3) * 16 + (lane & 15);
-    const bool have = soft && nt > 0 && !*abort;
-    const bool mine = soft && r < nq;
-    const int cb = half * 64 + sub * 32;  // this lane's first O column
-    uint32_t rr[32];
-    if (have) {  // this lane's 32 columns of the O row, while the peers finish
-      const uint32_t oa = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 128 + half * 64;
-      tmem_ld16x2<32>(oa, rr);
-      tmem_ld16x2<32>(oa + 16, rr + 16);
-      tmem_wait_ld32(rr);
-    }
+    const bool mine = warp < SOFT_WARPS && r < nq;
+    const bool have = warp < SOFT_WARPS && quad * 16 < nq && nt > strm && !*abort;
+    uint32_t rr[4][16];
+    if (have) tmem_ld_row(tmem + tlane + O_COL + strm * 128, rr);  // this lane's 64 columns, while the peers finish
     __syncwarp();
     if (S > 1) cluster_wait();
-    if (soft) {
-      const int owner = mine ? r / rpc : 0;
-      const uint32_t slot = smem_u32(recv + (s * rpc + (mine ? r - owner * rpc : 0)) * PREC);
+    if (mine) {
+      const int owner = r / rpc;
+      const uint32_t slot = smem_u32(recv + ((2 * s + strm) * rpc + r - owner * rpc) * PREC);
       const uint32_t dst = S > 1 ? dsmem_addr(slot, owner) : slot;
-      const float lr = mine ? s_lh[r] + s_lh[NQ + r] : 0.f;
-      const bool keep = have && lr > 0.f;
-      if (mine) {
+      const bool keep = have && l > 0.f;
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          const float4 v = keep ? make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]),
-                                              __uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3]))
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+          const float4 v = keep ? make_float4(__uint_as_float(rr[c][j]), __uint_as_float(rr[c][j + 1]),
+                                              __uint_as_float(rr[c][j + 2]), __uint_as_float(rr[c][j + 3]))
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-          st_dsmem4(dst + static_cast<uint32_t>((cb + j) * 4), v);
+          st_dsmem4(dst + static_cast<uint32_t>((64 * sub + 16 * c + j) * 4), v);
         }
-        if (half == 0 && sub == 0) {
-          st_dsmem(dst + HD * 4, nt > 0 ? s_stat[2 * r] : -INFINITY);
-          st_dsmem(dst + (HD + 1) * 4, nt > 0 ? lr : 0.f);
-        }
+      if (sub == 0) {
+        st_dsmem(dst + HD * 4, have ? m_used : -INFINITY);
+        st_dsmem(dst + (HD + 1) * 4, have ? l : 0.f);
       }
     }
   }
@@ -782,36 +762,36 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   __syncwarp();
   if (S > 1) cluster_sync();  // every push into this CTA is complete and visible
 
-  // ---- merge the S partials of this CTA's rows (local shared memory) ----
+  // ---- merge the 2 S partials of this CTA's rows (local shared memory) ----
   bf16* out = static_cast<bf16*>(p.out);
   bf16* out_lo = static_cast<bf16*>(p.out_lo);
-  const int q0 = s * rpc, nrows = max(0, min(nq, q0 + rpc) - q0);
+  const int q0 = s * rpc, nrows = max(0, min(nq, q0 + rpc) - q0), parts = 2 * S;
   for (int rl = threadIdx.x; rl < nrows; rl += blockDim.x) {
-    float mv[8], M = -INFINITY;
+    float mv[MAX_PARTS], M = -INFINITY;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      mv[k] = k < S ? recv[(k * rpc + rl) * PREC + HD] : -INFINITY;
+    for (int k = 0; k < MAX_PARTS; ++k) {
+      mv[k] = k < parts ? recv[(k * rpc + rl) * PREC + HD] : -INFINITY;
       M = fmaxf(M, mv[k]);
     }
     float L = 0.f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      mv[k] = (k < S && M != -INFINITY && mv[k] != -INFINITY) ? exp2f(mv[k] - M) : 0.f;
-      if (k < S) L += mv[k] * recv[(k * rpc + rl) * PREC + HD + 1];
+    for (int k = 0; k < MAX_PARTS; ++k) {
+      mv[k] = (k < parts && M != -INFINITY && mv[k] != -INFINITY) ? exp2f(mv[k] - M) : 0.f;
+      if (k < parts) L += mv[k] * recv[(k * rpc + rl) * PREC + HD + 1];
     }
     const float inv = L > 0.f ? 1.f / L : 0.f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < S) s_w[rl * 8 + k] = mv[k] * inv;
+    for (int k = 0; k < MAX_PARTS; ++k)
+      if (k < parts) s_w[rl * MAX_PARTS + k] = mv[k] * inv;
   }
   __syncthreads();
   for (int it = threadIdx.x; it < nrows * (HD / 4); it += blockDim.x) {
     const int rl = it / (HD / 4), c = (it % (HD / 4)) * 4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      if (k < S) {
-        const float w = s_w[rl * 8 + k];
+    for (int k = 0; k < MAX_PARTS; ++k) {
+      if (k < parts) {
+        const float w = s_w[rl * MAX_PARTS + k];
         const float4 v = *reinterpret_cast<const float4*>(recv + (k * rpc + rl) * PREC + c);
         acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
       }
@@ -824,7 +804,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
 template <bool SPLIT>
 size_t tc_smem() {
   const size_t np = SPLIT ? 4 : 2;
-  return 1024 + 2 * TILE64 + 4 * NQ * 128 + STAGES * np * TILE64 + 18 * 8 + 16 + PAGE_CACHE * 4 + 8 * NQ * 4;
+  return 1024 + 2 * TILE64 + 4 * NQ * 128 + STAGES * np * TILE64 + 18 * 8 + 16 + PAGE_CACHE * 4;
 }
 
 // The dynamic shared memory limit is an attribute of the device that is current when it
@@ -856,8 +836,10 @@ cudaError_t launch_tc(const AttnParams& p, cudaStream_t s) {
   TcArgs args;
   memset(&args, 0, sizeof(args));
   args.p = p;
-  if (encode_2d_bf16(&args.kv_map, p.pool, HD, static_cast<uint64_t>(p.pool_rows), HD, 64, 16) != 0)
-    return cudaErrorInvalidValue;
+  const uint64_t dims[5] = {64, 8, 2, static_cast<uint64_t>(p.pool_rows / 16), 2};
+  const uint64_t strides[4] = {HD * 2, 128, 16 * HD * 2, 8 * HD * 2};
+  const uint32_t box[5] = {64, 8, 2, SPLIT ? 2u : 1u, 2};
+  if (encode_5d_bf16(&args.kv_map, p.pool, dims, strides, box) != 0) return cudaErrorInvalidValue;
   cudaLaunchAttribute at[2];
   int na = 0;
   at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;

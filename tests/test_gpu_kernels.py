@@ -168,6 +168,9 @@ ATT_CASES = [
     (3, 2, 128, [16, 1, 129], 5, 1, 4, 3),     # draft-style: one query, local rows 0..4
     (1, 2, 128, [1000], 64, 64, 0, 8),
     (2, 3, 128, [700, 3], 64, 64, 0, 4),     # a split whose key range is empty for b=1
+    (1, 2, 128, [0], 3, 3, 0, 1),            # one tile: the odd-tile stream has none
+    (2, 2, 128, [100, 63], 17, 17, 0, 1),    # two tiles (and a row in a second warp), 80 keys
+    (1, 2, 128, [1500], 33, 33, 0, 2),       # many tiles per stream, row counts no multiple of 16
 ]
 
 
