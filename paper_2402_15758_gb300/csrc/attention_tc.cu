@@ -20,18 +20,16 @@
 // A tile's chain (QK product, softmax, PV product and the barriers between them) is
 // longer than its K and V take to stream in, so the even and the odd tiles of a CTA are
 // two independent softmax streams: each has its own four warps, S accumulator, P buffer,
-// running max and sum, and O accumulator, and nothing passes between them until the
-// merge, which takes 2 S partials per row instead of S.
+// running max and sum, and O accumulator, and nothing passes between them until the end.
 //
 // What bounds it (GB300, split planes, 4 splits of 32 heads): at a 16384-row context the K
 // and V stream (91.5 us, 5.9 TB/s; 75 us with the loads left out), at a 1000-row one the
 // latency of the prologue and of the merge (15.5 us, of which about 9 do not depend on
 // the context).  Before: 128.4 and 18.1 us, bound by the MMA issue: one lane moved the
-// operands of 36 small MMAs a tile to uniform registers (54 cycles each).  Also
-// measured: both streams in one, eight warps sharing a tile and its row maxima (2 % slower
-// then); K in 2 KB boxes and an L2 prefetch three tiles ahead (108.9 us, without the
-// prefetch 95.8); QK products of 32 keys, to allow boxes of a page with its rows together
-// (8 us slower).
+// operands of 36 small MMAs a tile to uniform registers (54 cycles each).  Also measured,
+// at 16384 rows: an L2 prefetch three tiles ahead of the rings 108.9 us against 95.8
+// without; QK products of 32 keys, which let a box keep a page's 16 rows together, 95.8
+// against 91.5.
 //
 // Warps: 0..7 softmax + epilogue (warp w: stream w / 4, tensor-memory lanes 32 (w % 4)..,
 // rows 16 (w % 4) .. + 15; a warp whose rows are all past nq only keeps the barriers
@@ -65,8 +63,12 @@ constexpr int PAGE_CACHE = 1024;
 constexpr float RESCALE_LOG2 = 11.5f;        // raise the running max when it grows by > 2^11.5 (~e^8)
 constexpr uint32_t TMEM_COLS = 512;          // S[2] (64 cols each), O[2] (128 cols each)
 constexpr uint32_t O_COL = 128;
-constexpr int MAX_PARTS = 16;                // partials of a row: 2 streams x 8 splits
+constexpr int MAX_PARTS = 16;                // partials of a row: one or two per split
+constexpr int MANY_NQ = 32;                  // more query rows than this take the MANY variant
 constexpr int PREC = HD + 4;                 // partial record (o[128], m, l, pad)
+constexpr int PART_FLOATS = (2 * MANY_NQ + 16) * PREC;  // the partial records of a CTA (<= NQ + 14 rows)
+constexpr int TILE_BYTES = 192 * 1024;       // Q, P, K and V tiles (with plain planes: and 64 KB of staging)
+static_assert((3 * PART_FLOATS + NQ * MAX_PARTS) * 4 <= TILE_BYTES, "partials and merge weights fit over the tiles");
 
 // Byte offset of 16-byte chunk c (0..7) of row r inside a 128-byte-swizzled atom column.
 __device__ __forceinline__ uint32_t swz(int r, int c) {
@@ -164,7 +166,12 @@ __device__ __forceinline__ void split4(float4 v, uint2& hi, uint2& lo) {
 // sub-partition q (warp w reaches sub-partition w % 4).
 
 
-template <bool SPLIT>
+// MANY: more than MANY_NQ query rows.  Their rows and the local tile's are staged through
+// shared memory, and a CTA merges its two streams before it sends them; with fewer rows
+// each of these steps adds more latency than it saves (one query 9.9 us without, 10.6
+// with them; 64 queries 15.7 and 14.5), and both paths in one kernel cost each other
+// (64 queries 15.3).
+template <bool SPLIT, bool MANY>
 __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_constant__ TcArgs args) {
   const AttnParams& p = args.p;
   constexpr int NP = SPLIT ? 4 : 2;
@@ -183,8 +190,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   uint8_t* p_buf = q_lo + TILE64;           // [2 buffers][hi, lo] 64 x 64 (one atom each, 8 KB)
   uint8_t* kbuf = p_buf + 4 * (NQ * 128);   // [STAGES][KP planes] 64 keys x 128 dims
   uint8_t* vbuf = kbuf + STAGES * HALF_BYTES;
-  float* part = reinterpret_cast<float*>(smem);  // partial records, over the Q, P, K and V tiles after the loop
-  uint64_t* bars = reinterpret_cast<uint64_t*>(vbuf + STAGES * HALF_BYTES);
+  // fp32 rows of the projections on their way into the tiles: q, and the local tile's k and v
+  float* q_st = reinterpret_cast<float*>(p_buf);
+  float* k_st = reinterpret_cast<float*>(SPLIT ? kbuf + HALF_BYTES : vbuf + STAGES * HALF_BYTES);
+  float* v_st = reinterpret_cast<float*>(SPLIT ? vbuf + HALF_BYTES : vbuf + STAGES * HALF_BYTES + 2 * TILE64);
+  float* part = reinterpret_cast<float*>(smem);  // partial records, over the tiles after the loop
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + TILE_BYTES);
   uint64_t* k_full = bars;           // [2] count 1 + transaction bytes (TMA)
   uint64_t* v_full = bars + 2;       // [2] count 1 + transaction bytes (TMA)
   uint64_t* k_empty = bars + 4;      // [2] tcgen05.commit after QK
@@ -197,6 +208,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_pages = s_abort + 2;        // [PAGE_CACHE]
+  int* s_lpages = s_pages + PAGE_CACHE;  // [8] pages of the local rows
   volatile int* abort = s_abort;
 
   const int s = blockIdx.x, h = blockIdx.y;
@@ -249,6 +261,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     const int np = min((t1 - t0) * 4, p.max_pages - t0 * 4);
     for (int i = threadIdx.x; i < np; i += blockDim.x) s_pages[i] = p.page_table[b * p.max_pages + t0 * 4 + i];
   }
+  if (hl && threadIdx.x >= THREADS - 5) {
+    const int i = threadIdx.x - (THREADS - 5);
+    s_lpages[i] = (nctx >> 4) + i < p.max_pages ? p.page_table[b * p.max_pages + (nctx >> 4) + i] : 0;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -280,14 +296,38 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       __syncwarp();
       // pool tiles whose rows are all committed (local mode: rows at or past nctx are
       // masked; the pool holds finite values there, the pools being cleared at set-up)
-      while (hl + pre < nt && hl + pre < STAGES && (lmode || (t0 + pre + 1) * KT <= nctx)) {
+      // (with many rows and split planes the local tile's owner stages k and v in stage 1 first)
+      while (hl + pre < nt && hl + pre < STAGES && !(SPLIT && MANY && hl) && (lmode || (t0 + pre + 1) * KT <= nctx)) {
         issue_half(t0 + pre, (hl + pre) & 1, nctx, false);
         issue_half(t0 + pre, (hl + pre) & 1, nctx, true);
         ++pre;
       }
     }
-    pdl_wait();
+    __syncwarp();
   }
+  // The angles of this thread's two query items (item it: row it / 8, dims 8j .. and 64 + 8j
+  // .., j = it % 8): neither they nor the positions depend on the kernel before, and their
+  // two dependent loads, after the wait, outlast the copy of the rows (1.2 us of 2.8)
+  constexpr int ITEMS = MANY ? 2 : 1;
+  float2 cs[ITEMS][8];
+  if (p.qkv) {
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const int it = threadIdx.x + k * THREADS, r = it >> 3;
+      if (r < p.nq) {
+        const int pos = min(max(nctx + p.pos_base + (p.pos_off ? p.pos_off[r] : r), 0), p.max_pos - 1);
+        const float4* tab = reinterpret_cast<const float4*>(p.rope + static_cast<size_t>(pos) * (HD / 2) + 8 * (it & 7));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 t = tab[e];
+          cs[k][2 * e] = make_float2(t.x, t.y);
+          cs[k][2 * e + 1] = make_float2(t.z, t.w);
+        }
+      }
+    }
+  }
+
+  if (p.prewait_kv) pdl_wait();
   pdl_trigger();
 
   const int nloc = p.q_blocks > 1 ? qb.nloc : min(p.n_local_dev ? p.n_local_dev[b] : p.n_local, p.n_local);
@@ -295,26 +335,51 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   const int total = nctx + nloc;
   const int dm = p.H * HD;
 
+  const float* q_src = p.qkv ? p.qkv + static_cast<size_t>(qb.row0) * p.ldqkv + h * HD
+                             : p.q + static_cast<size_t>(qb.row0) * p.ldq + h * HD;
+  const float* k_src = hl ? p.qkv + static_cast<size_t>(qb.row0) * p.ldqkv + dm + h * HD : nullptr;
+  const float* v_src = hl ? k_src + dm : nullptr;
+  int q_ld = p.qkv ? p.ldqkv : p.ldq, kv_ld = p.ldqkv;
+  if constexpr (MANY) {
+    // fp32 rows into shared memory, every copy of a thread in flight at once (loaded item by
+    // item, q took 2.8 us and the local tile another 4.3)
+    auto stage_rows = [&](float* dst, const float* src, int ld) {
+      for (int it = threadIdx.x; it < nq * (HD / 4); it += THREADS)
+        cp_async16(dst + it * 4, src + static_cast<size_t>(it / (HD / 4)) * ld + it % (HD / 4) * 4);
+    };
+    stage_rows(q_st, q_src, q_ld);
+    if (hl) {
+      stage_rows(k_st, k_src, kv_ld);
+      stage_rows(v_st, v_src, kv_ld);
+    }
+    q_src = q_st;
+    k_src = k_st;
+    v_src = v_st;
+    q_ld = kv_ld = HD;
+    cp_async_wait_all();
+    __syncthreads();
+  }
+
   // ---- queries: rotate (fused mode), split, write the swizzled Q tiles ----
-  for (int it = threadIdx.x; it < NQ * 8; it += blockDim.x) {
-    const int r = it >> 3, j = it & 7;  // row, 8-dim chunk j of the first half (dims 8j.., 64 + 8j..)
+  static_assert(NQ * 8 <= 2 * THREADS && MANY_NQ * 8 <= THREADS, "two items per thread, or one");
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int it = threadIdx.x + k * THREADS;
+    if (it >= NQ * 8) break;
+    const int r = it >> 3, j = it & 7;
     float lo_half[8], hi_half[8];
-    if (r < nq) {
-      const float* src = p.qkv ? p.qkv + static_cast<size_t>(qb.row0 + r) * p.ldqkv + h * HD + 8 * j
-                               : p.q + static_cast<size_t>(qb.row0 + r) * p.ldq + h * HD + 8 * j;
+    if (k < ITEMS && r < nq) {  // (up to MANY_NQ rows: a thread's second item is past them)
+      const float* src = q_src + static_cast<size_t>(r) * q_ld + 8 * j;
       const float4 a0 = *reinterpret_cast<const float4*>(src), a1 = *reinterpret_cast<const float4*>(src + 4);
       const float4 b0 = *reinterpret_cast<const float4*>(src + HD / 2),
                    b1 = *reinterpret_cast<const float4*>(src + HD / 2 + 4);
       const float x1[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
       const float x2[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
       if (p.qkv) {
-        const int pos = min(max(nctx + p.pos_base + (p.pos_off ? p.pos_off[r] : r), 0), p.max_pos - 1);
-        const float2* tab = p.rope + static_cast<size_t>(pos) * (HD / 2) + 8 * j;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const float2 cs = tab[e];
-          lo_half[e] = x1[e] * cs.x - x2[e] * cs.y;
-          hi_half[e] = x2[e] * cs.x + x1[e] * cs.y;
+          lo_half[e] = x1[e] * cs[k < ITEMS ? k : 0][e].x - x2[e] * cs[k < ITEMS ? k : 0][e].y;
+          hi_half[e] = x2[e] * cs[k < ITEMS ? k : 0][e].x + x1[e] * cs[k < ITEMS ? k : 0][e].y;
         }
       } else {
 #pragma unroll
@@ -347,7 +412,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   // rows to the pool (for later steps) and into its stage-0 K and V tiles; rows past the
   // fresh ones are zero there ----
   if (hl) {
-    for (int it = threadIdx.x; it < KT * 16; it += blockDim.x) {
+    for (int it = threadIdx.x; it < KT * 16; it += THREADS) {
       const int i = it >> 4, j = (it & 15) * 4;  // local row, pair index j .. j + 3 of the first half
       uint2 kh0 = make_uint2(0u, 0u), kl0 = kh0, kh1 = kh0, kl1 = kh0, vh0 = kh0, vl0 = kh0, vh1 = kh0, vl1 = kh0;
       if (i < nq) {
@@ -356,11 +421,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         if (pos < 0 || pos >= p.max_pos || (slot >> 4) >= p.max_pages) {
           if (p.err) atomicOr(p.err, ERR_CAPACITY);
         } else {
-          const float* src = p.qkv + static_cast<size_t>(b * p.q_rows + i) * p.ldqkv + h * HD + j;
-          const float4 k1 = *reinterpret_cast<const float4*>(src + dm);
-          const float4 k2 = *reinterpret_cast<const float4*>(src + dm + HD / 2);
-          const float4 v1 = *reinterpret_cast<const float4*>(src + 2 * dm);
-          const float4 v2 = *reinterpret_cast<const float4*>(src + 2 * dm + HD / 2);
+          const size_t o = static_cast<size_t>(i) * kv_ld + j;
+          const float4 k1 = *reinterpret_cast<const float4*>(k_src + o);
+          const float4 k2 = *reinterpret_cast<const float4*>(k_src + o + HD / 2);
+          const float4 v1 = *reinterpret_cast<const float4*>(v_src + o);
+          const float4 v2 = *reinterpret_cast<const float4*>(v_src + o + HD / 2);
           const float2* tab = p.rope + static_cast<size_t>(pos) * (HD / 2) + j;
           const float4 cs01 = *reinterpret_cast<const float4*>(tab);
           const float4 cs23 = *reinterpret_cast<const float4*>(tab + 2);
@@ -370,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           split4(rot_hi(k1, k2, c, sn), kh1, kl1);
           split4(v1, vh0, vl0);
           split4(v2, vh1, vl1);
-          const int page = p.page_table[b * p.max_pages + (slot >> 4)];
+          const int page = s_lpages[(slot >> 4) - (nctx >> 4)];
           bf16* base = pool + (static_cast<size_t>(page) * p.H + h) * NP * 16 * HD + (slot & 15) * HD + j;
           constexpr size_t plane = 16 * HD;
           if (SPLIT) {
@@ -707,10 +772,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's sum over the stream's tiles
   }
 
-  // ---- epilogue: every stream pushes its partial rows (O, m, l) to the cluster CTA that
-  // finishes them (rows [r * ceil(nq / S), ...) belong to rank r); the receive buffer
-  // reuses the tiles, so the pushes start once every CTA of the cluster is past its
-  // main loop (split cluster barrier) ----
+  // ---- epilogue: a CTA's partial rows (O, m, l) go to the cluster CTA that finishes them
+  // (rows [r * ceil(nq / S), ...) belong to rank r) once every CTA of the cluster is past
+  // its main loop; everything lies over the tiles.  Few rows: each stream pushes its own from
+  // the registers.  Many: that is bound by the traffic (64 rows: 3.3 us), so the streams are
+  // merged first, while the cluster gathers, and whole records are pushed (1.1 us). ----
   if (warp < SOFT_WARPS) {
     if (nt > 0) {
       mbar_wait(o_done, 0, abort);
@@ -722,74 +788,128 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   __syncwarp();
   if (S > 1) cluster_arrive();
   const int rpc = (nq + S - 1) / S;
-  float* recv = part;                         // [2 S][rpc][PREC], S * rpc <= NQ + 7 rows (75 KB)
-  float* s_w = part + 2 * (NQ + 8) * PREC;    // [rpc][MAX_PARTS] merge weights, past the receive slots
-  {
-    const bool mine = warp < SOFT_WARPS && r < nq;
-    const bool have = warp < SOFT_WARPS && quad * 16 < nq && nt > strm && !*abort;
+  constexpr int ps = MANY ? 1 : 2;              // partials per CTA
+  const int blk = ps * rpc * PREC;            // what a CTA sends to an owner: [ps][rpc][PREC]
+  float* recv = part + PART_FLOATS;           // [S] blocks
+  float* other = recv + PART_FLOATS;          // [64][PREC] the odd tiles' rows
+  float* s_w = other + PART_FLOATS;           // [rpc][MAX_PARTS] merge weights
+  if (warp < SOFT_WARPS) {
+    const bool mine = r < nq;
+    const bool have = quad * 16 < nq && nt > strm && !*abort;
+    const int owner = mine ? r / rpc : 0, orow = r - owner * rpc;
     uint32_t rr[4][16];
-    if (have) tmem_ld_row(tmem + tlane + O_COL + strm * 128, rr);  // this lane's 64 columns, while the peers finish
+    if (have) tmem_ld_row(tmem + tlane + O_COL + strm * 128, rr);  // this lane's 64 columns
+    auto piece = [&](int c, int j) {
+      return make_float4(__uint_as_float(rr[c][j]), __uint_as_float(rr[c][j + 1]), __uint_as_float(rr[c][j + 2]),
+                         __uint_as_float(rr[c][j + 3]));
+    };
     __syncwarp();
-    if (S > 1) cluster_wait();
-    if (mine) {
-      const int owner = r / rpc;
-      const uint32_t slot = smem_u32(recv + ((2 * s + strm) * rpc + r - owner * rpc) * PREC);
-      const uint32_t dst = S > 1 ? dsmem_addr(slot, owner) : slot;
-      const bool keep = have && l > 0.f;
+    if constexpr (!MANY) {
+      if (S > 1) cluster_wait();  // every CTA's tiles are idle
+      if (mine) {
+        const uint32_t slot = smem_u32(recv + s * blk + (strm * rpc + orow) * PREC);
+        const uint32_t dst = S > 1 ? dsmem_addr(slot, owner) : slot;
+        const bool keep = have && l > 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int j = 0; j < 16; j += 4) {
-          const float4 v = keep ? make_float4(__uint_as_float(rr[c][j]), __uint_as_float(rr[c][j + 1]),
-                                              __uint_as_float(rr[c][j + 2]), __uint_as_float(rr[c][j + 3]))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-          st_dsmem4(dst + static_cast<uint32_t>((64 * sub + 16 * c + j) * 4), v);
+          for (int j = 0; j < 16; j += 4)
+            st_dsmem4(dst + static_cast<uint32_t>((64 * sub + 16 * c + j) * 4),
+                      keep ? piece(c, j) : make_float4(0.f, 0.f, 0.f, 0.f));
+        if (sub == 0)
+          st_dsmem4(dst + HD * 4, make_float4(have ? m_used : -INFINITY, have ? l : 0.f, 0.f, 0.f));
+      }
+    } else {
+      float* o1 = other + r * PREC;
+      if (strm == 1 && have && mine) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(o1 + 64 * sub + 16 * c + j) = piece(c, j);
+        if (sub == 0) {
+          o1[HD] = m_used;
+          o1[HD + 1] = l;
         }
-      if (sub == 0) {
-        st_dsmem(dst + HD * 4, have ? m_used : -INFINITY);
-        st_dsmem(dst + (HD + 1) * 4, have ? l : 0.f);
+      }
+      named_bar(1 + quad, 64);  // the two warps of these rows
+      if (strm == 0 && mine) {
+        const bool have1 = nt > 1 && !*abort;
+        const float m0 = have ? m_used : -INFINITY, l0 = have ? l : 0.f;
+        const float m1 = have1 ? o1[HD] : -INFINITY, l1 = have1 ? o1[HD + 1] : 0.f;
+        const float m = fmaxf(m0, m1);
+        const float w0 = l0 > 0.f ? exp2f(m0 - m) : 0.f, w1 = l1 > 0.f ? exp2f(m1 - m) : 0.f;
+        float* dst = (owner == s ? recv + s * blk : part + owner * blk) + orow * PREC;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int j = 0; j < 16; j += 4) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (l0 > 0.f) {
+              const float4 t = piece(c, j);
+              v = make_float4(w0 * t.x, w0 * t.y, w0 * t.z, w0 * t.w);
+            }
+            if (l1 > 0.f) {
+              const float4 t = *reinterpret_cast<const float4*>(o1 + 64 * sub + 16 * c + j);
+              v.x += w1 * t.x; v.y += w1 * t.y; v.z += w1 * t.z; v.w += w1 * t.w;
+            }
+            *reinterpret_cast<float4*>(dst + 64 * sub + 16 * c + j) = v;
+          }
+        if (sub == 0) {
+          dst[HD] = m;
+          dst[HD + 1] = w0 * l0 + w1 * l1;
+        }
       }
     }
+  } else if (!MANY && S > 1) {
+    cluster_wait();
   }
   tc_fence_before();
   __syncthreads();
   __syncwarp();
+  if (MANY && S > 1) {
+    cluster_wait();
+    for (int it = threadIdx.x; it < nq * (PREC / 4); it += THREADS) {  // 512 contiguous bytes per warp
+      const int row = it / (PREC / 4), c = it % (PREC / 4) * 4, owner = row / rpc;
+      const int o = owner * blk + (row - owner * rpc) * PREC + c;
+      if (owner != s)
+        st_dsmem4(dsmem_addr(smem_u32(recv + o + (s - owner) * blk), owner), *reinterpret_cast<const float4*>(part + o));
+    }
+    __syncwarp();
+  }
+  if (S > 1) cluster_arrive();
   if (warp == MMA_WARP) {
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
   }
   if (threadIdx.x == 0 && *abort && p.err) atomicOr(p.err, ERR_TIMEOUT);
   __syncwarp();
-  if (S > 1) cluster_sync();  // every push into this CTA is complete and visible
+  if (S > 1) cluster_wait();  // the peers' partials are in
 
-  // ---- merge the 2 S partials of this CTA's rows (local shared memory) ----
+  // ---- merge the partials of this CTA's rows (local shared memory) ----
   bf16* out = static_cast<bf16*>(p.out);
   bf16* out_lo = static_cast<bf16*>(p.out_lo);
-  const int q0 = s * rpc, nrows = max(0, min(nq, q0 + rpc) - q0), parts = 2 * S;
-  for (int rl = threadIdx.x; rl < nrows; rl += blockDim.x) {
-    float mv[MAX_PARTS], M = -INFINITY;
+  const int q0 = s * rpc, nrows = max(0, min(nq, q0 + rpc) - q0), parts = ps * S;
+  constexpr int LPR = 8 * ps;  // lanes per row, one partial each
+  for (int r0 = warp * (32 / LPR); r0 < nrows; r0 += 32 / LPR * (THREADS / 32)) {
+    const int rl = r0 + lane / LPR, k = lane % LPR;
+    const bool on = rl < nrows && k < parts;
+    const float* rec = recv + (k * rpc + rl) * PREC;
+    const float m = on ? rec[HD] : -INFINITY, ls = on ? rec[HD + 1] : 0.f;
+    float M = m;
 #pragma unroll
-    for (int k = 0; k < MAX_PARTS; ++k) {
-      mv[k] = k < parts ? recv[(k * rpc + rl) * PREC + HD] : -INFINITY;
-      M = fmaxf(M, mv[k]);
-    }
-    float L = 0.f;
+    for (int o = LPR / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float e = m == -INFINITY ? 0.f : exp2f(m - M);
+    float L = e * ls;
 #pragma unroll
-    for (int k = 0; k < MAX_PARTS; ++k) {
-      mv[k] = (k < parts && M != -INFINITY && mv[k] != -INFINITY) ? exp2f(mv[k] - M) : 0.f;
-      if (k < parts) L += mv[k] * recv[(k * rpc + rl) * PREC + HD + 1];
-    }
-    const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-    for (int k = 0; k < MAX_PARTS; ++k)
-      if (k < parts) s_w[rl * MAX_PARTS + k] = mv[k] * inv;
+    for (int o = LPR / 2; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    if (on) s_w[rl * MAX_PARTS + k] = L > 0.f ? e / L : 0.f;
   }
   __syncthreads();
   for (int it = threadIdx.x; it < nrows * (HD / 4); it += blockDim.x) {
     const int rl = it / (HD / 4), c = (it % (HD / 4)) * 4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < MAX_PARTS; ++k) {
+    for (int k = 0; k < LPR; ++k) {
       if (k < parts) {
         const float w = s_w[rl * MAX_PARTS + k];
         const float4 v = *reinterpret_cast<const float4*>(recv + (k * rpc + rl) * PREC + c);
@@ -801,37 +921,34 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   }
 }
 
-template <bool SPLIT>
-size_t tc_smem() {
-  const size_t np = SPLIT ? 4 : 2;
-  return 1024 + 2 * TILE64 + 4 * NQ * 128 + STAGES * np * TILE64 + 18 * 8 + 16 + PAGE_CACHE * 4;
-}
+constexpr size_t TC_SMEM = 1024 + TILE_BYTES + 18 * 8 + 16 + (PAGE_CACHE + 8) * 4;
 
 // The dynamic shared memory limit is an attribute of the device that is current when it
 // is set: raised once per device (and kernel variant), the return code checked.
 constexpr int ATT_MAX_DEVICES = 64;
 std::mutex g_att_attr_mu;
-bool g_att_attr[2][ATT_MAX_DEVICES];
+bool g_att_attr[4][ATT_MAX_DEVICES];
 
-template <bool SPLIT>
+template <bool SPLIT, bool MANY>
 cudaError_t tc_attr() {
+  constexpr int variant = (SPLIT ? 2 : 0) + (MANY ? 1 : 0);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= ATT_MAX_DEVICES) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_att_attr_mu);
-  if (!g_att_attr[SPLIT ? 1 : 0][dev]) {
-    e = cudaFuncSetAttribute(attn_tc_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tc_smem<SPLIT>()));
+  if (!g_att_attr[variant][dev]) {
+    e = cudaFuncSetAttribute(attn_tc_kernel<SPLIT, MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(TC_SMEM));
     if (e != cudaSuccess) return e;
-    g_att_attr[SPLIT ? 1 : 0][dev] = true;
+    g_att_attr[variant][dev] = true;
   }
   return cudaSuccess;
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool MANY>
 cudaError_t launch_tc(const AttnParams& p, cudaStream_t s) {
-  cudaError_t ae = tc_attr<SPLIT>();
+  cudaError_t ae = tc_attr<SPLIT, MANY>();
   if (ae != cudaSuccess) return ae;
   TcArgs args;
   memset(&args, 0, sizeof(args));
@@ -855,17 +972,17 @@ cudaError_t launch_tc(const AttnParams& p, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.splits, p.H, p.B * std::max(1, p.q_blocks));
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = tc_smem<SPLIT>();
+  cfg.dynamicSmemBytes = TC_SMEM;
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = na;
-  cudaLaunchKernelEx(&cfg, attn_tc_kernel<SPLIT>, args);
+  cudaLaunchKernelEx(&cfg, attn_tc_kernel<SPLIT, MANY>, args);
   return cudaGetLastError();
 }
 
 template <bool SPLIT>
 int tc_splits(int BH, int want) {
-  if (tc_attr<SPLIT>() != cudaSuccess) return 1;
+  if (tc_attr<SPLIT, true>() != cudaSuccess) return 1;  // both row variants have the same footprint
   int S = std::max(1, std::min(8, want));
   for (; S > 1; --S) {
     cudaLaunchAttribute at[1];
@@ -876,11 +993,11 @@ int tc_splits(int BH, int want) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, BH, 1);
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = tc_smem<SPLIT>();
+    cfg.dynamicSmemBytes = TC_SMEM;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<SPLIT>, &cfg) == cudaSuccess && n >= BH) break;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<SPLIT, true>, &cfg) == cudaSuccess && n >= BH) break;
     cudaGetLastError();
   }
   return S;
@@ -897,7 +1014,8 @@ cudaError_t attention_tc(const AttnParams& p, cudaStream_t s) {
   if (p.planes != 2 && p.planes != 4) return cudaErrorInvalidValue;
   if (p.qkv && (!p.rope || !p.err || p.max_pos < 1 || (p.ldqkv & 3))) return cudaErrorInvalidValue;
   if (!p.qkv && (p.ldq & 3)) return cudaErrorInvalidValue;
-  return p.planes == 4 ? launch_tc<true>(p, s) : launch_tc<false>(p, s);
+  if (p.nq_max > MANY_NQ) return p.planes == 4 ? launch_tc<true, true>(p, s) : launch_tc<false, true>(p, s);
+  return p.planes == 4 ? launch_tc<true, false>(p, s) : launch_tc<false, false>(p, s);
 }
 
 int attention_tc_splits(int planes, int BH, int want) {
