@@ -7,16 +7,12 @@
 // KV layout: pool[layer][block][head][plane][16 rows][hd], page_table[b][slot / 16];
 // planes K, V (fp32 models, plain bf16) or K_hi, K_lo, V_hi, V_lo (bf16 two-term split).
 //
-// Grid (splits, heads, batch).  Each CTA loads every KV tile of its key range once
-// into shared memory for all the sequence's queries; online softmax in fp32.  This
-// file holds the SIMT kernel (fp32 models, and bf16 models with head_dim 64), whose
+// This file holds the SIMT kernel (fp32 models, and bf16 models with head_dim 64), whose
 // splits merge in the last CTA of each (b, h) through a global workspace, and the
-// dispatch; bf16 models with head_dim 128 take the tensor-core kernel of
-// attention_tc.cu, which can also fuse RoPE and the KV write of the step's fresh rows.
+// dispatch; bf16 models with head_dim 128 take the tensor-core kernel of attention_tc.cu,
+// which can also fuse RoPE and the KV write of the step's fresh rows.
 #include <algorithm>
 #include <cmath>
-
-#include <mutex>
 
 #include "attention.cuh"
 #include "common.cuh"
@@ -26,22 +22,11 @@
 namespace chimera {
 namespace {
 
-constexpr int KT = 32;      // keys per tile
 constexpr int WARPS = 8;
-constexpr int QPW = 8;      // queries per warp (nq <= 64)
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-
+constexpr int THREADS = WARPS * 32;
+constexpr int KEYS = 64;         // keys of a CTA in flight: a row of each of four pages per half-warp
+constexpr int MAX_NQ = 64;       // query rows per block
+constexpr int SPLIT_KEYS = 256;  // a split is not worth fewer keys (four passes)
 constexpr int MAX_SPLITS = 16;
 
 // Merge the per-split partials (unnormalised output, running max, running sum) of the
@@ -122,166 +107,260 @@ __device__ void combine_splits(const AttnParams& p, const float* wsb, int nq, in
   }
 }
 
-template <typename TKV, typename T, int HD>
-__global__ void __launch_bounds__(WARPS * 32) attn_kernel(const AttnParams p) {
+// Four consecutive elements of a KV row as fp32 (split planes: hi + lo); one element at a
+// time when the pool is not aligned for vectors.
+__device__ __forceinline__ float4 load_row4(const float* p, bool vec) {
+  return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ float4 load_row4(const bf16* p, bool vec) {
+  if (!vec) return make_float4(to_f(p[0]), to_f(p[1]), to_f(p[2]), to_f(p[3]));
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+template <typename TKV>
+__device__ __forceinline__ float4 load_kv4(const TKV* p, int lo_ofs, bool vec) {
+  float4 v = load_row4(p, vec);
+  if (lo_ofs) {
+    const float4 w = load_row4(p + lo_ofs, vec);
+    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+  }
+  return v;
+}
+
+// Sum v[0..NV) over each half-warp (NV <= 16): lane l returns the total of value
+// (l % 16) / (16 / NV); every step halves the values a lane still holds.
+template <int NV>
+__device__ __forceinline__ float half_sum_many(float (&v)[NV], int lane) {
+  int o = 8;
+#pragma unroll
+  for (int n = NV / 2; n >= 1; n /= 2, o /= 2) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float send = up ? v[i] : v[i + n];
+      const float keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  float t = v[0];
+  for (; o >= 1; o /= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// Latency bounds this kernel (the fp32 model's contexts are a few hundred rows), so it
+// keeps dependent memory trips few: a half-warp takes one row of each of four pages, 16
+// lanes per row, with the K and V of all four in flight at once, and scores them against
+// QG queries from shared memory; the 16 partial sums of a query group are reduced
+// together, and a lane keeps the running max and sum of one query.  No tile is staged and
+// the warps meet once, at the end.  More queries than QG are further CTAs.  Measured (GB300,
+// fp32, 4 heads of 64, an event pair around every launch): one query at 70 rows 19 -> 9 us,
+// 16 tree rows 17 -> 13; a 64-token prompt and eight steps 2.70 -> 2.26 ms.  The kernel
+// before staged 32-key tiles for all queries, kept seven of eight warps idle for one
+// query, and always split 16 ways.
+template <typename TKV, typename T, int HD, int QG>
+__global__ void __launch_bounds__(THREADS) attn_kernel(const AttnParams p, int groups) {
   pdl_trigger();  // the next kernel may start its prologue
   pdl_wait();     // inputs of this kernel are complete
-  // SIMT path: fp32 models and bf16 models with head_dim 64
-  constexpr int DPL = HD / 32;
-  extern __shared__ float sm[];
-  float* Ks = sm;                   // [KT][HD + 1]
-  float* Vs = Ks + KT * (HD + 1);   // [KT][HD]
-  float* Qs = Vs + KT * HD;         // [nq][HD]
+  constexpr int DV = HD / 64;        // float4 of a row per lane
+  constexpr int LPQ = 16 / QG;       // lanes that hold the same query's state
+  __shared__ __align__(16) float qs[QG * HD];
+  __shared__ __align__(16) float s_acc[WARPS * 1024];  // [WARPS][QG][HD], later combine_splits' weights
+  __shared__ float s_m[WARPS * QG], s_l[WARPS * QG];
   __shared__ int s_last;
 
-  const int s = blockIdx.x, h = blockIdx.y;
-  const QueryBlock qb(p, blockIdx.z);
-  const int b = qb.b, nctx = qb.nctx, nloc = qb.nloc, nq = qb.nq;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = nctx + nloc;
-  const int ntiles = nq > 0 ? (total + KT - 1) / KT : 0;
-  const int tps = (ntiles + p.splits - 1) / p.splits;
-  const int t0 = s * tps;
-  const int t1 = min(ntiles, t0 + tps);
-  const float* q = p.q;
+  const int s = blockIdx.x, h = blockIdx.y, g = blockIdx.z % groups;
+  const QueryBlock qb(p, blockIdx.z / groups);
+  const int b = qb.b, nctx = qb.nctx, nq = qb.nq;
+  const int q0 = g * QG, nqg = max(0, min(QG, nq - q0));
+  if (nqg == 0 && p.splits == 1) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hl = lane & 15, hw = warp * 2 + (lane >> 4);
+  const int total = nctx + qb.nloc;
+  const int per = ((total + p.splits - 1) / p.splits + KEYS - 1) / KEYS * KEYS;
+  const int k0 = s * per, k1 = nqg > 0 ? min(total, k0 + per) : 0;
   const TKV* pool = static_cast<const TKV*>(p.pool) + static_cast<size_t>(p.layer) * p.pool_layer_stride;
+  const bool vec = (reinterpret_cast<uintptr_t>(p.pool) & (4 * sizeof(TKV) - 1)) == 0;
+  const int v_ofs = p.planes / 2 * 16 * HD, lo_ofs = p.planes == 4 ? 16 * HD : 0;
 
-  for (int idx = threadIdx.x; idx < nq * HD; idx += blockDim.x) {
-    const int i = idx / HD, dd = idx % HD;
-    Qs[idx] = q[static_cast<size_t>(qb.row0 + i) * p.ldq + h * HD + dd];
-  }
-
-  float m[QPW], l[QPW], acc[QPW][DPL];
-  unsigned long long msk[QPW];
-#pragma unroll
-  for (int qq = 0; qq < QPW; ++qq) {
-    m[qq] = -INFINITY;
-    l[qq] = 0.f;
-    const int qi = warp + WARPS * qq;
-    msk[qq] = qi < nq ? p.anc[p.q_local0 + qi] : 0ull;
-#pragma unroll
-    for (int r = 0; r < DPL; ++r) acc[qq][r] = 0.f;
-  }
-
-  for (int t = t0; t < t1; ++t) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < KT * HD; idx += blockDim.x) {
-      const int j = idx / HD, dd = idx % HD;
-      const int key = t * KT + j;
-      float kv = 0.f, vv = 0.f;
-      if (key < total) {
-        const int page = p.page_table[b * p.max_pages + (key >> 4)];
-        const TKV* base = pool + (static_cast<size_t>(page) * p.H + h) * p.planes * 16 * HD + (key & 15) * HD + dd;
-        const int vp = p.planes / 2;
-        kv = to_f(base[0]);
-        vv = to_f(base[vp * 16 * HD]);
-        if (p.planes == 4) {
-          kv += to_f(base[16 * HD]);
-          vv += to_f(base[3 * 16 * HD]);
-        }
-      }
-      Ks[j * (HD + 1) + dd] = kv;
-      Vs[j * HD + dd] = vv;
+  const int qi = hl / LPQ;           // this lane's query within the group
+  const unsigned long long mask = qi < nqg ? p.anc[p.q_local0 + q0 + qi] : 0ull;
+  for (int it = threadIdx.x; it < QG * (HD / 4); it += THREADS) {
+    const int i = it / (HD / 4), c = it % (HD / 4) * 4;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < nqg) {
+      const float* src = p.q + static_cast<size_t>(qb.row0 + q0 + i) * p.ldq + h * HD + c;
+      x = make_float4(src[0], src[1], src[2], src[3]);
     }
-    __syncthreads();
-    const int key = t * KT + lane;
+    *reinterpret_cast<float4*>(qs + i * HD + c) = x;
+  }
+  __syncthreads();
+
+  float m = -INFINITY, l = 0.f;
+  float4 acc[QG][DV];
 #pragma unroll
-    for (int qq = 0; qq < QPW; ++qq) {
-      const int qi = warp + WARPS * qq;
-      if (qi < nq) {
-        const bool vis = key < nctx || (key < total && ((msk[qq] >> (key - nctx)) & 1ull));
-        float sc = -INFINITY;
-        if (vis) {
-          float d = 0.f;
-#pragma unroll 16
-          for (int dd = 0; dd < HD; ++dd) d = fmaf(Qs[qi * HD + dd], Ks[lane * (HD + 1) + dd], d);
-          sc = d * p.scale;
-        }
-        const float mnew = fmaxf(m[qq], warp_max(sc));
-        if (mnew != -INFINITY) {
-          const float pj = vis ? expf(sc - mnew) : 0.f;
-          const float corr = expf(m[qq] - mnew);
-          l[qq] = l[qq] * corr + warp_sum(pj);
+  for (int q = 0; q < QG; ++q)
 #pragma unroll
-          for (int r = 0; r < DPL; ++r) acc[qq][r] *= corr;
-          for (int j = 0; j < KT; ++j) {
-            const float pjj = __shfl_sync(0xffffffffu, pj, j);
+    for (int d = 0; d < DV; ++d) acc[q][d] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+  for (int base = k0; base < k1; base += KEYS) {
+    // key base + 16 u + hw: row hw of page base / 16 + u
+    float4 kk[4][DV], vv[4][DV];
 #pragma unroll
-            for (int r = 0; r < DPL; ++r) acc[qq][r] = fmaf(pjj, Vs[j * HD + lane + 32 * r], acc[qq][r]);
-          }
-          m[qq] = mnew;
+    for (int u = 0; u < 4; ++u) {
+      const bool in = base + 16 * u + hw < k1;
+      const int page = in ? p.page_table[b * p.max_pages + base / 16 + u] : 0;
+      const TKV* row = pool + (static_cast<size_t>(page) * p.H + h) * p.planes * 16 * HD + hw * HD + hl * 4;
+#pragma unroll
+      for (int d = 0; d < DV; ++d) {
+        kk[u][d] = in ? load_kv4(row + 64 * d, lo_ofs, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vv[u][d] = in ? load_kv4(row + v_ofs + 64 * d, lo_ofs, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    float part[4][QG];
+#pragma unroll
+    for (int q = 0; q < QG; ++q) {
+#pragma unroll
+      for (int d = 0; d < DV; ++d) {
+        const float4 x = *reinterpret_cast<const float4*>(qs + q * HD + 64 * d + hl * 4);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float t = fmaf(x.x, kk[u][d].x, fmaf(x.y, kk[u][d].y, fmaf(x.z, kk[u][d].z, x.w * kk[u][d].w)));
+          part[u][q] = d ? part[u][q] + t : t;
         }
       }
     }
+    float sc[4], mx = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int key = base + 16 * u + hw;
+      const float t = half_sum_many(part[u], lane);
+      const bool vis = key < k1 && (key < nctx || ((mask >> (key - nctx)) & 1ull));
+      sc[u] = vis ? t * p.scale : -INFINITY;
+      mx = fmaxf(mx, sc[u]);
+    }
+    const float mn = fmaxf(m, mx);
+    const float corr = m == mn ? 1.f : expf(m - mn);  // (m = -inf: 0)
+    float pr[4];
+    l *= corr;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      pr[u] = sc[u] == -INFINITY ? 0.f : expf(sc[u] - mn);
+      l += pr[u];
+    }
+    m = mn;
+    const bool rescale = __any_sync(0xffffffffu, corr != 1.f);
+#pragma unroll
+    for (int q = 0; q < QG; ++q) {
+      const int src = (lane & 16) + q * LPQ;
+      if (rescale) {
+        const float c = __shfl_sync(0xffffffffu, corr, src);
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+          acc[q][d].x *= c; acc[q][d].y *= c; acc[q][d].z *= c; acc[q][d].w *= c;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float w = __shfl_sync(0xffffffffu, pr[u], src);
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+          acc[q][d].x = fmaf(w, vv[u][d].x, acc[q][d].x);
+          acc[q][d].y = fmaf(w, vv[u][d].y, acc[q][d].y);
+          acc[q][d].z = fmaf(w, vv[u][d].z, acc[q][d].z);
+          acc[q][d].w = fmaf(w, vv[u][d].w, acc[q][d].w);
+        }
+      }
+    }
   }
 
+  // ---- the two half-warps of a warp, then the eight warps ----
+  {
+    const float M = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    const float f = m == -INFINITY ? 0.f : expf(m - M);
+    l *= f;
+    l += __shfl_xor_sync(0xffffffffu, l, 16);
+#pragma unroll
+    for (int q = 0; q < QG; ++q) {
+      const float c = __shfl_sync(0xffffffffu, f, (lane & 16) + q * LPQ);
+#pragma unroll
+      for (int d = 0; d < DV; ++d) {
+        float4 t = acc[q][d];
+        t.x *= c; t.y *= c; t.z *= c; t.w *= c;
+        t.x += __shfl_xor_sync(0xffffffffu, t.x, 16);
+        t.y += __shfl_xor_sync(0xffffffffu, t.y, 16);
+        t.z += __shfl_xor_sync(0xffffffffu, t.z, 16);
+        t.w += __shfl_xor_sync(0xffffffffu, t.w, 16);
+        if (lane < 16) *reinterpret_cast<float4*>(s_acc + (warp * QG + q) * HD + 64 * d + hl * 4) = t;
+      }
+    }
+    if (lane < 16 && hl % LPQ == 0) {
+      s_m[warp * QG + qi] = M;
+      s_l[warp * QG + qi] = l;
+    }
+  }
+  __syncthreads();
   T* out = static_cast<T*>(p.out);
   T* out_lo = static_cast<T*>(p.out_lo);
-  if (p.splits == 1) {
-#pragma unroll
-    for (int qq = 0; qq < QPW; ++qq) {
-      const int qi = warp + WARPS * qq;
-      if (qi < nq) {
-        const float inv = l[qq] > 0.f ? 1.f / l[qq] : 0.f;
-#pragma unroll
-        for (int r = 0; r < DPL; ++r)
-          store_act(out, out_lo, static_cast<size_t>(qb.row0 + qi) * p.ldo + h * HD + lane + 32 * r,
-                    acc[qq][r] * inv);
-      }
-    }
-    return;
-  }
-
   const size_t rec = HD + 4;
   float* wsb = p.ws + (static_cast<size_t>(b * p.H + h) * p.splits) * p.nq_max * rec;
+  for (int it = threadIdx.x; it < nqg * (HD / 4); it += THREADS) {
+    const int q = it / (HD / 4), c = it % (HD / 4) * 4;
+    float M = -INFINITY, L = 0.f;
 #pragma unroll
-  for (int qq = 0; qq < QPW; ++qq) {
-    const int qi = warp + WARPS * qq;
-    if (qi < nq) {
-      float* w = wsb + (static_cast<size_t>(s) * p.nq_max + qi) * rec;
+    for (int w = 0; w < WARPS; ++w) M = fmaxf(M, s_m[w * QG + q]);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int r = 0; r < DPL; ++r) __stcg(&w[lane + 32 * r], acc[qq][r]);
-      if (lane == 0) {
-        __stcg(&w[HD], m[qq]);
-        __stcg(&w[HD + 1], l[qq]);
+    for (int w = 0; w < WARPS; ++w) {
+      const float mw = s_m[w * QG + q];
+      const float f = mw == -INFINITY ? 0.f : expf(mw - M);
+      L += f * s_l[w * QG + q];
+      const float4 t = *reinterpret_cast<const float4*>(s_acc + (w * QG + q) * HD + c);
+      o.x = fmaf(f, t.x, o.x); o.y = fmaf(f, t.y, o.y); o.z = fmaf(f, t.z, o.z); o.w = fmaf(f, t.w, o.w);
+    }
+    if (p.splits == 1) {
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+      const float4 y = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
+      const size_t at = static_cast<size_t>(qb.row0 + q0 + q) * p.ldo + h * HD + c;
+      store_act(out, out_lo, at, y.x);
+      store_act(out, out_lo, at + 1, y.y);
+      store_act(out, out_lo, at + 2, y.z);
+      store_act(out, out_lo, at + 3, y.w);
+    } else {
+      float* w = wsb + (static_cast<size_t>(s) * p.nq_max + q0 + q) * rec;
+      __stcg(reinterpret_cast<float4*>(w + c), o);
+      if (c == 0) {
+        __stcg(&w[HD], M);
+        __stcg(&w[HD + 1], L);
       }
     }
   }
+  if (p.splits == 1) return;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     const int old = atomicAdd(&p.counters[b * p.H + h], 1);
-    s_last = (old == p.splits - 1) ? 1 : 0;
+    s_last = (old == p.splits * groups - 1) ? 1 : 0;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  combine_splits(p, wsb, nq, HD, qb.row0, h, out, out_lo, sm);  // the K/V tile area is free now
+  combine_splits(p, wsb, nq, HD, qb.row0, h, out, out_lo, s_acc);
   if (threadIdx.x == 0) p.counters[b * p.H + h] = 0;
 }
 
-constexpr int ATT_MAX_DEVICES = 64;
-std::mutex g_attr_mu;
-
 template <typename TKV, typename T, int HD>
-cudaError_t launch(const AttnParams& p, cudaStream_t s) {
-  const size_t smem = (KT * (HD + 1) + KT * HD + static_cast<size_t>(p.nq_max) * HD) * sizeof(float);
-  // the shared-memory limit is a per-device attribute: raised once per device
-  static bool attr[ATT_MAX_DEVICES];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= ATT_MAX_DEVICES) return cudaErrorInvalidDevice;
-  {
-    std::lock_guard<std::mutex> lk(g_attr_mu);
-    if (!attr[dev]) {
-      e = cudaFuncSetAttribute(attn_kernel<TKV, T, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (e != cudaSuccess) return e;
-      attr[dev] = true;
-    }
-  }
-  dim3 grid(p.splits, p.H, p.B * std::max(1, p.q_blocks));
-  launch_pdl(attn_kernel<TKV, T, HD>, dim3(grid), dim3(WARPS * 32), smem, s, p);
+cudaError_t launch(AttnParams p, cudaStream_t s) {
+  constexpr int QG = 1024 / HD;  // 16 queries of 64 dims or 8 of 128 per CTA
+  static_assert(WARPS * 1024 >= MAX_NQ * MAX_SPLITS, "the merge weights fit over the partials");
+  // the page table bounds the context: a split of fewer than SPLIT_KEYS keys only adds a merge
+  p.splits = std::max(1, std::min(p.splits, (p.max_pages * 16 + SPLIT_KEYS - 1) / SPLIT_KEYS));
+  const int groups = p.nq_max == 1 ? 1 : (p.nq_max + QG - 1) / QG;
+  const dim3 grid(p.splits, p.H, p.B * std::max(1, p.q_blocks) * groups);
+  if (p.nq_max == 1)
+    launch_pdl(attn_kernel<TKV, T, HD, 1>, grid, dim3(THREADS), 0, s, p, groups);
+  else
+    launch_pdl(attn_kernel<TKV, T, HD, QG>, grid, dim3(THREADS), 0, s, p, groups);
   return cudaGetLastError();
 }
 
@@ -299,7 +378,7 @@ int attn_pick_splits(int dtype, int hd, int planes, int B, int H, int want) {
 }
 
 cudaError_t attention(const AttnParams& p, int dtype, cudaStream_t s) {
-  if (p.nq_max > WARPS * QPW || p.n_local > 64 || p.splits > MAX_SPLITS || p.splits < 1) return cudaErrorInvalidValue;
+  if (p.nq_max > MAX_NQ || p.nq_max < 1 || p.n_local > 64 || p.splits > MAX_SPLITS || p.splits < 1) return cudaErrorInvalidValue;
   if (p.planes != 2 && !(p.planes == 4 && dtype == 1)) return cudaErrorInvalidValue;
   // blocks of prompt rows: device row counts, no fused projections, one split per block
   if (p.q_blocks > 1 && (p.qkv || !p.nq_dev || !p.n_local_dev || p.q_local0 != 0 || p.nq != 64 || p.n_local != 64 || p.splits != 1))

@@ -231,6 +231,51 @@ def test_attention_tree_masked_paged(dtype, case):
             assert err <= tol, (b, i, err)
 
 
+# the SIMT kernel (fp32 models, head_dim 64): one query and query groups of 16 (8 at head_dim
+# 128), contexts below, at and past a 64-key pass and a 256-key split, planes of both types,
+# a pool that is not aligned for vectors
+@pytest.mark.parametrize("dtype,hd", [("fp32", 64), ("fp32", 128), ("bf16", 64), ("bf16_split", 64)])
+@pytest.mark.parametrize("nctx,nq,splits", [([0], 1, 1), ([64, 63], 1, 16), ([700, 5], 1, 3), ([130], 9, 2), ([300, 0], 64, 16)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_attention_simt(dtype, hd, nctx, nq, splits, offset):
+    B, H, n_local = len(nctx), 3, max(nq, 2)
+    rng = np.random.default_rng(nq + splits)
+    max_pages = (max(nctx) + n_local + 15) // 16
+    perm = rng.permutation(B * max_pages).reshape(B, max_pages).astype(np.int32)
+    kv = torch.randn(B * max_pages, H, 2, 16, hd, generator=torch.Generator().manual_seed(nq))
+    hi = kv.to(torch.bfloat16)
+    pool = kv if dtype == "fp32" else hi
+    ref_kv = pool.double().numpy()
+    if dtype == "bf16_split":
+        lo = (kv - hi.float()).to(torch.bfloat16)
+        pool = torch.stack([hi[:, :, 0], lo[:, :, 0], hi[:, :, 1], lo[:, :, 1]], dim=2)
+        ref_kv = np.stack([(hi + 0).double().numpy()[:, :, i] + lo.double().numpy()[:, :, i] for i in (0, 1)], 2)
+    flat = torch.zeros(pool.numel() + 4, dtype=pool.dtype, device="cuda")
+    flat[offset:offset + pool.numel()] = pool.reshape(-1).cuda()
+    dev = flat[offset:offset + pool.numel()].view(pool.shape)
+    q = torch.randn(B * nq, H * hd, generator=torch.Generator().manual_seed(9))
+    q0 = n_local - nq  # the queries are the last local rows of a causal chain
+    anc = np.array([(1 << (i + 1)) - 1 for i in range(n_local)], dtype=np.uint64)
+    out = torch.zeros(B * nq, H * hd, dtype=torch.float32 if dtype == "fp32" else torch.bfloat16, device="cuda")
+    out_lo = None if dtype == "fp32" else torch.zeros_like(out)
+    for _ in range(2):  # the split counters are back at zero after a launch
+        pkg.op_attention(q.cuda(), dev, torch.tensor(perm, device="cuda"),
+                         torch.tensor(nctx, dtype=torch.int32, device="cuda"),
+                         torch.tensor(anc.view(np.int64), device="cuda"), out, nq=nq, q_local0=q0, n_local=n_local,
+                         q_rows=nq, n_heads=H, head_dim=hd, splits=splits, out_lo=out_lo)
+        pkg.op_sync()
+    got = out.double() + (0 if out_lo is None else out_lo.double())
+    got = got.cpu().numpy().reshape(B, nq, H, hd)
+    Q = q.double().numpy().reshape(B, nq, H, hd)
+    for b in range(B):
+        for i in range(nq):
+            slots = range(nctx[b] + q0 + i + 1)
+            K, V = (np.stack([ref_kv[perm[b, t // 16], :, j, t % 16] for t in slots]) for j in (0, 1))
+            ref = co.attend(Q[b, i], K, V)
+            # fp32 sums; a bf16 output is a hi + lo pair (2^-17)
+            assert np.max(np.abs(got[b, i] - ref)) / np.max(np.abs(ref)) <= (1e-5 if dtype == "fp32" else 2e-5), (b, i)
+
+
 @pytest.mark.parametrize("jump", [40.0, 150.0])
 @pytest.mark.parametrize("splits", [1, 2])
 def test_attention_rescale_after_one_sided_tile(jump, splits):
