@@ -426,3 +426,25 @@ def test_prefill_chunks(name, lens):
             rk = st.dK[:len(x)] if layer < 0 else st.K[layer, :len(x)]
             rv = st.dV[:len(x)] if layer < 0 else st.V[layer, :len(x)]
             assert rel_rows(k, rk) <= tol and rel_rows(v, rv) <= tol, (b, layer)
+
+
+@pytest.mark.parametrize("name", ["tiny", "mini"])
+def test_prefill_again(name):
+    # prompts of the same and of other lengths, batches and chunks on one context: the plans and
+    # step graphs it keeps must be those that a new context would make
+    cfg, w_cpu, w_dev = _setup(name)
+    rng = np.random.default_rng(3)
+    ctx = pkg.Chimera(cfg, w_dev, max_batch=2, max_seq_len=800)
+    for lens in ([40], [40], [300, 20], [33, 64], [500], [40]):
+        prompts = [rng.integers(0, cfg["vocab"], n).tolist() for n in lens]
+        got = []
+        for c in (ctx, pkg.Chimera(cfg, w_dev, max_batch=2, max_seq_len=800)):
+            c.prefill(prompts)
+            got.append((c.read("prefill_logits"), c.step(), c.read("verify_logits"), c.read("draft_logits"),
+                        c.ar_generate(1), c.read("prefill_logits")))
+        # two contexts sum the same split-K partials in different orders
+        for a, b in zip(*got):
+            if isinstance(a, np.ndarray):
+                assert rel_rows(a, b) <= (1e-6 if name == "tiny" else 1e-4), lens
+            else:
+                assert a == b, lens
