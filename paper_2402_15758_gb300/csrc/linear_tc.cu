@@ -97,23 +97,55 @@ __device__ __forceinline__ void epi_store16(const TcLinearParams& p, int m0, int
   }
 }
 
-// EPI_RESID with float4 reductions: the warp's 32 feature rows x 16 token columns go
-// through shared memory (sw: [16][33] floats) so that each lane adds runs of four
-// consecutive features of one token (one vector red.global.add instead of four).
-__device__ __forceinline__ void epi_red16(const TcLinearParams& p, int m0, int f0, int lane, const float (&v)[16],
-                                          float* sw) {
+// 32 lanes x 16 columns without a wait, and the wait (naming the registers, so that no use
+// of them is moved above it).
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+
+// EPI_RESID with float4 reductions: the warp's 32 feature rows x 16 NB token columns (with a
+// split, the hi columns plus the lo ones BN further) go through shared memory
+// (sw: [16 NB][RED_PITCH] floats) so that each lane adds runs of four consecutive features
+// of one token (one vector red.global.add instead of four).  All of the tensor-memory
+// loads are in flight before the one wait: a 64-row tile's drain, which ends every launch,
+// took 1.35 us with a wait after each 16 columns, hi and lo.
+constexpr int RED_PITCH = 36;
+template <int NB>
+__device__ __forceinline__ void epi_red(const TcLinearParams& p, uint32_t taddr, int m0, int f0, int lane, float* sw) {
+  uint32_t hi[NB][16], lo[NB][16];
 #pragma unroll
-  for (int j = 0; j < 16; ++j) sw[j * 33 + lane] = v[j];
+  for (int b = 0; b < NB; ++b) tmem_ld16_async(taddr + 16 * b, hi[b]);
+  if (p.has_lo) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) tmem_ld16_async(taddr + p.BN + 16 * b, lo[b]);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) tmem_wait16(lo[b]);
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    tmem_wait16(hi[b]);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      sw[(16 * b + j) * RED_PITCH + lane] =
+          p.has_lo ? __uint_as_float(hi[b][j]) + __uint_as_float(lo[b][j]) : __uint_as_float(hi[b][j]);
+  }
   __syncwarp();
   float* y = static_cast<float*>(p.Y);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int idx = i * 32 + lane;
-    const int c = idx >> 3, k = (idx & 7) * 4;  // token c, features f0 + k .. f0 + k + 3
-    if (m0 + c < p.M && f0 + k < p.N) {
-      const float* s = sw + c * 33 + k;
-      red_add_v4(y + static_cast<size_t>(m0 + c) * p.ldy + f0 + k, make_float4(s[0], s[1], s[2], s[3]));
-    }
+  for (int i = 0; i < 4 * NB; ++i) {
+    const int c = i * 4 + (lane >> 3), k = (lane & 7) * 4;  // token c, features f0 + k .. f0 + k + 3
+    if (m0 + c < p.M && f0 + k < p.N)
+      red_add_v4(y + static_cast<size_t>(m0 + c) * p.ldy + f0 + k, *reinterpret_cast<const float4*>(sw + c * RED_PITCH + k));
   }
   __syncwarp();
 }
@@ -132,6 +164,12 @@ __device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
 }
 
 
+// RED: the fp32 accumulating epilogue with vector reductions, which every linear of a step
+// but the trigram encoder's takes.  The other epilogues are a variant of their own: their
+// workspace path needs 70 more registers, and a CTA that holds them leaves the SM too
+// few for two CTAs of the row kernel that overlaps the launch (SwiGLU: 62 x 256; one
+// kernel for both made the linears 1 % faster and the step 1 % slower).
+template <bool RED>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const __grid_constant__ TcLinearParams p) {
   if (p.skip) {
     // the flag is written by the previous kernel: read it after the dependency wait,
@@ -158,7 +196,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_last = s_abort + 1;
-  float* s_red = reinterpret_cast<float*>(smem + p.stages * stage_bytes + 1024);  // [4 warps][16][33]
+  float* s_red = reinterpret_cast<float*>(smem + p.stages * stage_bytes + 1024);  // [4 warps][32][RED_PITCH]
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -346,21 +384,29 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       if (bar_any(1, 128, !ok)) break;
       tc_fence_after();
       const int ft = t / p.tok_tiles, tt = t % p.tok_tiles;
+      const int m0 = tt * p.BN;
+      const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * p.acc_stride;
+      if constexpr (RED) {
+        float* sw = s_red + q * 32 * RED_PITCH;
+        int c0 = 0;
+        for (; c0 + 32 <= p.BN; c0 += 32) epi_red<2>(p, tbase + c0, m0 + c0, ft * BM + q * 32, lane, sw);
+        if (c0 < p.BN) epi_red<1>(p, tbase + c0, m0 + c0, ft * BM + q * 32, lane, sw);
+        tc_fence_before();
+        mbar_arrive(&tempty[buf]);
+        buf ^= 1;
+        if (buf == 0) aphase ^= 1u;
+        continue;
+      }
       const uint32_t tu0 = static_cast<uint32_t>(t) * KB;
       const int c_first = cta_of_unit(tu0, U, G);
       const int c_last = cta_of_unit(tu0 + KB - 1, U, G);
       const int nparts = c_last - c_first + 1;
       const int f = ft * BM + row;
-      const int m0 = tt * p.BN;
-      const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * p.acc_stride;
       if (nparts == 1 || p.epi == EPI_RESID) {
         for (int c0 = 0; c0 < p.BN; c0 += 16) {
           float v[16];
           load16(tbase + c0, v);
-          if (p.vec_red)
-            epi_red16(p, m0 + c0, ft * BM + q * 32, lane, v, s_red + q * 16 * 33);
-          else
-            epi_store16(p, m0 + c0, f, v);
+          epi_store16(p, m0 + c0, f, v);
         }
         tc_fence_before();
         mbar_arrive(&tempty[buf]);
@@ -580,7 +626,7 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   plan->grid = static_cast<int>(p.units < sms ? p.units : sms);
   // float4 reductions need 16-byte aligned rows of Y and whole float4 runs of features
   p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && N % 4 == 0) ? 1 : 0;
-  plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 16 * 33 * sizeof(float);
+  plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 32 * RED_PITCH * sizeof(float);
   plan->weight_bytes = 2.0 * N * K;
   plan->pair.grid = 0;
   if (X_lo && M > PAIR_ROWS) {
@@ -611,12 +657,17 @@ cudaError_t tc_linear_launch(const TcLinearPlan& plan, cudaStream_t s) {
   {
     std::lock_guard<std::mutex> lk(g_attr_mu);
     if (!g_attr_set[dev]) {
-      e = cudaFuncSetAttribute(tc_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      e = cudaFuncSetAttribute(tc_linear_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc_linear_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       if (e != cudaSuccess) return e;
       g_attr_set[dev] = true;
     }
   }
-  launch_pdl(tc_linear_kernel, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
+  if (plan.p.vec_red)
+    launch_pdl(tc_linear_kernel<true>, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
+  else
+    launch_pdl(tc_linear_kernel<false>, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
   return cudaGetLastError();
 }
 
