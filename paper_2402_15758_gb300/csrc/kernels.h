@@ -178,10 +178,18 @@ cudaError_t chain_launch(const ChainPlan& plan, cudaStream_t s);
 // skip (optional, device): when *skip != 0 at run time the launch does nothing (its
 // output was provided another way, e.g. by the trigram cache).  W2 (optional, N2 rows):
 // a second weight whose outputs follow W's in Y.  early_w: no kernel of the stream
-// writes the weights, so they may be read before the launch's dependency wait.
+// writes the weights, so they may be read before the launch's dependency wait.  The
+// prologue folds the row operation before the linear into it: y = W RMSNorm(x; g, eps), or
+// W (SiLU(x[:K]) x[K:2K]) with rows of 2K (worth it up to F32_SWIGLU_ROWS rows).
+constexpr int F32_SWIGLU_ROWS = 4;
+struct F32Prologue {
+  const float* g = nullptr;
+  float eps = 0.f;
+  bool swiglu = false;
+};
 cudaError_t f32_linear(int M, int N, int K, const float* X, int ldx, const float* W, float* Y,
                        int ldy, int epi, cudaStream_t s, const int* skip = nullptr, const float* W2 = nullptr,
-                       int N2 = 0, bool early_w = false);
+                       int N2 = 0, bool early_w = false, const F32Prologue& pro = F32Prologue());
 
 // ----------------------------------------------------------------------------
 // attention over the paged KV cache with a per-query ancestor bitmask

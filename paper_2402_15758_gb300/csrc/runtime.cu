@@ -41,6 +41,7 @@ struct Lin {
   int N2 = 0;
   void* Y = nullptr;
   const int* skip = nullptr;  // device flag: nonzero -> the launch does nothing
+  F32Prologue pro;            // fp32 models: the row operation folded in
   double bytes = 0;
 };
 
@@ -351,7 +352,7 @@ cudaError_t run_lin(chimera_ctx* ctx, const Lin& l) {
   if (l.tc) return tc_linear_launch(l.tp, ctx->stream);
   return f32_linear(l.M, l.N, l.K, static_cast<const float*>(l.X), l.ldx, static_cast<const float*>(l.W),
                     static_cast<float*>(l.Y), l.ldy, l.epi, ctx->stream, l.skip, static_cast<const float*>(l.W2), l.N2,
-                    true);
+                    true, l.pro);
 }
 
 bool make_lin(chimera_ctx* ctx, Lin* l, int M, int N, int K, const void* X, const void* X_lo, int ldx,
@@ -518,6 +519,25 @@ cudaError_t run_norm(chimera_ctx* ctx, const float* X, const void* g, int rows, 
                  zcols, zcols, ctx->stream);
 }
 
+// fp32 models fold a norm into the linear that follows it, which also stores its output
+// instead of adding to a cleared one; see fold_norm.
+bool folds(const chimera_ctx* ctx) { return ctx->dtype == 0; }
+void fold_norm(const chimera_ctx* ctx, Lin* l, const float* X, const void* g) {
+  if (!folds(ctx)) return;
+  l->X = X;
+  l->ldx = ctx->d;
+  l->pro.g = static_cast<const float*>(g);
+  l->pro.eps = ctx->cfg.rms_eps;
+}
+// SwiGLU of `rows` rows is folded into the down projection.
+bool folds_swiglu(const chimera_ctx* ctx, int rows) { return folds(ctx) && rows <= F32_SWIGLU_ROWS; }
+void fold_swiglu(const chimera_ctx* ctx, Lin* l) {
+  if (!folds_swiglu(ctx, l->M)) return;
+  l->X = ctx->gu;
+  l->ldx = 2 * ctx->F;
+  l->pro.swiglu = true;
+}
+
 // Final norm: H_LLM rows in fp32 plus the LM-head operand (+ lo half); zeroes the
 // logits rows when the LM head follows.
 cudaError_t run_final_norm(chimera_ctx* ctx, int rows, bool zero_logits) {
@@ -581,7 +601,7 @@ cudaError_t enqueue_layer(chimera_ctx* ctx, int l, const Lin* lin, int rows, int
   // the accumulators of the QKV and gate|up linears are cleared by the norms, or (tensor-
   // core linears) by the previous layer's down linear and this layer's O linear
   const bool z = !ctx->tc_zero;
-  RUN(run_norm(ctx, ctx->x, w.attn_norm, rows, (z || l == 0) ? ctx->qkv : nullptr, 3 * d));
+  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.attn_norm, rows, (z || l == 0) ? ctx->qkv : nullptr, 3 * d));
   RUN(run_lin(ctx, lin[0]));
   const int blocks = (rows_per_seq + CHUNK - 1) / CHUNK, nq = std::min(rows_per_seq, CHUNK);
   if (blocks == 1 && attn_fuses_rope(ctx->dtype, ctx->hd)) {
@@ -593,10 +613,11 @@ cudaError_t enqueue_layer(chimera_ctx* ctx, int l, const Lin* lin, int rows, int
                       nullptr, blocks));
   }
   RUN(run_lin(ctx, lin[1]));
-  RUN(run_norm(ctx, ctx->x, w.ffn_norm, rows, z ? ctx->gu : nullptr, 2 * ctx->F));
+  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.ffn_norm, rows, z ? ctx->gu : nullptr, 2 * ctx->F));
   RUN(run_lin(ctx, lin[2]));
   RUN(run_lin(ctx, lin[3]));
-  LAUNCH(CHIMERA_KIND_SWIGLU, 0, swiglu(ctx->dtype, ctx->gu, 2 * ctx->F, ctx->F, ctx->hf, ctx->hf_lo, ctx->F, rows, ctx->stream));
+  if (!folds_swiglu(ctx, rows))
+    LAUNCH(CHIMERA_KIND_SWIGLU, 0, swiglu(ctx->dtype, ctx->gu, 2 * ctx->F, ctx->F, ctx->hf, ctx->hf_lo, ctx->F, rows, ctx->stream));
   RUN(run_lin(ctx, lin[4]));
   return cudaSuccess;
 }
@@ -637,7 +658,7 @@ cudaError_t enqueue_step(chimera_ctx* ctx) {
     }
     // sub-step 0 also clears every head's score rows, which the head linears accumulate
     // into (off the chain of the later sub-steps)
-    const bool sep_heads = !ctx->use_chain;
+    const bool sep_heads = !ctx->use_chain && !folds(ctx);
     LAUNCH(CHIMERA_KIND_EMBED, 0, launch_trigram_gather(ctx->dtype, ctx->embed, d, V, ctx->d_n, ctx->d_tok, ctx->tok_stride, ctx->d_topk, K,
                                 ctx->KMAX, k, ctx->tbuf, B, ctx->d_err, ctx->dres, s,
                                 (sep_heads && k == 0) ? ctx->hlog : nullptr, static_cast<long long>(K) * B * V));
@@ -662,7 +683,7 @@ cudaError_t enqueue_step(chimera_ctx* ctx) {
                                              ctx->topk_ws_v, ctx->topk_ws_i, ctx->topk_cnt, s));
       continue;
     }
-    RUN(run_norm(ctx, ctx->dres, ctx->draft.attn_norm, B, ctx->qkv, 3 * d));
+    if (!folds(ctx)) RUN(run_norm(ctx, ctx->dres, ctx->draft.attn_norm, B, ctx->qkv, 3 * d));
     RUN(run_lin(ctx, ctx->dqkv));
     if (attn_fuses_rope(ctx->dtype, ctx->hd)) {
       RUN(run_attention(ctx, true, 0, 1, nullptr, k, k + 1, nullptr, ctx->d_chain, 1, ctx->att_splits_draft, 1,
@@ -673,10 +694,11 @@ cudaError_t enqueue_step(chimera_ctx* ctx) {
                         kv_read_bytes(ctx, k + 1, true)));
     }
     RUN(run_lin(ctx, ctx->dwo));
-    RUN(run_norm(ctx, ctx->dres, ctx->draft.ffn_norm, B, ctx->gu, 2 * ctx->F));
+    if (!folds(ctx)) RUN(run_norm(ctx, ctx->dres, ctx->draft.ffn_norm, B, ctx->gu, 2 * ctx->F));
     RUN(run_lin(ctx, ctx->dgate));
     RUN(run_lin(ctx, ctx->dup));
-    LAUNCH(CHIMERA_KIND_SWIGLU, 0, swiglu(ctx->dtype, ctx->gu, 2 * ctx->F, ctx->F, ctx->hf, ctx->hf_lo, ctx->F, B, s));
+    if (!folds_swiglu(ctx, B))
+      LAUNCH(CHIMERA_KIND_SWIGLU, 0, swiglu(ctx->dtype, ctx->gu, 2 * ctx->F, ctx->F, ctx->hf, ctx->hf_lo, ctx->F, B, s));
     RUN(run_lin(ctx, ctx->ddown));
     LAUNCH(CHIMERA_KIND_OTHER, 0, launch_hfull_store(ctx->dtype, ctx->dres, d, ctx->headin, ctx->headin_lo,
                              ctx->hfull_log + static_cast<size_t>(k) * B * d, nullptr, V, B, s));
@@ -700,7 +722,7 @@ cudaError_t enqueue_step(chimera_ctx* ctx) {
     for (int l = 0; l < ctx->L; ++l)
       RUN(enqueue_layer(ctx, l, &ctx->ver[5 * l], B * N, N, nullptr, ctx->d_depth, ctx->d_anc, ctx->att_splits_ver,
                         kvb));
-    RUN(run_final_norm(ctx, B * N, true));
+    RUN(run_final_norm(ctx, B * N, !folds(ctx)));
     RUN(run_lin(ctx, ctx->ver_lm));
   }
   LAUNCH(CHIMERA_KIND_ARGMAX, 0, argmax_rows(ctx->logits, V, B * N, ctx->d_amax, s, ctx->d_stats));
@@ -723,7 +745,7 @@ cudaError_t enqueue_step(chimera_ctx* ctx) {
   if (ctx->use_chain) {
     RUN(run_chain(ctx, ctx->commit_chain));
   } else {
-    RUN(run_norm(ctx, ctx->hsel, ctx->draft.attn_norm, B * ctx->D1, ctx->kvtmp, 2 * d));
+    if (!folds(ctx)) RUN(run_norm(ctx, ctx->hsel, ctx->draft.attn_norm, B * ctx->D1, ctx->kvtmp, 2 * d));
     RUN(run_lin(ctx, ctx->commit_kv));
   }
   RUN(run_rope(ctx, true, 0, ctx->kvtmp, 2 * d, -1, 0, d, ctx->D1, ctx->d_L, 1, 0, 0, nullptr));
@@ -750,7 +772,7 @@ cudaError_t enqueue_ar_step(chimera_ctx* ctx) {
   } else {
     for (int l = 0; l < ctx->L; ++l)
       RUN(enqueue_layer(ctx, l, &ctx->ar[5 * l], B, 1, nullptr, nullptr, ctx->d_chain, ctx->att_splits_ar, kvb));
-    RUN(run_final_norm(ctx, B, true));
+    RUN(run_final_norm(ctx, B, !folds(ctx)));
     RUN(run_lin(ctx, ctx->ar_lm));
   }
   LAUNCH(CHIMERA_KIND_ARGMAX, 0, argmax_rows(ctx->logits, V, B, ctx->d_amax, s));
@@ -764,7 +786,7 @@ cudaError_t enqueue_ar_step(chimera_ctx* ctx) {
   if (ctx->use_chain) {
     RUN(run_chain(ctx, ctx->commit_chain));
   } else {
-    RUN(run_norm(ctx, ctx->hsel, ctx->draft.attn_norm, B * ctx->D1, ctx->kvtmp, 2 * d));
+    if (!folds(ctx)) RUN(run_norm(ctx, ctx->hsel, ctx->draft.attn_norm, B * ctx->D1, ctx->kvtmp, 2 * d));
     RUN(run_lin(ctx, ctx->commit_kv));
   }
   RUN(run_rope(ctx, true, 0, ctx->kvtmp, 2 * d, -1, 0, d, ctx->D1, ctx->d_L, 1, 0, 0, nullptr));
@@ -971,35 +993,40 @@ bool build_plans(chimera_ctx* ctx, int B) {
   ctx->plan_batch = ctx->plan_chunk = 0;  // (until every plan is built)
   const int d = ctx->d, F = ctx->F, V = ctx->V, N = ctx->N;
   const int f32 = 1, tb = ctx->dtype == 0 ? 1 : 0;  // bf16 storage -> out_f32 = 0
-  // fp32 outputs accumulate (split-K partials added atomically) into buffers that the
-  // preceding kernel zeroed, or into the residual stream itself
+  // bf16 models' fp32 outputs accumulate (split-K partials added atomically) into buffers
+  // that an earlier kernel zeroed, or into the residual stream itself
+  const int OUT = folds(ctx) ? EPI_STORE : EPI_RESID;
   constexpr int ACC = EPI_RESID;
   void *xn = ctx->xn, *xl = ctx->xn_lo, *ao = ctx->ao, *al = ctx->ao_lo, *hf = ctx->hf, *hl = ctx->hf_lo;
   auto layer_plans = [&](std::vector<Lin>& v, int M) {
     for (int l = 0; l < ctx->L; ++l) {
       const chimera_block_weights& w = ctx->layers[l];
       Lin* p = &v[5 * l];
-      if (!make_lin(ctx, &p[0], M, 3 * d, d, xn, xl, d, w.wqkv, ctx->qkv, nullptr, 3 * d, ACC, f32)) return false;
+      if (!make_lin(ctx, &p[0], M, 3 * d, d, xn, xl, d, w.wqkv, ctx->qkv, nullptr, 3 * d, OUT, f32)) return false;
+      fold_norm(ctx, &p[0], ctx->x, w.attn_norm);
       // the O linear clears the gate|up accumulator of this layer, the down linear the
       // QKV accumulator of the next one (their epilogue warps, off the critical path)
       if (!make_lin(ctx, &p[1], M, d, d, ao, al, d, w.wo, ctx->x, nullptr, d, ACC, f32, nullptr, 0,
                     ctx->tc_zero ? ctx->gu : nullptr, static_cast<long long>(M) * 2 * F))
         return false;
       // gate and up: one launch writing gu[:, 0:F] and gu[:, F:2F]
-      if (!make_lin(ctx, &p[2], M, F, d, xn, xl, d, w.w_gate, ctx->gu, nullptr, 2 * F, ACC, f32, w.w_up, F))
+      if (!make_lin(ctx, &p[2], M, F, d, xn, xl, d, w.w_gate, ctx->gu, nullptr, 2 * F, OUT, f32, w.w_up, F))
         return false;
+      fold_norm(ctx, &p[2], ctx->x, w.ffn_norm);
       p[3] = Lin();  // N = 0: nothing to launch
       if (!make_lin(ctx, &p[4], M, d, F, hf, hl, F, w.w_down, ctx->x, nullptr, d, ACC, f32, nullptr, 0,
                     ctx->tc_zero ? ctx->qkv : nullptr, static_cast<long long>(M) * 3 * d))
         return false;
+      fold_swiglu(ctx, &p[4]);
     }
     return true;
   };
   ctx->pre.assign(5 * ctx->L, Lin());
   if (!layer_plans(ctx->pre, B * ctx->chunk)) return false;
   const void* dl_kv = eoff(ctx, const_cast<void*>(ctx->draft.wqkv), static_cast<size_t>(d) * d);
-  if (!make_lin(ctx, &ctx->pre_dkv, B * ctx->chunk, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, ACC, f32))
+  if (!make_lin(ctx, &ctx->pre_dkv, B * ctx->chunk, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, OUT, f32))
     return false;
+  fold_norm(ctx, &ctx->pre_dkv, ctx->hfin32, ctx->draft.attn_norm);
   if (same_batch) {
     ctx->plan_batch = B;
     ctx->plan_chunk = ctx->chunk;
@@ -1009,18 +1036,19 @@ bool build_plans(chimera_ctx* ctx, int B) {
   ctx->ar.assign(5 * ctx->L, Lin());
   if (!layer_plans(ctx->ver, B * N)) return false;
   if (!layer_plans(ctx->ar, B)) return false;
-  if (!make_lin(ctx, &ctx->ar_lm, B, V, d, ctx->hfin, ctx->hfin_lo, d, ctx->lm_head, ctx->logits, nullptr, V, ACC,
+  if (!make_lin(ctx, &ctx->ar_lm, B, V, d, ctx->hfin, ctx->hfin_lo, d, ctx->lm_head, ctx->logits, nullptr, V, OUT,
                 f32))
     return false;
   if (!make_lin(ctx, &ctx->ver_lm, B * N, V, d, ctx->hfin, ctx->hfin_lo, d, ctx->lm_head, ctx->logits, nullptr, V,
-                ACC, f32))
+                OUT, f32))
     return false;
   if (!make_lin(ctx, &ctx->pre_lm, B, V, d, ctx->headin, ctx->headin_lo, 2 * d, ctx->lm_head, ctx->logits, nullptr, V,
-                ACC, f32))
+                OUT, f32))
     return false;
-  if (!make_lin(ctx, &ctx->commit_kv, B * ctx->D1, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, ACC,
+  if (!make_lin(ctx, &ctx->commit_kv, B * ctx->D1, 2 * d, d, xn, xl, d, dl_kv, ctx->kvtmp, nullptr, 2 * d, OUT,
                 f32))
     return false;
+  fold_norm(ctx, &ctx->commit_kv, ctx->hsel, ctx->draft.attn_norm);
   // draft (M = B rows); the trigram input is a gather of bf16 embeddings: exact, no lo half
   // W2 stores h_tri (partials summed in a fixed order): the same trigram always gives
   // the same row, so a cached row equals a recomputed one bit for bit
@@ -1031,12 +1059,15 @@ bool build_plans(chimera_ctx* ctx, int B) {
                 f32, nullptr, 0, nullptr, 0, ctx->tc_skip))
     return false;
   const chimera_block_weights& w = ctx->draft;
-  if (!make_lin(ctx, &ctx->dqkv, B, 3 * d, d, xn, xl, d, w.wqkv, ctx->qkv, nullptr, 3 * d, ACC, f32)) return false;
+  if (!make_lin(ctx, &ctx->dqkv, B, 3 * d, d, xn, xl, d, w.wqkv, ctx->qkv, nullptr, 3 * d, OUT, f32)) return false;
+  fold_norm(ctx, &ctx->dqkv, ctx->dres, w.attn_norm);
   if (!make_lin(ctx, &ctx->dwo, B, d, d, ao, al, d, w.wo, ctx->dres, nullptr, d, ACC, f32)) return false;
-  if (!make_lin(ctx, &ctx->dgate, B, F, d, xn, xl, d, w.w_gate, ctx->gu, nullptr, 2 * F, ACC, f32, w.w_up, F))
+  if (!make_lin(ctx, &ctx->dgate, B, F, d, xn, xl, d, w.w_gate, ctx->gu, nullptr, 2 * F, OUT, f32, w.w_up, F))
     return false;
+  fold_norm(ctx, &ctx->dgate, ctx->dres, w.ffn_norm);
   ctx->dup = Lin();
   if (!make_lin(ctx, &ctx->ddown, B, d, F, hf, hl, F, w.w_down, ctx->dres, nullptr, d, ACC, f32)) return false;
+  fold_swiglu(ctx, &ctx->ddown);
   ctx->dhead.assign(ctx->K, Lin());
   // residual heads read [h_LLM_n ; h_full] (2d); heads without the residual h_full alone
   const bool no_resid = (ctx->draft_mode & 2) != 0;
@@ -1045,7 +1076,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
   const void* hx_lo = ctx->headin_lo ? (no_resid ? eoff(ctx, ctx->headin_lo, d) : ctx->headin_lo) : nullptr;
   for (int k = 0; k < ctx->K; ++k)
     if (!make_lin(ctx, &ctx->dhead[k], B, V, hk, hx, hx_lo, 2 * d, ctx->heads[k],
-                  ctx->hlog + static_cast<size_t>(k) * B * V, nullptr, V, ACC, f32))
+                  ctx->hlog + static_cast<size_t>(k) * B * V, nullptr, V, OUT, f32))
       return false;
   if (ctx->use_chain && !build_chains(ctx, B)) return false;
   ctx->plan_batch = B;
@@ -1535,7 +1566,7 @@ chimera_status chimera_prefill(chimera_ctx* ctx, int batch, const int32_t* token
                        ctx->att_splits_pre, 0));
     CK(run_final_norm(ctx, B * C, false));
     // draft-layer K/V of the chunk's H_LLM rows
-    CK(run_norm(ctx, ctx->hfin32, dl_norm, B * C, ctx->kvtmp, 2 * d));
+    if (!folds(ctx)) CK(run_norm(ctx, ctx->hfin32, dl_norm, B * C, ctx->kvtmp, 2 * d));
     CK(run_lin(ctx, ctx->pre_dkv));
     CK(run_rope(ctx, true, 0, ctx->kvtmp, 2 * d, -1, 0, d, C, ctx->d_valid, 0, 0, 0, nullptr));
     CK(launch_prefill_advance(ctx->dtype, ctx->hfin32, d, C, ctx->d_valid, ctx->d_last, ctx->d_n, ctx->headin,
