@@ -50,7 +50,7 @@ struct TcPairParams {
   int M, N;
   int halves, half_split; // 128-feature halves in all, and those taken from W
   int TT;                 // tokens per tile (<= 128)
-  int tok_tiles, feat_tiles, kblocks, stages;
+  int tok_tiles, feat_tiles, kblocks, b_stages;
   int width;              // pairs per group: token tiles that share the weight tiles in time
   uint32_t units;         // of a group: (round of width token tiles, feature tile, K block)
   int epi, out_f32, vec_red;

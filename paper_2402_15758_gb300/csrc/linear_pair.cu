@@ -3,7 +3,7 @@
 //
 //   Y[M][N] (epilogue)= (X + X_lo)[M][K] . W[N][K]^T,  fp32 accumulation.
 //
-// Past 128 rows a linear on hi + lo activations does so much tensor work per weight byte
+// Past 64 rows a linear on hi + lo activations does so much tensor work per weight byte
 // (4 M flops per 2 bytes) that it is bound by the tensor cores and by what feeds them:
 // shared-memory reads of the operands, L2 reads of the tiles.  Two SMs share a tile:
 //
@@ -14,8 +14,11 @@
 //     its own accumulator, added at the end.
 //
 // A stage of 128 K is 64 KB per CTA and 1024 tensor cycles (the traffic of a 256 x 256
-// tile of a plain GEMM); three are in flight.  Stages of 64 K (six in flight) were 12-19 %
-// slower: a weight request then takes 128 B of each row, half of what DRAM pages like.
+// tile of a plain GEMM); three of weights and three or more of tokens are in flight.
+// Stages of 64 K (six in flight) were 12-19 % slower: a weight request then takes 128 B of
+// each row, half of what DRAM pages like.  Two token tiles per weight stage (48 KB per 1024
+// cycles, both accumulators taken) won 3-5 % at 1024 rows and lost 2-14 % from 256 to 640
+// (more partial tiles to add at the end).
 //
 // Work split: stream-K over (feature tile, K block) units and groups of pairs.  The W
 // pairs of a group take the same units for W token tiles, so a weight tile is read by
@@ -32,10 +35,11 @@
 // 1.9e-6, 9.3e-6 for linear_tc.cu.
 //
 // Measured (GB300, EPI_RESID, against the kernel of linear_tc.cu on the same shape):
-// 256 rows: 22016 x 4096 77.5 -> 66.4 us (1.39 PFLOP/s), 4096 x 11008 41.7 -> 38.6,
-// 160 rows: 72.8 -> 54.5, 38.9 -> 30.8; 512 rows: 150.7 -> 116.2 (1.59), 76.7 -> 61.4.
-// With the loads left out (wrong results) 256 rows take 54.9 us: launch, ramp and tail are
-// about 8 us, the rest is the tensor rate.
+// 22016 x 4096: 72 rows 34.8 -> 31.9 us, 128 rows 41.1 -> 35.1, 256 rows 77.5 -> 60.6
+// (1.52 PFLOP/s), 512 rows 150.7 -> 108.7 (1.70);  4096 x 11008: 20.0 -> 18.8,
+// 23.8 -> 20.7, 41.7 -> 32.5, 76.7 -> 55.2.
+// With the loads left out (wrong results) 256 rows of 22016 x 4096 take 45.7 us, without
+// the weights' alone 47.8: what is left is the L2's feed of the SMs.
 //
 // Roles (576 threads per CTA): warp 0 issues the TMA loads of its CTA (both CTAs signal
 // the full barrier of CTA 0), warp 1 of CTA 0 issues the MMAs of the pair, warps 2..17
@@ -59,7 +63,8 @@ constexpr int BK = ATOM * BKA;
 constexpr int UK = 16;
 constexpr int A_ATOM = BM * ATOM * 2;
 constexpr int A_BYTES = A_ATOM * BKA;
-constexpr int MAX_STAGES = 8;
+constexpr int A_STAGES = 3;      // weight tiles in shared memory
+constexpr int MAX_B_STAGES = 8;  // token tiles
 constexpr int PIPE_SMEM = 200 * 1024;
 constexpr int EPI_WARPS = 16;   // four per TMEM lane quarter: a quarter of the tile's tokens each
 constexpr int THREADS = (2 + EPI_WARPS) * 32;
@@ -143,6 +148,345 @@ __device__ __forceinline__ uint32_t unit_begin(uint32_t c, uint32_t U, uint32_t 
 
 constexpr int G = 4;  // 8-token groups a warp holds: its quarter of the token tile
 
+struct Ctrl {  // at the start of the aligned dynamic shared memory
+  uint64_t full_a[A_STAGES], empty_a[A_STAGES], full_b[MAX_B_STAGES], empty_b[MAX_B_STAGES];
+  uint64_t tfull[2], tempty[2], drain;
+  uint32_t tmem;
+  int abort, last;
+};
+constexpr int CTRL_BYTES = 1024;
+static_assert(sizeof(Ctrl) <= CTRL_BYTES, "control block");
+__device__ __forceinline__ uint8_t* smem_base() {
+  extern __shared__ uint8_t smem_raw[];
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+}
+__device__ __forceinline__ int b_bytes_of(const TcPairParams& p) { return p.TT * BK * 2; }  // a token tile in shared memory
+
+// The units of this CTA's pair: W pairs side by side (a group) take the same units for W
+// token tiles.
+struct Work {
+  uint32_t KB, W, U, P, pair, grp, begin, end;
+  __device__ __forceinline__ explicit Work(const TcPairParams& p)
+      : KB(p.kblocks), W(p.width), U(p.units), P(gridDim.x / (2 * p.width)), pair(blockIdx.x / 2), grp(pair / W),
+        begin(unit_begin(grp, U, P)), end(unit_begin(grp + 1, U, P)) {}
+  // tile of unit u: feature tile and token tile
+  __device__ __forceinline__ int ft(const TcPairParams& p, uint32_t u) const {
+    return static_cast<int>(u / KB % p.feat_tiles);
+  }
+  __device__ __forceinline__ int tt(const TcPairParams& p, uint32_t u) const {
+    return static_cast<int>(u / KB / p.feat_tiles * W + pair % W);
+  }
+};
+
+// Each role derives what it needs by itself, and the epilogue is written so that nothing is
+// spilled at the 96 registers that 18 warps leave: shared memory takes almost all of L1, so
+// a spill goes to L2.  With values shared between the roles, the reductions and the other
+// epilogues in one kernel and 148 bytes of spills: 256 rows, 22016 x 4096 67.1 us (60.6),
+// 4096 x 11008 40.0 (32.5); 640 rows 141.9 (132.3) and 75.6 (67.8).
+__device__ __forceinline__ void produce(const TcPairParams& p, int lane, uint32_t rank) {
+  if (lane == 0) {
+    uint8_t* base = smem_base();
+    Ctrl* c = reinterpret_cast<Ctrl*>(base);
+    uint8_t* smem = base + CTRL_BYTES;
+    uint8_t* smem_b = smem + A_STAGES * A_BYTES;
+    const int b_bytes = b_bytes_of(p), b_atom = b_bytes / BKA;
+    const Work w(p);
+    volatile int* abort = &c->abort;
+    // ---------------- TMA producer (each CTA: its features, its rows of B) ----------------
+    const uint64_t pol_w = policy_evict_first();
+    uint32_t issued = 0, issued_par = 0;  // bits 0..: weight tiles, bits 8..: token tiles
+    const CUtensorMap* bmap = rank ? &p.tmB2 : &p.tmB;
+    int sa = 0, sb = 0;
+    uint32_t pa = 0, pb = 0;
+    auto load_a = [&](uint32_t u) {
+      const int half = w.ft(p, u) * 2 + static_cast<int>(rank), k = static_cast<int>(u % w.KB) * BK;
+      const bool second = half >= p.half_split;
+      const CUtensorMap* map = second ? &p.tmA2 : &p.tmA;
+      const int row = (second ? half - p.half_split : half) * BM;
+      const uint32_t bar = dsmem_addr(smem_u32(&c->full_a[sa]), 0);
+      if (!rank) mbar_arrive_expect_tx(&c->full_a[sa], static_cast<uint32_t>(2 * A_BYTES));
+#pragma unroll
+      for (int a = 0; a < BKA; ++a) {
+        if (p.tok_tiles == 1)  // read by this pair alone
+          tma_load_2d_pair_hint(smem + sa * A_BYTES + a * A_ATOM, map, k + a * ATOM, row, bar, pol_w);
+        else
+          tma_load_2d_pair(smem + sa * A_BYTES + a * A_ATOM, map, k + a * ATOM, row, bar);
+      }
+      issued |= 1u << sa;
+      issued_par = (issued_par & ~(1u << sa)) | (pa << sa);
+      if (++sa == A_STAGES) {
+        sa = 0;
+        pa ^= 1u;
+      }
+    };
+    auto load_b = [&](uint32_t u) {
+      const int row = w.tt(p, u) * p.TT, k = static_cast<int>(u % w.KB) * BK;
+      const uint32_t bar = dsmem_addr(smem_u32(&c->full_b[sb]), 0);
+      if (!rank) mbar_arrive_expect_tx(&c->full_b[sb], static_cast<uint32_t>(2 * b_bytes));
+#pragma unroll
+      for (int a = 0; a < BKA; ++a)
+        tma_load_2d_pair(smem_b + sb * b_bytes + a * b_atom, bmap, k + a * ATOM, row, bar);
+      issued |= 256u << sb;
+      issued_par = (issued_par & ~(256u << sb)) | (pb << (8 + sb));
+      if (++sb == p.b_stages) {
+        sb = 0;
+        pb ^= 1u;
+      }
+    };
+    // the weights do not depend on earlier kernels: the first two units' (as in
+    // linear_tc.cu) are requested before the dependency wait
+    uint32_t ua = w.begin;
+    for (; ua < min(w.begin + 2, w.end); ++ua) load_a(ua);
+    pdl_wait();
+    pdl_trigger();
+    bool ok = true;
+    for (uint32_t u = w.begin; ok && u < w.end && !*abort; ++u) {
+      if (u == ua) {
+        ok = mbar_wait(&c->empty_a[sa], pa ^ 1u, abort, p.wait_ns);
+        if (ok) load_a(ua++);
+      }
+      ok = ok && mbar_wait(&c->empty_b[sb], pb ^ 1u, abort, p.wait_ns);
+      if (ok) load_b(u);
+    }
+    // After a timeout copies may still be in flight, and a CTA must not end before its
+    // own have landed.  They signal CTA 0's barriers, which CTA 1 cannot wait on and
+    // which stay short of bytes when only one CTA requested a stage: CTA 0 waits for
+    // its stages within a limit, and both let 10 ms pass (a copy takes microseconds).
+    if (*abort) {
+      if (!rank)
+        for (int i = 0; i < 8 + p.b_stages; ++i)
+          if (issued >> i & 1u)
+            mbar_wait_plain(i < 8 ? &c->full_a[i] : &c->full_b[i - 8], issued_par >> i & 1u, 20000000ull);
+      for (const uint64_t t0 = global_timer_ns(); global_timer_ns() - t0 < 10000000ull;) {
+      }
+    }
+  } else {
+    pdl_wait();
+    pdl_trigger();
+  }
+}
+
+__device__ __forceinline__ void multiply(const TcPairParams& p, uint32_t rank) {
+  pdl_wait();
+  pdl_trigger();
+  __syncwarp();
+  if (!rank) {
+    uint8_t* base = smem_base();
+    Ctrl* c = reinterpret_cast<Ctrl*>(base);
+    uint8_t* smem = base + CTRL_BYTES;
+    uint8_t* smem_b = smem + A_STAGES * A_BYTES;
+    const int b_bytes = b_bytes_of(p), b_atom = b_bytes / BKA;
+    const Work w(p);
+    volatile int* abort = &c->abort;
+    const uint32_t tmem_base = c->tmem;
+    // ---------------- MMA issuer of the pair (the whole warp, one elected lane issues) ----------------
+    const uint32_t elected = elect_one();
+    const uint32_t n = 2 * p.TT;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
+    const uint64_t desc_a = sw128_desc(smem_u32(smem)), desc_b = sw128_desc(smem_u32(smem_b));
+    int sa = 0, sb = 0, buf = 0;
+    uint32_t pa = 0, pb = 0, aphase = 0;
+    bool ok = true;
+    for (uint32_t u = w.begin; ok && u < w.end;) {
+      const uint32_t tile_end = min(w.end, (u / w.KB + 1) * w.KB);
+      const uint32_t seg_end = min(tile_end, u + SEG_UNITS);
+      ok = mbar_wait_warp(&c->tempty[buf], aphase ^ 1u, abort, p.wait_ns);
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + buf * 256;
+      uint32_t acc = 0;
+      for (; ok && u < seg_end; ++u) {
+        ok = mbar_wait_warp(&c->full_a[sa], pa, abort, p.wait_ns) && mbar_wait_warp(&c->full_b[sb], pb, abort, p.wait_ns);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t da = desc_a + static_cast<uint64_t>((sa * A_BYTES) >> 4);
+        const uint64_t db = desc_b + static_cast<uint64_t>((sb * b_bytes) >> 4);
+#pragma unroll
+        for (int a = 0; a < BKA; ++a)
+#pragma unroll
+          for (int k = 0; k < ATOM / UK; ++k) {
+            tc_mma_bf16_pair(d_tmem, da + static_cast<uint64_t>((a * A_ATOM + k * 32) >> 4),
+                             db + static_cast<uint64_t>((a * b_atom + k * 32) >> 4), idesc, acc, elected);
+            acc = 1;
+          }
+        tc_commit_pair(&c->empty_a[sa], elected);
+        tc_commit_pair(&c->empty_b[sb], elected);
+        if (++sa == A_STAGES) {
+          sa = 0;
+          pa ^= 1u;
+        }
+        if (++sb == p.b_stages) {
+          sb = 0;
+          pb ^= 1u;
+        }
+      }
+      if (ok) tc_commit_pair(&c->tfull[buf], elected);
+      buf ^= 1;
+      if (buf == 0) aphase ^= 1u;
+    }
+    if (!ok) {  // every MMA issued so far must complete before tensor memory is released
+      tc_commit_pair(&c->drain, elected);
+      mbar_wait_plain(&c->drain, 0, 200000000ull);
+    }
+  }
+  __syncwarp();
+}
+
+template <bool RED>
+__device__ __forceinline__ void drain_tiles(const TcPairParams& p, int warp, int lane, uint32_t rank) {
+  pdl_wait();  // Y, the workspace and the counters are shared with earlier kernels
+  pdl_trigger();
+  if (p.zero) {  // this CTA's share (float4s) of a later linear's accumulator
+    const long long n4 = p.zero_floats / 4, per = (n4 + gridDim.x - 1) / gridDim.x, z0 = blockIdx.x * per;
+    float4* z = reinterpret_cast<float4*>(p.zero);
+    for (long long i = z0 + (threadIdx.x - 64); i < min(n4, z0 + per); i += EPI_WARPS * 32)
+      z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  uint8_t* base = smem_base();
+  Ctrl* c = reinterpret_cast<Ctrl*>(base);
+  const Work w(p);
+  volatile int* abort = &c->abort;
+  const uint32_t tmem_base = c->tmem;
+  const int q = warp & 3, th = (warp - 2) >> 2;
+  const int row = q * 32 + lane;
+  // this warp's 8-token groups: a quarter of the tile's
+  const int ng = p.TT / 8, per4 = (ng + 3) / 4;
+  const int g0 = min(ng, th * per4), gn = min(ng, g0 + per4) - g0;
+  const uint32_t tempty0 = dsmem_addr(smem_u32(&c->tempty[0]), 0);
+  float* sw = reinterpret_cast<float*>(base + CTRL_BYTES + A_STAGES * A_BYTES + p.b_stages * b_bytes_of(p)) +
+              (warp - 2) * 8 * RED_PITCH;  // this warp's transpose buffer
+  float acc[G][8];
+  int buf = 0;
+  uint32_t aphase = 0;
+  // 8 tokens (this warp's group `g`) x 32 features to the transpose buffer
+  auto stage_group = [&](int g) {
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+      if (i == g) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sw[j * RED_PITCH + lane] = acc[i][j];
+      }
+    __syncwarp();
+  };
+  bool ok = true;
+  for (uint32_t u = w.begin; u < w.end;) {
+    const uint32_t t = u / w.KB, tile_end = min(w.end, (t + 1) * w.KB);
+    const int half = w.ft(p, u) * 2 + static_cast<int>(rank), tt = w.tt(p, u);
+    const int f0 = half * BM + q * 32, m0 = tt * p.TT + g0 * 8;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
+    while (ok && u < tile_end) {
+      u = min(tile_end, u + SEG_UNITS);
+      ok = mbar_wait(&c->tfull[buf], aphase, abort, p.wait_ns);
+      ok = !bar_any(1, EPI_WARPS * 32, !ok);
+      tc_fence_after();
+      const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * 256 + g0 * 8;
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        if (ok && g < gn) {
+          uint32_t r[8];
+          uint32_t lo[8];
+          tmem_ld8(tbase + g * 8, r);
+          tmem_ld8(tbase + p.TT + g * 8, lo);
+          tmem_wait8x2(r, lo);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[g][j] += __uint_as_float(r[j]) + __uint_as_float(lo[j]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(tempty0 + buf * 8);
+      buf ^= 1;
+      if (buf == 0) aphase ^= 1u;
+    }
+    if (!ok) break;
+    if (RED) {  // float4 reductions
+#pragma unroll 1
+      for (int g = 0; g < gn; ++g) {
+        stage_group(g);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int j = h * 4 + (lane >> 3), k = (lane & 7) * 4, m = m0 + g * 8 + j;
+          if (m < p.M && f0 + k < p.N)
+            red_add_v4(static_cast<float*>(p.Y) + static_cast<size_t>(m) * p.ldy + f0 + k,
+                       *reinterpret_cast<const float4*>(sw + j * RED_PITCH + k));
+        }
+        __syncwarp();
+      }
+      continue;
+    }
+    // ---- this pair's part of tile t is complete ----
+    const int f = f0 + lane;
+    const uint32_t c_first = pair_of_unit(t * w.KB, w.U, w.P), c_last = pair_of_unit(t * w.KB + w.KB - 1, w.U, w.P);
+    auto store = [&](int m, float x) {
+      if (m >= p.M || f >= p.N) return;
+      if (p.epi == EPI_SILU) x = silu_f(x);
+      const size_t idx = static_cast<size_t>(m) * p.ldy + f;
+      if (p.out_f32)
+        static_cast<float*>(p.Y)[idx] = x;
+      else
+        store_act(static_cast<bf16*>(p.Y), static_cast<bf16*>(p.Y2), idx, x);
+    };
+    // slot of group c's partial of this token tile: [token][feature]
+    auto slot = [&](uint32_t c) {
+      const int first_slot = (unit_begin(c, w.U, w.P) / w.KB == t) ? 0 : 1;
+      return p.ws + static_cast<size_t>(2 * (2 * (c * w.W + w.pair % w.W) + rank) + first_slot) * BM * p.TT +
+             static_cast<size_t>(g0 * 8) * BM + row;
+    };
+    const bool parts = p.epi != EPI_RESID && c_first != c_last;
+    float* wsp = parts ? slot(w.grp) : nullptr;
+    int* counter = p.counters + 2 * (t * w.W + w.pair % w.W) + rank;
+#pragma unroll 1
+    for (int g = 0; g < gn; ++g) {
+      stage_group(g);
+#pragma unroll 1
+      for (int j = 0; j < 8; ++j) {
+        const float x = sw[j * RED_PITCH + lane];
+        const int m = m0 + g * 8 + j;
+        if (parts)
+          __stcg(wsp + (g * 8 + j) * BM, x);
+        else if (p.epi != EPI_RESID)
+          store(m, x);
+        else if (m < p.M && f < p.N)
+          red_add_f32(static_cast<float*>(p.Y) + static_cast<size_t>(m) * p.ldy + f, x);
+      }
+      __syncwarp();
+    }
+    if (parts) {  // the last pair to arrive sums the partials in pair order
+      __threadfence();
+      named_bar(1, EPI_WARPS * 32);
+      if (threadIdx.x == 64) c->last = atomicAdd(counter, 1) == static_cast<int>(c_last - c_first) ? 1 : 0;
+      named_bar(1, EPI_WARPS * 32);
+      if (c->last) {
+        __threadfence();
+#pragma unroll 1
+        for (int g = 0; g < gn; ++g) {
+          float v[8];
+          for (uint32_t c = c_first; c <= c_last; ++c) {
+            const float* src = slot(c) + g * 8 * BM;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float w = __ldcg(src + j * BM);
+              v[j] = c == c_first ? w : v[j] + w;
+            }
+          }
+#pragma unroll 1
+          for (int j = 0; j < 8; ++j) {
+            float x = v[0];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) x = j == i ? v[i] : x;
+            store(m0 + g * 8 + j, x);
+          }
+        }
+        if (threadIdx.x == 64) *counter = 0;
+      }
+      named_bar(1, EPI_WARPS * 32);
+    }
+  }
+}
+
+template <bool RED>
 __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
     tc_pair_kernel(const __grid_constant__ TcPairParams p) {
   if (p.skip) {  // written by the previous kernel; the same value in both CTAs
@@ -152,37 +496,27 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
       return;
     }
   }
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~static_cast<uintptr_t>(1023));
-  const int b_atom = p.TT * ATOM * 2;
-  const int stage_bytes = A_BYTES + b_atom * BKA;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes);
-  uint64_t* empty = full + MAX_STAGES;
-  uint64_t* tfull = empty + MAX_STAGES;
-  uint64_t* tempty = tfull + 2;
-  uint64_t* drain = tempty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-  int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
-  int* s_last = s_abort + 1;
-  float* s_red = reinterpret_cast<float*>(smem + p.stages * stage_bytes + 1024);  // [EPI_WARPS][8][RED_PITCH]
-
+  Ctrl* c = reinterpret_cast<Ctrl*>(smem_base());
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < A_STAGES; ++s) {
+      mbar_init(&c->full_a[s], 1);
+      mbar_init(&c->empty_a[s], 1);
+    }
+    for (int s = 0; s < p.b_stages; ++s) {
+      mbar_init(&c->full_b[s], 1);
+      mbar_init(&c->empty_b[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], 2 * EPI_WARPS);
+      mbar_init(&c->tfull[b], 1);
+      mbar_init(&c->tempty[b], 2 * EPI_WARPS);
     }
-    mbar_init(drain, 1);
-    *s_abort = 0;
-    *s_last = 0;
+    mbar_init(&c->drain, 1);
+    c->abort = 0;
+    c->last = 0;
     mbar_fence_init();
   }
   if (warp == 0 && lane == 0) {
@@ -192,7 +526,7 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
     prefetch_tensormap(&p.tmB2);
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&c->tmem)), "r"(512)
                  : "memory");
     __syncwarp();
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -202,273 +536,12 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
   __syncwarp();
   cluster_sync();  // the peer's barriers and tensor memory are ready
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
-  // W pairs side by side (a group) take the same units for W token tiles
-  const uint32_t KB = p.kblocks, W = p.width;
-  const uint32_t U = p.units, P = gridDim.x / (2 * W);
-  const uint32_t pair = blockIdx.x / 2, grp = pair / W;
-  const uint32_t u_begin = unit_begin(grp, U, P), u_end = unit_begin(grp + 1, U, P);
-  // tile of unit u: feature tile and token tile
-  auto ft_of = [&](uint32_t u) { return static_cast<int>(u / KB % p.feat_tiles); };
-  auto tt_of = [&](uint32_t u) { return static_cast<int>(u / KB / p.feat_tiles * W + pair % W); };
-  volatile int* abort = s_abort;
-
-  if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (each CTA: its features, its rows of B) ----------------
-      const uint64_t pol_w = policy_evict_first();
-      uint32_t issued_mask = 0, issued_par = 0;
-      const CUtensorMap* bmap = rank ? &p.tmB2 : &p.tmB;
-      auto load_a = [&](uint32_t u, int s) {
-        const int half = ft_of(u) * 2 + static_cast<int>(rank), k = static_cast<int>(u % KB) * BK;
-        const bool second = half >= p.half_split;
-        const CUtensorMap* map = second ? &p.tmA2 : &p.tmA;
-        const int row = (second ? half - p.half_split : half) * BM;
-        const uint32_t bar = dsmem_addr(smem_u32(&full[s]), 0);
-#pragma unroll
-        for (int a = 0; a < BKA; ++a) {
-          if (p.tok_tiles == 1)  // read by this pair alone
-            tma_load_2d_pair_hint(smem + s * stage_bytes + a * A_ATOM, map, k + a * ATOM, row, bar, pol_w);
-          else
-            tma_load_2d_pair(smem + s * stage_bytes + a * A_ATOM, map, k + a * ATOM, row, bar);
-        }
-      };
-      auto load_b = [&](uint32_t u, int s) {
-        const int row = tt_of(u) * p.TT, k = static_cast<int>(u % KB) * BK;
-        const uint32_t bar = dsmem_addr(smem_u32(&full[s]), 0);
-#pragma unroll
-        for (int a = 0; a < BKA; ++a)
-          tma_load_2d_pair(smem + s * stage_bytes + A_BYTES + a * b_atom, bmap, k + a * ATOM, row, bar);
-      };
-      // the weights do not depend on earlier kernels: the first two stages' (as in
-      // linear_tc.cu) are requested before the dependency wait
-      const uint32_t npre = min(2u, u_end - u_begin);
-      for (uint32_t i = 0; i < npre; ++i) {
-        if (!rank) mbar_arrive_expect_tx(&full[i], static_cast<uint32_t>(2 * stage_bytes));
-        load_a(u_begin + i, i);
-        issued_mask |= 1u << i;
-      }
-      pdl_wait();
-      pdl_trigger();
-      for (uint32_t i = 0; i < npre; ++i) load_b(u_begin + i, i);
-      int stage = static_cast<int>(npre % p.stages);
-      uint32_t phase = (npre == static_cast<uint32_t>(p.stages)) ? 1u : 0u;
-      for (uint32_t u = u_begin + npre; u < u_end && !*abort; ++u) {
-        if (!mbar_wait(&empty[stage], phase ^ 1u, abort, p.wait_ns)) break;
-        if (!rank) mbar_arrive_expect_tx(&full[stage], static_cast<uint32_t>(2 * stage_bytes));
-        load_a(u, stage);
-        load_b(u, stage);
-        issued_mask |= 1u << stage;
-        issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
-        if (++stage == p.stages) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
-      // After a timeout copies may still be in flight, and a CTA must not end before its
-      // own have landed.  They signal CTA 0's barriers, which CTA 1 cannot wait on and
-      // which stay short of bytes when only one CTA requested a stage: CTA 0 waits for
-      // its stages within a limit, and both let 10 ms pass (a copy takes microseconds).
-      if (*abort) {
-        if (!rank)
-          for (int s = 0; s < p.stages; ++s)
-            if (issued_mask >> s & 1u) mbar_wait_plain(&full[s], issued_par >> s & 1u, 20000000ull);
-        for (const uint64_t t0 = global_timer_ns(); global_timer_ns() - t0 < 10000000ull;) {
-        }
-      }
-    } else {
-      pdl_wait();
-      pdl_trigger();
-    }
-  } else if (warp == 1) {
-    pdl_wait();
-    pdl_trigger();
-    __syncwarp();
-    if (!rank) {
-      // ---------------- MMA issuer of the pair (the whole warp, one elected lane issues) ----------------
-      const uint32_t elected = elect_one();
-      const uint32_t n = 2 * p.TT;
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
-      const uint64_t desc0 = sw128_desc(smem_u32(smem));
-      int stage = 0, buf = 0;
-      uint32_t phase = 0, aphase = 0;
-      bool ok = true;
-      for (uint32_t u = u_begin; ok && u < u_end;) {
-        const uint32_t tile_end = min(u_end, (u / KB + 1) * KB);
-        const uint32_t seg_end = min(tile_end, u + SEG_UNITS);
-        ok = mbar_wait_warp(&tempty[buf], aphase ^ 1u, abort, p.wait_ns);
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * 256;
-        uint32_t acc = 0;
-        for (; ok && u < seg_end; ++u) {
-          ok = mbar_wait_warp(&full[stage], phase, abort, p.wait_ns);
-          if (!ok) break;
-          tc_fence_after();
-          const uint64_t da = desc0 + static_cast<uint64_t>((stage * stage_bytes) >> 4);
-          const uint64_t db = da + static_cast<uint64_t>(A_BYTES >> 4);
-#pragma unroll
-          for (int a = 0; a < BKA; ++a)
-#pragma unroll
-            for (int k = 0; k < ATOM / UK; ++k) {
-              tc_mma_bf16_pair(d_tmem, da + static_cast<uint64_t>((a * A_ATOM + k * 32) >> 4),
-                               db + static_cast<uint64_t>((a * b_atom + k * 32) >> 4), idesc, acc, elected);
-              acc = 1;
-            }
-          tc_commit_pair(&empty[stage], elected);
-          if (++stage == p.stages) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-        if (ok) tc_commit_pair(&tfull[buf], elected);
-        buf ^= 1;
-        if (buf == 0) aphase ^= 1u;
-      }
-      if (!ok) {  // every MMA issued so far must complete before tensor memory is released
-        tc_commit_pair(drain, elected);
-        mbar_wait_plain(drain, 0, 200000000ull);
-      }
-    }
-    __syncwarp();
-  } else {
-    // ---------------- epilogue ----------------
-    pdl_wait();  // Y, the workspace and the counters are shared with earlier kernels
-    pdl_trigger();
-    if (p.zero) {  // this CTA's share (float4s) of a later linear's accumulator
-      const long long n4 = p.zero_floats / 4, per = (n4 + gridDim.x - 1) / gridDim.x, z0 = blockIdx.x * per;
-      float4* z = reinterpret_cast<float4*>(p.zero);
-      for (long long i = z0 + (threadIdx.x - 64); i < min(n4, z0 + per); i += EPI_WARPS * 32)
-        z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const int q = warp & 3, th = (warp - 2) >> 2;
-    const int row = q * 32 + lane;
-    // this warp's 8-token groups: a quarter of the tile's
-    const int ng = p.TT / 8, per4 = (ng + 3) / 4;
-    const int g0 = min(ng, th * per4), gn = min(ng, g0 + per4) - g0;
-    const uint32_t tempty0 = dsmem_addr(smem_u32(&tempty[0]), 0);
-    float* sw = s_red + (warp - 2) * 8 * RED_PITCH;
-    float acc[G][8];
-    int buf = 0;
-    uint32_t aphase = 0;
-    for (uint32_t u = u_begin; u < u_end;) {
-      const uint32_t t = u / KB;
-      const uint32_t tile_end = min(u_end, (t + 1) * KB);
-      const uint32_t seg_end = min(tile_end, u + SEG_UNITS);
-      const bool first = u == u_begin || u == t * KB, last = seg_end == tile_end;
-      u = seg_end;
-      const bool ok = mbar_wait(&tfull[buf], aphase, abort, p.wait_ns);
-      if (bar_any(1, EPI_WARPS * 32, !ok)) break;
-      tc_fence_after();
-      const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * 256 + g0 * 8;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        if (g < gn) {
-          uint32_t r[8];
-          uint32_t lo[8];
-          tmem_ld8(tbase + g * 8, r);
-          tmem_ld8(tbase + p.TT + g * 8, lo);
-          tmem_wait8x2(r, lo);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float v = __uint_as_float(r[j]) + __uint_as_float(lo[j]);
-            acc[g][j] = first ? v : acc[g][j] + v;
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty0 + buf * 8);
-      buf ^= 1;
-      if (buf == 0) aphase ^= 1u;
-      if (!last) continue;
-      // ---- this pair's part of tile t is complete ----
-      const int half = ft_of(t * KB) * 2 + static_cast<int>(rank), tt = tt_of(t * KB);
-      const int f0 = half * BM + q * 32, f = f0 + lane;
-      const int m0 = tt * p.TT + g0 * 8;
-      const uint32_t c_first = pair_of_unit(t * KB, U, P), c_last = pair_of_unit(t * KB + KB - 1, U, P);
-      auto store = [&](int m, float x) {
-        if (m >= p.M || f >= p.N) return;
-        if (p.epi == EPI_SILU) x = silu_f(x);
-        const size_t idx = static_cast<size_t>(m) * p.ldy + f;
-        if (p.out_f32)
-          static_cast<float*>(p.Y)[idx] = x;
-        else
-          store_act(static_cast<bf16*>(p.Y), static_cast<bf16*>(p.Y2), idx, x);
-      };
-      // slot of group c's partial of this token tile: [token][feature]
-      auto slot = [&](uint32_t c) {
-        const int first_slot = (unit_begin(c, U, P) / KB == t) ? 0 : 1;
-        return p.ws + static_cast<size_t>(2 * (2 * (c * W + pair % W) + rank) + first_slot) * BM * p.TT + static_cast<size_t>(g0 * 8) * BM + row;
-      };
-      const bool parts = p.epi != EPI_RESID && c_first != c_last;
-      float* wsp = parts ? slot(grp) : nullptr;
-      int* counter = p.counters + 2 * (t * W + pair % W) + rank;
-#pragma unroll 1
-      for (int g = 0; g < gn; ++g) {
-        // 8 tokens x 32 features through shared memory
-#pragma unroll
-        for (int gg = 0; gg < G; ++gg)
-          if (gg == g) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sw[j * RED_PITCH + lane] = acc[gg][j];
-          }
-        __syncwarp();
-        if (p.vec_red) {  // float4 reductions
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int c = i * 4 + (lane >> 3), k = (lane & 7) * 4, m = m0 + g * 8 + c;
-            if (m < p.M && f0 + k < p.N)
-              red_add_v4(static_cast<float*>(p.Y) + static_cast<size_t>(m) * p.ldy + f0 + k,
-                         *reinterpret_cast<const float4*>(sw + c * RED_PITCH + k));
-          }
-        } else {
-#pragma unroll 1
-          for (int j = 0; j < 8; ++j) {
-            const float x = sw[j * RED_PITCH + lane];
-            const int m = m0 + g * 8 + j;
-            if (parts)
-              __stcg(wsp + (g * 8 + j) * BM, x);
-            else if (p.epi != EPI_RESID)
-              store(m, x);
-            else if (m < p.M && f < p.N)
-              red_add_f32(static_cast<float*>(p.Y) + static_cast<size_t>(m) * p.ldy + f, x);
-          }
-        }
-        __syncwarp();
-      }
-      if (parts) {  // the last pair to arrive sums the partials in pair order
-        __threadfence();
-        named_bar(1, EPI_WARPS * 32);
-        if (threadIdx.x == 64) *s_last = atomicAdd(counter, 1) == static_cast<int>(c_last - c_first) ? 1 : 0;
-        named_bar(1, EPI_WARPS * 32);
-        if (*s_last) {
-          __threadfence();
-#pragma unroll 1
-          for (int g = 0; g < gn; ++g) {
-            float v[8];
-            for (uint32_t c = c_first; c <= c_last; ++c) {
-              const float* src = slot(c) + g * 8 * BM;
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float w = __ldcg(src + j * BM);
-                v[j] = c == c_first ? w : v[j] + w;
-              }
-            }
-#pragma unroll 1
-            for (int j = 0; j < 8; ++j) {
-              float x = v[0];
-#pragma unroll
-              for (int i = 1; i < 8; ++i) x = j == i ? v[i] : x;
-              store(m0 + g * 8 + j, x);
-            }
-          }
-          if (threadIdx.x == 64) *counter = 0;
-        }
-        named_bar(1, EPI_WARPS * 32);
-      }
-    }
-  }
+  if (warp == 0)
+    produce(p, lane, rank);
+  else if (warp == 1)
+    multiply(p, rank);
+  else
+    drain_tiles<RED>(p, warp, lane, rank);
 
   tc_fence_before();
   __syncthreads();
@@ -476,9 +549,9 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
   cluster_sync();  // both CTAs are done with each other's shared and tensor memory
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(c->tmem), "r"(512) : "memory");
   }
-  if (threadIdx.x == 0 && *abort) atomicOr(p.err, ERR_TIMEOUT);
+  if (threadIdx.x == 0 && *const_cast<volatile int*>(&c->abort)) atomicOr(p.err, ERR_TIMEOUT);
 }
 
 constexpr int MAX_DEVICES = 64;
@@ -499,6 +572,7 @@ int tc_pair_plan(TcPairPlan* plan, int M, int N1, int N2, int K, const void* X, 
   // zeros): without a second weight every half, that one too, belongs to W's tensor map
   p.half_split = W2 ? N1 / BM : p.halves + 1;
   // token tiles of equal height, at most 128; the pair's MMA takes N = 2 TT in steps of 32
+  p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && p.N % 4 == 0) ? 1 : 0;
   p.tok_tiles = (M + 127) / 128;
   p.TT = ((M + p.tok_tiles - 1) / p.tok_tiles + 15) / 16 * 16;
   p.kblocks = (K + BK - 1) / BK;
@@ -508,19 +582,21 @@ int tc_pair_plan(TcPairPlan* plan, int M, int N1, int N2, int K, const void* X, 
   p.feat_tiles = (p.halves + 1) / 2;
   const int groups = tc_num_sms() / 2 / p.width;
   const long long units = static_cast<long long>(rounds) * p.feat_tiles * p.kblocks;
-  // A pair with few stages spends its time on the ramp and on adding its part of a tile:
-  // 256 x 4096 x 4096 (13.5 stages) 20.9 us here, 19.6 in linear_tc.cu; 160 rows equal.
-  if (units < 14ll * groups) return -1;
+  // A pair with little work spends its time on the ramp and on adding its part of a tile.
+  // The line lies at 1000 stage-tokens per pair: 862 (256 rows, 2048 x 4096) 12.5 us here
+  // and in linear_tc.cu, 539 (160 rows, same) 10.5 and 9.7, 808 (80 rows, 6144 x 4096) 13.9
+  // and 13.5; 1078 (160 rows, 4096 x 4096) 14.9 and 15.8, 1132 (112 rows, 6144 x 4096) 15.1
+  // and 15.5, 1724 (256 rows, 4096 x 4096) 17.1 and 19.2.
+  if (units * p.TT < 1000ll * groups) return -1;
   if (2ll * rounds * p.width * p.feat_tiles > MAX_TILES || groups < 1 || units * (groups + 1) >= (1ll << 32)) return -1;
   p.units = static_cast<uint32_t>(units);
-  const int stage_bytes = A_BYTES + p.TT * BK * 2;
-  p.stages = std::min(MAX_STAGES, PIPE_SMEM / stage_bytes);
+  const int b_bytes = p.TT * BK * 2;
+  p.b_stages = std::min(MAX_B_STAGES, (PIPE_SMEM - A_STAGES * A_BYTES) / b_bytes);
   p.epi = epi;
   p.out_f32 = out_f32;
   p.Y = Y;
   p.Y2 = out_f32 ? nullptr : Y_lo;
   p.ldy = ldy;
-  p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && p.N % 4 == 0) ? 1 : 0;
   p.ws = ws;
   p.counters = counters;
   p.err = err;
@@ -528,7 +604,7 @@ int tc_pair_plan(TcPairPlan* plan, int M, int N1, int N2, int K, const void* X, 
   p.zero = zero;
   p.zero_floats = zero ? zero_floats : 0;
   plan->grid = 2 * p.width * static_cast<int>(std::min<long long>(units, groups));
-  plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + EPI_WARPS * 8 * RED_PITCH * sizeof(float);
+  plan->smem = 1024 + CTRL_BYTES + A_STAGES * A_BYTES + static_cast<size_t>(p.b_stages) * b_bytes + EPI_WARPS * 8 * RED_PITCH * sizeof(float);
   if (encode_2d_bf16(&p.tmA, W, K, N1, K, ATOM, BM) != 0) return -2;
   if (W2 && encode_2d_bf16(&p.tmA2, W2, K, N2, K, ATOM, BM) != 0) return -2;
   if (encode_2d_bf16(&p.tmB, X, K, M, ldx, ATOM, p.TT) != 0) return -2;
@@ -544,12 +620,14 @@ cudaError_t tc_pair_launch(const TcPairPlan& plan, cudaStream_t s) {
   {
     std::lock_guard<std::mutex> lk(g_pair_mu);
     if (!g_pair_attr[dev]) {
-      e = cudaFuncSetAttribute(tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e != cudaSuccess) return e;
+      for (auto k : {tc_pair_kernel<false>, tc_pair_kernel<true>}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+      }
       g_pair_attr[dev] = true;
     }
   }
-  launch_pdl(tc_pair_kernel, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
+  launch_pdl(plan.p.vec_red ? tc_pair_kernel<true> : tc_pair_kernel<false>, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
   return cudaGetLastError();
 }
 

@@ -61,11 +61,11 @@ constexpr int CTAS_PER_SM = CHIMERA_LIN_CTAS_PER_SM;
 constexpr int PIPE_SMEM = CHIMERA_LIN_PIPE_KB * 1024;
 constexpr int MAX_BN = 256;
 constexpr int MAX_TILES = 8192;
-// Split activations of more than PAIR_ROWS rows go to linear_pair.cu.  Up to 128 rows this
-// kernel reads the weights once as well and starts faster (128 rows, 12288 x 4096: 26.1 us
-// here, 27.9 there); past 128 it would read them once per token tile (136 rows: 41.5, 33.9).
+// Split activations of more than PAIR_ROWS rows go to linear_pair.cu when there is enough
+// work per pair.  12288 x 4096, 22016 x 4096, 4096 x 11008 at 64 rows: 18.0, 29.1, 16.6 us
+// here, 20.6, 31.3, 18.4 there; at 65 rows (80 of a tile) 21.6, 34.7, 20.1 and 20.8, 31.8, 18.8.
 // One-term activations stay here: a token tile is 256 rows, its work half of a split's.
-constexpr int PAIR_ROWS = 128;
+constexpr int PAIR_ROWS = 64;
 
 
 // Stream-K partition in 32-bit arithmetic (the host checks units * grid < 2^32).

@@ -78,10 +78,11 @@ def test_linear_bf16_split_operand(M, N, K):
     assert _rel_rows(Y.cpu().numpy(), ref) > 1e-4
 
 
-# the CTA-pair kernel: split activations of more than 128 rows with at least 14 stages per
-# pair.  Ragged token tiles (2 of 80 rows, 3 of 96, 9 in two rounds of 5), an odd number of
-# 128-feature halves, columns that are no multiple of 4, a ragged last K block
-@pytest.mark.parametrize("M,N,K", [(129, 4224, 4096), (256, 2050, 8000), (257, 1000, 12296), (640, 1536, 5000),
+# the CTA-pair kernel: split activations of more than 64 rows with at least 1000 stages x
+# tokens per pair.  Ragged token tiles (1 of 80 and of 112 rows, 2 of 80, 3 of 96, 9 in two
+# rounds of 5), an odd number of 128-feature halves, columns that are no multiple of 4, a
+# ragged last K block
+@pytest.mark.parametrize("M,N,K", [(65, 8200, 4096), (100, 6001, 4104), (129, 4224, 4096), (256, 2050, 8000), (257, 1000, 12296), (640, 1536, 5000),
                                    (1100, 1024, 3400)])
 @pytest.mark.parametrize("epi,out_f32", [(0, True), (1, False), (2, True)])
 def test_linear_pair_kernel(M, N, K, epi, out_f32):
