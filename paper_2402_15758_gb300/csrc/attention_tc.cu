@@ -23,19 +23,26 @@
 // running max and sum, and O accumulator, and nothing passes between them until the end.
 //
 // What bounds it (GB300, split planes, 4 splits of 32 heads): at a 16384-row context the K
-// and V stream (91.5 us, 5.9 TB/s; 75 us with the loads left out), at a 1000-row one the
-// latency of the prologue and of the merge (15.5 us, of which about 9 do not depend on
-// the context).  Before: 128.4 and 18.1 us, bound by the MMA issue: one lane moved the
-// operands of 36 small MMAs a tile to uniform registers (54 cycles each).  Also measured,
-// at 16384 rows: an L2 prefetch three tiles ahead of the rings 108.9 us against 95.8
+// and V stream (85.2 us, 6.3 TB/s), at a 1000-row one the latency of the prologue and of the
+// merge (64 queries 13.9 us, of which about 9 do not depend on the context).
+//
+// A tile of K or V takes 1.4-1.7 us to arrive under load and holds its slot for 0.5 us more
+// while the tensor cores read it, so the bytes in flight decide: K and V share one ring of
+// five 32 KB slots, filled in the order of use, which takes all of shared memory, and each
+// product has a warp of its own that waits for nothing but its operands.  With two slots
+// for K, two for V and one warp polling for both products: 90.2 us and 14.5, eight ragged
+// sequences of 32-node trees 104.2 us (98.9), one query over 512 rows 10.1 (9.5), plain
+// planes at 16384 rows 73.3 (63.9).  Before the two streams, with one lane issuing the MMAs
+// (54 cycles each, operands moved to uniform registers): 128.4 and 18.1 us.  Also measured,
+// at 16384 rows: an L2 prefetch three tiles ahead of the ring 108.9 us against 95.8
 // without; QK products of 32 keys, which let a box keep a page's 16 rows together, 95.8
 // against 91.5.
 //
 // Warps: 0..7 softmax + epilogue (warp w: stream w / 4, tensor-memory lanes 32 (w % 4)..,
 // rows 16 (w % 4) .. + 15; a warp whose rows are all past nq only keeps the barriers
-// going), 8 loads the KV tiles (TMA copies of 16-row page boxes into two-stage rings for
-// K and for V, 128-byte swizzle applied by the copy engine), 9 issues the MMAs and owns
-// the tensor-memory allocation.
+// going), 8 loads the KV tiles (TMA copies of 16-row page boxes, 128-byte swizzle applied
+// by the copy engine), 9 issues the QK products, 10 the PV products (and owns the
+// tensor-memory allocation).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -51,15 +58,14 @@ namespace {
 constexpr int HD = 128;
 constexpr int KT = 64;                      // keys per tile
 constexpr int NQ = 64;                      // query rows (UMMA M)
-constexpr int SOFT_WARPS = 8, LOAD_WARPS = 1;  // softmax: warps w and w + 4 share rows, w / 4 = tile parity
+constexpr int SOFT_WARPS = 8;               // softmax: warps w and w + 4 share rows, w / 4 = tile parity
 constexpr int STREAM_WARPS = SOFT_WARPS / 2;
-constexpr int THREADS = (SOFT_WARPS + LOAD_WARPS + 1) * 32;
-constexpr int MMA_WARP = SOFT_WARPS + LOAD_WARPS;
+constexpr int LOAD_WARP = SOFT_WARPS, QK_WARP = LOAD_WARP + 1, PV_WARP = QK_WARP + 1;
+constexpr int THREADS = (PV_WARP + 1) * 32;
 constexpr int ATOM_ROWS64 = 64 * 128;       // bytes of one 64-row x 128-byte swizzle atom column
 constexpr int GROUP = 8 * 128;              // 8 rows x 64 dims: one swizzle atom
 constexpr int TILE64 = 2 * ATOM_ROWS64;     // 64 rows x 128 bf16 (two atoms): 16 KB
-constexpr int STAGES = 2;
-constexpr int PAGE_CACHE = 1024;
+constexpr int PAGE_CACHE = 448;
 constexpr float RESCALE_LOG2 = 11.5f;        // raise the running max when it grows by > 2^11.5 (~e^8)
 constexpr uint32_t TMEM_COLS = 512;          // S[2] (64 cols each), O[2] (128 cols each)
 constexpr uint32_t O_COL = 128;
@@ -67,7 +73,7 @@ constexpr int MAX_PARTS = 16;                // partials of a row: one or two pe
 constexpr int MANY_NQ = 32;                  // more query rows than this take the MANY variant
 constexpr int PREC = HD + 4;                 // partial record (o[128], m, l, pad)
 constexpr int PART_FLOATS = (2 * MANY_NQ + 16) * PREC;  // the partial records of a CTA (<= NQ + 14 rows)
-constexpr int TILE_BYTES = 192 * 1024;       // Q, P, K and V tiles (with plain planes: and 64 KB of staging)
+constexpr int TILE_BYTES = 224 * 1024;       // Q, P, K and V tiles (with plain planes: and 64 KB of staging)
 static_assert((3 * PART_FLOATS + NQ * MAX_PARTS) * 4 <= TILE_BYTES, "partials and merge weights fit over the tiles");
 
 // Byte offset of 16-byte chunk c (0..7) of row r inside a 128-byte-swizzled atom column.
@@ -169,14 +175,15 @@ __device__ __forceinline__ void split4(float4 v, uint2& hi, uint2& lo) {
 // MANY: more than MANY_NQ query rows.  Their rows and the local tile's are staged through
 // shared memory, and a CTA merges its two streams before it sends them; with fewer rows
 // each of these steps adds more latency than it saves (one query 9.9 us without, 10.6
-// with them; 64 queries 15.7 and 14.5), and both paths in one kernel cost each other
+// with them; 64 queries 15.7 and 14.5; two-slot rings), and both paths in one kernel cost each other
 // (64 queries 15.3).
 template <bool SPLIT, bool MANY>
 __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_constant__ TcArgs args) {
   const AttnParams& p = args.p;
   constexpr int NP = SPLIT ? 4 : 2;
   constexpr int KP = NP / 2;                 // planes of K (and of V): hi (, lo)
-  constexpr int HALF_BYTES = KP * TILE64;   // one stage of K or of V:
+  constexpr int SLOTS = SPLIT ? 5 : 6;       // ring of K and V tiles
+  constexpr int HALF_BYTES = KP * TILE64;   // one slot, a tile of K or of V:
   // [page][8-row group][plane][dim half][8 rows][128 B]: one box per page, and the groups of
   // a plane and dim half lie at one stride (ROW_STRIDE) over the whole tile, as the
   // descriptors need
@@ -188,24 +195,22 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   uint8_t* q_hi = smem;                     // 64 x 128 (two atoms)
   uint8_t* q_lo = q_hi + TILE64;
   uint8_t* p_buf = q_lo + TILE64;           // [2 buffers][hi, lo] 64 x 64 (one atom each, 8 KB)
-  uint8_t* kbuf = p_buf + 4 * (NQ * 128);   // [STAGES][KP planes] 64 keys x 128 dims
-  uint8_t* vbuf = kbuf + STAGES * HALF_BYTES;
+  uint8_t* ring = p_buf + 4 * (NQ * 128);   // [SLOTS][KP planes] 64 keys x 128 dims
   // fp32 rows of the projections on their way into the tiles: q, and the local tile's k and v
   float* q_st = reinterpret_cast<float*>(p_buf);
-  float* k_st = reinterpret_cast<float*>(SPLIT ? kbuf + HALF_BYTES : vbuf + STAGES * HALF_BYTES);
-  float* v_st = reinterpret_cast<float*>(SPLIT ? vbuf + HALF_BYTES : vbuf + STAGES * HALF_BYTES + 2 * TILE64);
+  float* k_st = reinterpret_cast<float*>(ring + (SPLIT ? 3 : SLOTS) * HALF_BYTES);
+  float* v_st = k_st + NQ * HD;
+  static_assert(SPLIT || (SLOTS * HALF_BYTES + 8 * TILE64 <= TILE_BYTES), "staging behind the ring");
   float* part = reinterpret_cast<float*>(smem);  // partial records, over the tiles after the loop
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + TILE_BYTES);
-  uint64_t* k_full = bars;           // [2] count 1 + transaction bytes (TMA)
-  uint64_t* v_full = bars + 2;       // [2] count 1 + transaction bytes (TMA)
-  uint64_t* k_empty = bars + 4;      // [2] tcgen05.commit after QK
-  uint64_t* v_empty = bars + 6;      // [2] tcgen05.commit after PV
-  uint64_t* s_full = bars + 8;       // [2] tcgen05.commit
-  uint64_t* s_free = bars + 10;      // [2] count 4 (the stream's softmax warps)
-  uint64_t* p_full = bars + 12;      // [2] count 4
-  uint64_t* pv_done = bars + 14;     // [2] tcgen05.commit
-  uint64_t* o_done = bars + 16;      // tcgen05.commit
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
+  uint64_t* full = bars;             // [SLOTS] count 1 + transaction bytes (TMA)
+  uint64_t* empty = bars + 6;        // [SLOTS] tcgen05.commit after the product
+  uint64_t* s_full = bars + 12;      // [2] tcgen05.commit
+  uint64_t* s_free = bars + 14;      // [2] count 4 (the stream's softmax warps)
+  uint64_t* p_full = bars + 16;      // [2] count 4
+  uint64_t* pv_done = bars + 18;     // [2] tcgen05.commit
+  uint64_t* o_done = bars + 20;      // count 2: tcgen05.commit of the QK and of the PV warp
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 21);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_pages = s_abort + 2;        // [PAGE_CACHE]
   int* s_lpages = s_pages + PAGE_CACHE;  // [8] pages of the local rows
@@ -217,21 +222,21 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   bf16* pool = static_cast<bf16*>(const_cast<void*>(p.pool)) + static_cast<size_t>(p.layer) * p.pool_layer_stride;
 
   if (threadIdx.x == 0) {
+    for (int i = 0; i < SLOTS; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&k_full[i], 1);
-      mbar_init(&v_full[i], 1);
-      mbar_init(&k_empty[i], 1);
-      mbar_init(&v_empty[i], 1);
       mbar_init(&s_full[i], 1);
       mbar_init(&s_free[i], STREAM_WARPS);
       mbar_init(&p_full[i], STREAM_WARPS);
       mbar_init(&pv_done[i], 1);
     }
-    mbar_init(o_done, 1);
+    mbar_init(o_done, 2);
     *s_abort = 0;
     mbar_fence_init();
   }
-  if (warp == MMA_WARP) tmem_alloc(tmem_slot, TMEM_COLS);
+  if (warp == PV_WARP) tmem_alloc(tmem_slot, TMEM_COLS);
 
   if (!p.prewait_kv) pdl_wait();
   const QueryBlock qb(p, blockIdx.z);  // (early reads: n_ctx; the device counts are used by prompt chunks only)
@@ -270,37 +275,55 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // ---- KV staging (the loader warp, all lanes together): K or V of tile t into stage st,
-  // a page's planes and dim halves as one box per lane (4 or 8 KB); pages at or past kend
-  // are requested out of bounds (zero fill). ----
+  // ---- KV loads (the loader warp, all lanes together).  The tiles go through the ring in
+  // the order in which they are consumed, K0 K1 V0 K2 V1 K3 ...: position 0 is K of tile 0,
+  // an odd position 2 i - 1 K of tile i, an even one 2 i + 2 V of tile i (the one that K of
+  // tile nt would have stays empty).  Tile index i: the local tile (i = 0 when hl; not
+  // loaded) or pool tile t0 + i - hl.  A page's planes and dim halves are one box per lane
+  // (4 or 8 KB); pages at or past kend are requested out of bounds (zero fill). ----
+  auto k_pos = [](int i) { return i > 0 ? 2 * i - 1 : 0; };
+  auto v_pos = [](int i) { return 2 * i + 2; };
   const int groups_per_layer = static_cast<int>(p.pool_layer_stride / (16 * HD));  // 16-row planes
-  auto issue_half = [&](int t, int st, int kend, bool is_v) {
-    uint64_t* bar = is_v ? &v_full[st] : &k_full[st];
-    if (lane == 0) mbar_arrive_expect_tx(bar, static_cast<uint32_t>(HALF_BYTES));
-    __syncwarp();
-    if (lane < 4) {
-      const int kg = t * KT + lane * 16;
-      int y = static_cast<int>(p.pool_rows / 16);  // out of bounds
-      if (kg < kend) {
-        const int page = cached ? s_pages[(t - t0) * 4 + lane] : p.page_table[b * p.max_pages + t * 4 + lane];
-        y = p.layer * groups_per_layer + (page * p.H + h) * NP + (is_v ? KP : 0);
-      }
-      tma_load_5d((is_v ? vbuf : kbuf) + st * HALF_BYTES + lane * PAGE_BYTES, &args.kv_map, 0, 0, 0, y, 0, bar);
+  auto tile_of = [&](int pos, bool& is_v) {
+    is_v = pos > 0 && (pos & 1) == 0;
+    return is_v ? (pos - 2) >> 1 : (pos + 1) >> 1;
+  };
+  auto box_of = [&](int pos, int end) {  // the box this lane requests
+    bool is_v;
+    const int t = t0 + tile_of(pos, is_v) - hl;
+    int y = static_cast<int>(p.pool_rows / 16);  // out of bounds
+    if (lane < 4 && t * KT + lane * 16 < end) {
+      const int page = cached ? s_pages[(t - t0) * 4 + lane] : p.page_table[b * p.max_pages + t * 4 + lane];
+      y = p.layer * groups_per_layer + (page * p.H + h) * NP + (is_v ? KP : 0);
     }
+    return y;
+  };
+  auto request = [&](int slot, int y) {
+    if (lane == 0) mbar_arrive_expect_tx(&full[slot], static_cast<uint32_t>(HALF_BYTES));
+    __syncwarp();
+    if (lane < 4) tma_load_5d(ring + slot * HALF_BYTES + lane * PAGE_BYTES, &args.kv_map, 0, 0, 0, y, 0, &full[slot]);
+  };
+  // a tile to load (or nothing at this position)
+  auto wanted = [&](int pos) {
+    bool is_v;
+    const int i = tile_of(pos, is_v);
+    return i < nt && !(hl && i == 0);
   };
 
-  int pre = 0;  // leading tiles (K and V) requested before the dependency wait
+  int next_pos = 0;  // positions requested before the dependency wait
   if (p.prewait_kv) {
-    if (warp == SOFT_WARPS) {
+    if (warp == LOAD_WARP) {
       if (lane == 0) prefetch_tensormap(&args.kv_map);
       __syncwarp();
       // pool tiles whose rows are all committed (local mode: rows at or past nctx are
       // masked; the pool holds finite values there, the pools being cleared at set-up)
-      // (with many rows and split planes the local tile's owner stages k and v in stage 1 first)
-      while (hl + pre < nt && hl + pre < STAGES && !(SPLIT && MANY && hl) && (lmode || (t0 + pre + 1) * KT <= nctx)) {
-        issue_half(t0 + pre, (hl + pre) & 1, nctx, false);
-        issue_half(t0 + pre, (hl + pre) & 1, nctx, true);
-        ++pre;
+      // (with many rows and split planes the local tile's owner stages k and v in slots 3 and 4 first)
+      const int lim = SPLIT && MANY && hl ? 3 : SLOTS;
+      for (; next_pos < lim; ++next_pos) {
+        bool is_v;
+        if (!wanted(next_pos)) continue;
+        if (!lmode && (t0 + tile_of(next_pos, is_v) + 1) * KT > nctx) break;
+        request(next_pos, box_of(next_pos, nctx));
       }
     }
     __syncwarp();
@@ -458,8 +481,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       // stage 0: row i, dims j .. j + 3 (half 0) and 64 + j .. (half 1): half of chunk j / 8
       const uint32_t o0 = (i >> 3) * ROW_STRIDE + swz(i & 7, j >> 3) + ((j & 7) << 1);
       const uint32_t o1 = GROUP + o0;
-      uint8_t* kt = kbuf;
-      uint8_t* vt = vbuf;
+      uint8_t* kt = ring + k_pos(0) * HALF_BYTES;
+      uint8_t* vt = ring + v_pos(0) * HALF_BYTES;
       *reinterpret_cast<uint2*>(kt + o0) = kh0;
       *reinterpret_cast<uint2*>(kt + o1) = kh1;
       *reinterpret_cast<uint2*>(vt + o0) = vh0;
@@ -516,9 +539,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   fence_async_smem();  // the Q tiles (and the local K, V tile) are read by the tensor cores (async proxy)
   __threadfence_block();
   __syncthreads();
-  if (hl && threadIdx.x == 0) {  // the local tile is in place: stage 0 of K and V is full
-    mbar_arrive(&k_full[0]);
-    mbar_arrive(&v_full[0]);
+  if (hl && threadIdx.x == 0) {  // the local tile is in place: the slots of K and V of tile 0 are full
+    mbar_arrive(&full[k_pos(0)]);
+    mbar_arrive(&full[v_pos(0)]);
   }
 
   // softmax state of this lane's row (softmax warps)
@@ -527,129 +550,93 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   const uint32_t tlane = static_cast<uint32_t>(quad * 32) << 16;
   float m_used = -INFINITY, l = 0.f;
 
-  if (warp == SOFT_WARPS) {
-    // ---------------- KV loader (the whole warp; lane 0 polls and decides) ----------------
+  if (warp == LOAD_WARP) {
+    // ---------------- KV loader (the whole warp) ----------------
     if (!p.prewait_kv && lane == 0) prefetch_tensormap(&args.kv_map);
     __syncwarp();
-    // K of tile j needs the QK product of tile j - 2 done, V of tile j the PV product
-    // of tile j - 2; both are polled so that neither waits behind the other
-    // tile index i: the local tile (i = 0 when hl) or pool tile t0 + i - hl, stage i & 1
-    const int kend = lmode ? nctx : total;
-    int nk = hl + pre, nv = hl + pre;
-    uint64_t last_progress = global_timer_ns();
-    while (nk < nt || nv < nt) {
-      bool moved = false;
-      const int kgo = __shfl_sync(0xffffffffu, (lane == 0 && nk < nt &&
-                                                (nk < STAGES || mbar_test(&k_empty[nk & 1], ((nk - STAGES) >> 1) & 1))) ? 1 : 0, 0);
-      if (kgo) {
-        issue_half(t0 + nk - hl, nk & 1, kend, false);
-        ++nk;
-        moved = true;
+    const int end = lmode ? nctx : total;
+    const int last_pos = nt > 0 ? v_pos(nt - 1) : -1;
+    int slot = next_pos % SLOTS;
+    uint32_t phase = static_cast<uint32_t>(next_pos / SLOTS) & 1u;
+    for (; next_pos <= last_pos; ++next_pos) {
+      if (wanted(next_pos)) {
+        const int y = box_of(next_pos, end);
+        if (next_pos >= SLOTS && !mbar_wait_warp(&empty[slot], phase ^ 1u, abort)) break;
+        request(slot, y);
       }
-      const int vgo = __shfl_sync(0xffffffffu, (lane == 0 && nv < nk &&
-                                                (nv < STAGES || mbar_test(&v_empty[nv & 1], ((nv - STAGES) >> 1) & 1))) ? 1 : 0, 0);
-      if (vgo) {
-        issue_half(t0 + nv - hl, nv & 1, kend, true);
-        ++nv;
-        moved = true;
+      if (++slot == SLOTS) {
+        slot = 0;
+        phase ^= 1u;
       }
-      int quit = 0;
-      if (lane == 0) {
-        if (moved)
-          last_progress = global_timer_ns();
-        else if (global_timer_ns() - last_progress > 2000000000ull)
-          *abort = 1;
-        quit = *abort;
-      }
-      if (__shfl_sync(0xffffffffu, quit, 0)) break;
     }
     // copies still in flight when the CTA gives up: let them land before it exits
-    if (lane == 0 && *abort) {
-      for (int j = nk - 1; j >= 0 && j >= nk - STAGES; --j) mbar_wait_plain(&k_full[j & 1], (j >> 1) & 1, 200000000ull);
-      for (int j = nv - 1; j >= 0 && j >= nv - STAGES; --j) mbar_wait_plain(&v_full[j & 1], (j >> 1) & 1, 200000000ull);
-    }
+    if (*abort)
+      for (int j = next_pos - 1; j >= 0 && j >= next_pos - SLOTS; --j)
+        if (wanted(j)) mbar_wait_plain(&full[j % SLOTS], (j / SLOTS) & 1, 200000000ull);
     __syncwarp();
-  } else if (warp == MMA_WARP) {
-    // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+  } else if (warp == QK_WARP || warp == PV_WARP) {
+    // ---------------- MMA issuers (a warp for each product, one elected lane issues) ----------------
     const int ntu = __shfl_sync(0xffffffffu, nt, 0);
     if (ntu > 0) {
       const uint32_t elected = elect_one();
-      const uint32_t id_qk = idesc_f16(NQ, KT, false);
-      const uint32_t id_pv = idesc_f16(NQ, HD, true);
+      constexpr uint64_t LO_OFS = PLANE_STRIDE >> 4;  // hi plane -> lo plane
       // descriptors are made once; advancing an operand by b bytes adds b >> 4 to its
       // start-address field (all operands lie below 256 KB of shared memory)
-      const uint64_t dq_h = desc_sw128(smem_u32(q_hi), 16, 1024), dq_l = desc_sw128(smem_u32(q_lo), 16, 1024);
-      const uint64_t dp = desc_sw128(smem_u32(p_buf), 16, 1024);
-      const uint64_t dk = desc_sw128(smem_u32(kbuf), 16, ROW_STRIDE);
-      // V as MN-major B: 64-dim atoms GROUP apart (leading), 8-key groups ROW_STRIDE apart
-      const uint64_t dv = desc_sw128(smem_u32(vbuf), GROUP, ROW_STRIDE);
-      constexpr uint64_t LO_OFS = PLANE_STRIDE >> 4;  // hi plane -> lo plane
-      constexpr uint64_t P_LO_OFS = (NQ * 128) >> 4;  // P hi -> P lo (8 KB)
-      auto pv = [&](int i) {  // O[i & 1] += P_i V_i
-        const uint32_t st = i & 1;
-        const uint32_t o_t = tmem + O_COL + st * 128;
-        const uint64_t a0 = dp + static_cast<uint64_t>(st * (2 * NQ * 128 >> 4));
-        const uint64_t b0 = dv + static_cast<uint64_t>(st * (HALF_BYTES >> 4));
-        uint32_t acc = i > 1 ? 1u : 0u;
-#pragma unroll
-        for (int ks = 0; ks < KT / 16; ++ks) {
-          const uint64_t a_h = a0 + static_cast<uint64_t>(ks * 2);                   // 32 bytes per K step
-          const uint64_t b_h = b0 + static_cast<uint64_t>(ks * (PAGE_BYTES >> 4));  // 16 keys: a page
-          tc_mma_bf16(o_t, a_h, b_h, id_pv, acc, elected);
-          acc = 1;
-          tc_mma_bf16(o_t, a_h + P_LO_OFS, b_h, id_pv, 1u, elected);
-          if (SPLIT) tc_mma_bf16(o_t, a_h, b_h + LO_OFS, id_pv, 1u, elected);
-        }
-        tc_commit(&pv_done[st], elected);
-        tc_commit(&v_empty[st], elected);
-      };
-      auto qk = [&](int i) {  // S_i = Q K_i^T into S buffer i & 1
-        const uint32_t st = i & 1;
-        const uint32_t s_t = tmem + st * 64;
-        const uint64_t b0 = dk + static_cast<uint64_t>(st * (HALF_BYTES >> 4));
-#pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const uint64_t a_ofs = static_cast<uint64_t>(((ks >> 2) * ATOM_ROWS64 + (ks & 3) * 32) >> 4);
-          const uint64_t b_h = b0 + static_cast<uint64_t>(((ks >> 2) * GROUP + (ks & 3) * 32) >> 4);
-          tc_mma_bf16(s_t, dq_h + a_ofs, b_h, id_qk, ks > 0 ? 1u : 0u, elected);
-          tc_mma_bf16(s_t, dq_l + a_ofs, b_h, id_qk, 1u, elected);
-          if (SPLIT) tc_mma_bf16(s_t, dq_h + a_ofs, b_h + LO_OFS, id_qk, 1u, elected);
-        }
-        tc_commit(&s_full[st], elected);
-        tc_commit(&k_empty[st], elected);
-      };
-      // issue whichever product is ready: PV(npv) when P and V of tile npv are in, QK(nqk)
-      // when K is in and the softmax of tile nqk - 2 has read its S buffer (so no barrier is
-      // ever two phases ahead of its waiter)
-      int nqk = 0, npv = 0;
-      uint64_t last_progress = global_timer_ns();
-      while (npv < ntu) {
-        bool moved = false;
-        if (npv < nqk && __all_sync(0xffffffffu, mbar_test(&p_full[npv & 1], (npv >> 1) & 1) &&
-                                                     mbar_test(&v_full[npv & 1], (npv >> 1) & 1))) {
+      if (warp == QK_WARP) {  // S_i = Q K_i^T into S buffer i & 1, once the softmax has read S_(i - 2)
+        const uint32_t id_qk = idesc_f16(NQ, KT, false);
+        const uint64_t dq_h = desc_sw128(smem_u32(q_hi), 16, 1024), dq_l = desc_sw128(smem_u32(q_lo), 16, 1024);
+        const uint64_t dk = desc_sw128(smem_u32(ring), 16, ROW_STRIDE);
+        for (int i = 0; i < ntu; ++i) {
+          const int pos = k_pos(i), slot = pos % SLOTS, st = i & 1;
+          if (i >= 2 && !mbar_wait_warp(&s_free[st], ((i - 2) >> 1) & 1, abort)) break;
+          // (K of tile i may follow V of tile i - 4 in its slot, whose load need not have landed
+          // yet: a wait two phases ahead would pass on the parity of the phase before)
+          if (pos >= SLOTS && !mbar_wait_warp(&empty[slot], (pos / SLOTS - 1) & 1, abort)) break;
+          if (!mbar_wait_warp(&full[slot], (pos / SLOTS) & 1, abort)) break;
           tc_fence_after();
-          pv(npv);
-          ++npv;
-          moved = true;
+          const uint32_t s_t = tmem + st * 64;
+          const uint64_t b0 = dk + static_cast<uint64_t>(slot * (HALF_BYTES >> 4));
+#pragma unroll
+          for (int ks = 0; ks < HD / 16; ++ks) {
+            const uint64_t a_ofs = static_cast<uint64_t>(((ks >> 2) * ATOM_ROWS64 + (ks & 3) * 32) >> 4);
+            const uint64_t b_h = b0 + static_cast<uint64_t>(((ks >> 2) * GROUP + (ks & 3) * 32) >> 4);
+            tc_mma_bf16(s_t, dq_h + a_ofs, b_h, id_qk, ks > 0 ? 1u : 0u, elected);
+            tc_mma_bf16(s_t, dq_l + a_ofs, b_h, id_qk, 1u, elected);
+            if (SPLIT) tc_mma_bf16(s_t, dq_h + a_ofs, b_h + LO_OFS, id_qk, 1u, elected);
+          }
+          tc_commit(&empty[slot], elected);
+          tc_commit(&s_full[st], elected);
         }
-        if (nqk < ntu &&
-            __all_sync(0xffffffffu, mbar_test(&k_full[nqk & 1], (nqk >> 1) & 1) &&
-                                        (nqk < 2 || mbar_test(&s_free[nqk & 1], ((nqk - 2) >> 1) & 1)))) {
+      } else {  // O[i & 1] += P_i V_i
+        const uint32_t id_pv = idesc_f16(NQ, HD, true);
+        const uint64_t dp = desc_sw128(smem_u32(p_buf), 16, 1024);
+        // V as MN-major B: 64-dim atoms GROUP apart (leading), 8-key groups ROW_STRIDE apart
+        const uint64_t dv = desc_sw128(smem_u32(ring), GROUP, ROW_STRIDE);
+        constexpr uint64_t P_LO_OFS = (NQ * 128) >> 4;  // P hi -> P lo (8 KB)
+        for (int i = 0; i < ntu; ++i) {
+          const int pos = v_pos(i), slot = pos % SLOTS, st = i & 1;
+          if (!mbar_wait_warp(&full[slot], (pos / SLOTS) & 1, abort)) break;
+          if (!mbar_wait_warp(&p_full[st], (i >> 1) & 1, abort)) break;
           tc_fence_after();
-          qk(nqk);
-          ++nqk;
-          moved = true;
-        }
-        if (moved) {
-          last_progress = global_timer_ns();
-        } else {
-          const bool late = global_timer_ns() - last_progress > 2000000000ull;
-          if (late) *abort = 1;
-          if (__any_sync(0xffffffffu, late || *abort)) break;
+          const uint32_t o_t = tmem + O_COL + st * 128;
+          const uint64_t a0 = dp + static_cast<uint64_t>(st * (2 * NQ * 128 >> 4));
+          const uint64_t b0 = dv + static_cast<uint64_t>(slot * (HALF_BYTES >> 4));
+          uint32_t acc = i > 1 ? 1u : 0u;
+#pragma unroll
+          for (int ks = 0; ks < KT / 16; ++ks) {
+            const uint64_t a_h = a0 + static_cast<uint64_t>(ks * 2);                   // 32 bytes per K step
+            const uint64_t b_h = b0 + static_cast<uint64_t>(ks * (PAGE_BYTES >> 4));  // 16 keys: a page
+            tc_mma_bf16(o_t, a_h, b_h, id_pv, acc, elected);
+            acc = 1;
+            tc_mma_bf16(o_t, a_h + P_LO_OFS, b_h, id_pv, 1u, elected);
+            if (SPLIT) tc_mma_bf16(o_t, a_h, b_h + LO_OFS, id_pv, 1u, elected);
+          }
+          tc_commit(&empty[slot], elected);
+          tc_commit(&pv_done[st], elected);
         }
       }
       tc_commit(o_done, elected);  // all MMAs issued by this lane, including any after an abort
-      // tensor memory and the KV stages are released only after every MMA completed
+      // tensor memory and the KV slots are released only after every MMA completed
       mbar_wait_plain(o_done, 0, 200000000ull);
     }
   } else {
@@ -684,11 +671,17 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&s_free[strm]);
-      // this stream's P buffer and O accumulator were used by the PV product of tile i - 2
-      if (i >= 2) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&pv_done[strm], ((i - 2) >> 1) & 1, abort))) break;
-        tc_fence_after();
-      }
+      // this stream's P buffer and O accumulator are used by the PV product of tile i - 2:
+      // waited for when one of them is first written, after the arithmetic
+      bool pv_ok = i < 2;
+      auto wait_pv = [&] {
+        if (!pv_ok) {
+          pv_ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[strm], ((i - 2) >> 1) & 1, abort));
+          tc_fence_after();
+        }
+        return pv_ok;
+      };
+      uint4 hh[4], ll[4];
       if (any) {
         // visibility of this lane's 32 keys (bit j: key 32 sub + j of the tile): the local
         // tile's keys are local rows (ancestor mask), a pool tile's keys are slots 64 t ..
@@ -729,6 +722,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           m_used = tmax;
         }
         if (__any_sync(0xffffffffu, rescale)) {  // factor 1 for rows that kept m
+          if (!wait_pv()) break;
           const float f = rescale ? corr : 1.f;
           const uint32_t oa = tmem + tlane + O_COL + strm * 128;
           uint32_t rr[4][16];
@@ -754,15 +748,20 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
             e[j] = ex2_approx(fmaf(sv[8 * c + j], scale2, -mm));
             l4[j & 3] += e[j];
           }
-          uint4 hh, ll;
-          split_pair(e[0], e[1], hh.x, ll.x);
-          split_pair(e[2], e[3], hh.y, ll.y);
-          split_pair(e[4], e[5], hh.z, ll.z);
-          split_pair(e[6], e[7], hh.w, ll.w);
-          *reinterpret_cast<uint4*>(ph + swz(r, 4 * sub + c)) = hh;
-          *reinterpret_cast<uint4*>(pl + swz(r, 4 * sub + c)) = ll;
+          split_pair(e[0], e[1], hh[c].x, ll[c].x);
+          split_pair(e[2], e[3], hh[c].y, ll[c].y);
+          split_pair(e[4], e[5], hh[c].z, ll[c].z);
+          split_pair(e[6], e[7], hh[c].w, ll[c].w);
         }
         l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+      }
+      if (!wait_pv()) break;
+      if (any) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          *reinterpret_cast<uint4*>(ph + swz(r, 4 * sub + c)) = hh[c];
+          *reinterpret_cast<uint4*>(pl + swz(r, 4 * sub + c)) = ll[c];
+        }
         fence_async_smem();
       }
       tc_fence_before();
@@ -877,7 +876,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     __syncwarp();
   }
   if (S > 1) cluster_arrive();
-  if (warp == MMA_WARP) {
+  if (warp == PV_WARP) {
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
   }
@@ -921,7 +920,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   }
 }
 
-constexpr size_t TC_SMEM = 1024 + TILE_BYTES + 18 * 8 + 16 + (PAGE_CACHE + 8) * 4;
+constexpr size_t TC_SMEM = 1024 + TILE_BYTES + 22 * 8 + 16 + (PAGE_CACHE + 8) * 4;
 
 // The dynamic shared memory limit is an attribute of the device that is current when it
 // is set: raised once per device (and kernel variant), the return code checked.

@@ -172,6 +172,7 @@ ATT_CASES = [
     (1, 2, 128, [0], 3, 3, 0, 1),            # one tile: the odd-tile stream has none
     (2, 2, 128, [100, 63], 17, 17, 0, 1),    # two tiles (and a row in a second warp), 80 keys
     (1, 2, 128, [1500], 33, 33, 0, 2),       # many tiles per stream, row counts no multiple of 16
+    (2, 40, 128, [2100, 330], 5, 1, 4, 2),   # one query, tiles around the ring, more CTAs than SMs
 ]
 
 
