@@ -9,10 +9,11 @@
 //
 // This file holds the SIMT kernel (fp32 models, and bf16 models with head_dim 64), whose
 // splits merge in the last CTA of each (b, h) through a global workspace, and the
-// dispatch; bf16 models with head_dim 128 take the tensor-core kernel of attention_tc.cu,
-// which can also fuse RoPE and the KV write of the step's fresh rows.
+// dispatch; bf16 models with head_dim 128 take the tensor-core kernel of attention_tc.cu.
+// Both can also fuse RoPE and the KV write of the step's fresh rows (fp32 models here).
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "attention.cuh"
 #include "common.cuh"
@@ -159,7 +160,12 @@ __device__ __forceinline__ float half_sum_many(float (&v)[NV], int lane) {
 // 16 tree rows 17 -> 13; a 64-token prompt and eight steps 2.70 -> 2.26 ms.  The kernel
 // before staged 32-key tiles for all queries, kept seven of eight warps idle for one
 // query, and always split 16 ways.
-template <typename TKV, typename T, int HD, int QG>
+//
+// ROPE: the queries come from the projections, and the CTA rotates and writes to the pool
+// the fresh rows of its own key range before it reads that range: no other CTA's rows are
+// needed, and CTAs of the same range (query groups) write the same values.  Six RoPE
+// launches of a step's 73 are saved (fp32, 256 wide, 16-node tree: 186 -> 179 us a step).
+template <typename TKV, typename T, int HD, int QG, bool ROPE>
 __global__ void __launch_bounds__(THREADS) attn_kernel(const AttnParams p, int groups) {
   pdl_trigger();  // the next kernel may start its prologue
   pdl_wait();     // inputs of this kernel are complete
@@ -185,14 +191,61 @@ __global__ void __launch_bounds__(THREADS) attn_kernel(const AttnParams p, int g
 
   const int qi = hl / LPQ;           // this lane's query within the group
   const unsigned long long mask = qi < nqg ? p.anc[p.q_local0 + q0 + qi] : 0ull;
-  for (int it = threadIdx.x; it < QG * (HD / 4); it += THREADS) {
-    const int i = it / (HD / 4), c = it % (HD / 4) * 4;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i < nqg) {
-      const float* src = p.q + static_cast<size_t>(qb.row0 + q0 + i) * p.ldq + h * HD + c;
-      x = make_float4(src[0], src[1], src[2], src[3]);
+  if constexpr (ROPE) {
+    constexpr int HALF = HD / 2, J4 = HALF / 4;
+    // (cos, sin) of position n_ctx + pos_base + .. of row i, dims j .. j + 3 of a half
+    auto angles = [&](int pos, int j, float4& c, float4& sn) {
+      const float4* t = reinterpret_cast<const float4*>(p.rope + static_cast<size_t>(pos) * HALF + j);
+      const float4 a = t[0], e = t[1];
+      c = make_float4(a.x, a.z, e.x, e.z);
+      sn = make_float4(a.y, a.w, e.y, e.w);
+    };
+    auto pos_of = [&](int i) { return nctx + p.pos_base + (p.pos_off ? p.pos_off[i] : i); };
+    for (int it = threadIdx.x; it < QG * J4; it += THREADS) {
+      const int i = it / J4, j = it % J4 * 4;
+      float4 y1 = make_float4(0.f, 0.f, 0.f, 0.f), y2 = y1;
+      if (i < nqg) {
+        float4 c, sn;
+        angles(min(max(pos_of(q0 + i), 0), p.max_pos - 1), j, c, sn);
+        const float* src = p.qkv + static_cast<size_t>(qb.row0 + q0 + i) * p.ldqkv + h * HD + j;
+        const float4 x1 = *reinterpret_cast<const float4*>(src), x2 = *reinterpret_cast<const float4*>(src + HALF);
+        y1 = rot_lo(x1, x2, c, sn);
+        y2 = rot_hi(x1, x2, c, sn);
+      }
+      *reinterpret_cast<float4*>(qs + i * HD + j) = y1;
+      *reinterpret_cast<float4*>(qs + i * HD + HALF + j) = y2;
     }
-    *reinterpret_cast<float4*>(qs + i * HD + c) = x;
+    const int fresh0 = nctx + p.q_local0, f0 = max(0, k0 - fresh0), f1 = min(nq, k1 - fresh0);
+    for (int it = threadIdx.x; it < (f1 - f0) * J4; it += THREADS) {
+      const int i = f0 + it / J4, j = it % J4 * 4, slot = fresh0 + i, pos = pos_of(i);
+      if (pos < 0 || pos >= p.max_pos || (slot >> 4) >= p.max_pages) {
+        if (p.err) atomicOr(p.err, ERR_CAPACITY);
+        continue;
+      }
+      float4 c, sn;
+      angles(pos, j, c, sn);
+      const float* src = p.qkv + static_cast<size_t>(qb.row0 + i) * p.ldqkv + (p.H + h) * HD + j;
+      const float4 x1 = *reinterpret_cast<const float4*>(src), x2 = *reinterpret_cast<const float4*>(src + HALF);
+      const float4 v1 = *reinterpret_cast<const float4*>(src + p.H * HD);
+      const float4 v2 = *reinterpret_cast<const float4*>(src + p.H * HD + HALF);
+      TKV* row = const_cast<TKV*>(pool) +
+                 (static_cast<size_t>(p.page_table[b * p.max_pages + (slot >> 4)]) * p.H + h) * p.planes * 16 * HD +
+                 (slot & 15) * HD + j;
+      store4<TKV>(row, rot_lo(x1, x2, c, sn));
+      store4<TKV>(row + HALF, rot_hi(x1, x2, c, sn));
+      store4<TKV>(row + v_ofs, v1);
+      store4<TKV>(row + v_ofs + HALF, v2);
+    }
+  } else {
+    for (int it = threadIdx.x; it < QG * (HD / 4); it += THREADS) {
+      const int i = it / (HD / 4), c = it % (HD / 4) * 4;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < nqg) {
+        const float* src = p.q + static_cast<size_t>(qb.row0 + q0 + i) * p.ldq + h * HD + c;
+        x = make_float4(src[0], src[1], src[2], src[3]);
+      }
+      *reinterpret_cast<float4*>(qs + i * HD + c) = x;
+    }
   }
   __syncthreads();
 
@@ -357,10 +410,15 @@ cudaError_t launch(AttnParams p, cudaStream_t s) {
   p.splits = std::max(1, std::min(p.splits, (p.max_pages * 16 + SPLIT_KEYS - 1) / SPLIT_KEYS));
   const int groups = p.nq_max == 1 ? 1 : (p.nq_max + QG - 1) / QG;
   const dim3 grid(p.splits, p.H, p.B * std::max(1, p.q_blocks) * groups);
-  if (p.nq_max == 1)
-    launch_pdl(attn_kernel<TKV, T, HD, 1>, grid, dim3(THREADS), 0, s, p, groups);
-  else
-    launch_pdl(attn_kernel<TKV, T, HD, QG>, grid, dim3(THREADS), 0, s, p, groups);
+  if constexpr (std::is_same_v<TKV, float>) {
+    if (p.qkv) {
+      launch_pdl(p.nq_max == 1 ? attn_kernel<TKV, T, HD, 1, true> : attn_kernel<TKV, T, HD, QG, true>, grid, dim3(THREADS),
+                 0, s, p, groups);
+      return cudaGetLastError();
+    }
+  }
+  launch_pdl(p.nq_max == 1 ? attn_kernel<TKV, T, HD, 1, false> : attn_kernel<TKV, T, HD, QG, false>, grid, dim3(THREADS),
+             0, s, p, groups);
   return cudaGetLastError();
 }
 
@@ -370,10 +428,12 @@ size_t attn_ws_floats(int B, int H, int splits, int nq_max, int hd) {
   return static_cast<size_t>(B) * H * splits * nq_max * (hd + 4);
 }
 
-bool attn_fuses_rope(int dtype, int hd) { return dtype == 1 && hd == 128; }
+bool attn_on_tensor_cores(int dtype, int hd) { return dtype == 1 && hd == 128; }
+// (bf16 models of 64-dim heads, for which no configuration is tuned, rotate in a launch of their own)
+bool attn_fuses_rope(int dtype, int hd) { return dtype == 0 || attn_on_tensor_cores(dtype, hd); }
 
 int attn_pick_splits(int dtype, int hd, int planes, int B, int H, int want) {
-  if (!attn_fuses_rope(dtype, hd)) return want;
+  if (!attn_on_tensor_cores(dtype, hd)) return want;
   return attention_tc_splits(planes, B * H, want);
 }
 
@@ -383,13 +443,12 @@ cudaError_t attention(const AttnParams& p, int dtype, cudaStream_t s) {
   // blocks of prompt rows: device row counts, no fused projections, one split per block
   if (p.q_blocks > 1 && (p.qkv || !p.nq_dev || !p.n_local_dev || p.q_local0 != 0 || p.nq != 64 || p.n_local != 64 || p.splits != 1))
     return cudaErrorInvalidValue;
+  if (p.qkv && (!p.rope || !p.err || p.max_pos < 1 || (p.ldqkv & 3))) return cudaErrorInvalidValue;
   if (dtype == 0) {
-    if (p.qkv) return cudaErrorInvalidValue;
     if (p.hd == 64) return launch<float, float, 64>(p, s);
     if (p.hd == 128) return launch<float, float, 128>(p, s);
   } else if (p.hd == 128) {
     if (p.splits > 8) return cudaErrorInvalidValue;  // one cluster of at most 8 CTAs per (b, h)
-    if (p.qkv && (!p.rope || !p.err || p.max_pos < 1 || (p.ldqkv & 3))) return cudaErrorInvalidValue;
     return attention_tc(p, s);
   } else if (p.hd == 64) {
     if (p.qkv) return cudaErrorInvalidValue;

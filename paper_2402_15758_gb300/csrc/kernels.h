@@ -225,7 +225,7 @@ struct AttnParams {
   // counts covering all of them (nq and n_local then per block: 64); its context is the n_ctx
   // committed rows and the 64 j local rows before it.
   int q_blocks;
-  // Fused RoPE + KV write (bf16 models, head_dim 128).  With qkv set, the queries and
+  // Fused RoPE + KV write (fp32 models; bf16 models, head_dim 128).  With qkv set, the queries and
   // the nq fresh local rows come from the fp32 projections: row (b * q_rows + i) holds
   // q at column h*hd, k at H*hd + h*hd, v at 2*H*hd + h*hd.  Query / fresh row i sits at
   // position n_ctx + pos_base + (pos_off ? pos_off[i] : i) and at local row q_local0 + i
@@ -261,6 +261,8 @@ int encode_5d_bf16(CUtensorMap* map, const void* base, const uint64_t (&dims)[5]
 // Tensor-core tree attention (bf16 planes, head_dim 128; splits <= 8 form one cluster).
 cudaError_t attention_tc(const AttnParams& p, cudaStream_t s);
 int attention_tc_splits(int planes, int BH, int want);
+// True when attention() takes the tensor-core kernel for this model.
+bool attn_on_tensor_cores(int dtype, int hd);
 // True when attention() fuses RoPE and the KV write (qkv given) for this model.
 bool attn_fuses_rope(int dtype, int hd);
 

@@ -392,7 +392,7 @@ bool make_lin(chimera_ctx* ctx, Lin* l, int M, int N, int K, const void* X, cons
 #define CHIMERA_ATT_TILES_PER_CTA 32
 #endif
 int att_splits(const chimera_ctx* ctx, int B, int nq, int n_keys) {
-  if (attn_fuses_rope(ctx->dtype, ctx->hd)) {
+  if (attn_on_tensor_cores(ctx->dtype, ctx->hd)) {
     // tensor-core tree attention: one cluster of S CTAs per (b, h).  While the B * H
     // clusters fit on the SMs at once, as many splits as keep them all resident; with
     // more (sequence, head) pairs than SMs the launch runs in waves whatever S is, so
@@ -414,8 +414,8 @@ int att_splits(const chimera_ctx* ctx, int B, int nq, int n_keys) {
 
 // With qkv (models where attn_fuses_rope holds) the kernel also rotates q and the nq
 // fresh rows' k (positions n + pos_base + pos_off[i]) and writes their k, v to the pool.
-// It then reads n_ctx, the page table and the committed KV rows BEFORE its own
-// dependency wait (prewait_kv).  That is only correct when the launch directly before
+// On the tensor cores it then reads n_ctx, the page table and the committed KV rows BEFORE
+// its own dependency wait (prewait_kv).  That is only correct when the launch directly before
 // it is a tensor-core linear: that kernel lets its dependents launch only after its
 // own griddepcontrol.wait, so every earlier kernel has completed by then.  Most row
 // kernels trigger before they wait; one of them directly before this launch could
@@ -425,8 +425,8 @@ cudaError_t run_attention(chimera_ctx* ctx, bool draft_pool, int layer, int nq, 
                           int nq_max, double bytes, const float* qkv = nullptr, int pos_base = 0,
                           const int* pos_off = nullptr, int q_blocks = 0) {
   if (filtered(ctx, CHIMERA_KIND_ATTENTION)) return cudaSuccess;
-  if (qkv && !ctx->filter_kind &&
-      !(ctx->dtype == 1 && (ctx->last_kind == CHIMERA_KIND_LINEAR || ctx->last_kind == CHIMERA_KIND_CHAIN))) {
+  const bool early = qkv && attn_on_tensor_cores(ctx->dtype, ctx->hd);
+  if (early && !ctx->filter_kind && ctx->last_kind != CHIMERA_KIND_LINEAR && ctx->last_kind != CHIMERA_KIND_CHAIN) {
     ctx->err = "attention with early KV reads must directly follow a tensor-core linear or chain";
     return cudaErrorInvalidValue;
   }
@@ -439,7 +439,7 @@ cudaError_t run_attention(chimera_ctx* ctx, bool draft_pool, int layer, int nq, 
     p.max_pos = ctx->max_pos;
     p.pos_base = pos_base;
     p.pos_off = pos_off;
-    p.prewait_kv = 1;
+    p.prewait_kv = early ? 1 : 0;
   }
   p.err = ctx->d_err;
   p.q = ctx->qr;

@@ -428,6 +428,34 @@ def test_prefill_chunks(name, lens):
             assert rel_rows(k, rk) <= tol and rel_rows(v, rv) <= tol, (b, layer)
 
 
+# fp32 attention that rotates and writes its fresh rows itself: tree rows on both sides of a
+# split's border (three splits of 128 keys, rows 250..), both head sizes, a context of 3 rows
+@pytest.mark.parametrize("heads", [4, 2])
+def test_fp32_fused_rope_splits(heads):
+    cfg, w_cpu, w_dev = _setup("tiny")
+    cfg = dict(cfg, n_heads=heads, head_dim=cfg["d_model"] // heads)
+    tol, tree, W = tol_of(cfg), ot.build_tree(cfg["topk"], cfg["tree_nodes"]), co.OracleWeights(w_cpu)
+    rng = np.random.default_rng(heads)
+    prompts = [rng.integers(0, cfg["vocab"], n).tolist() for n in (250, 3)]
+    ctx = pkg.Chimera(cfg, w_dev, max_batch=2, max_seq_len=600)
+    ctx.prefill(prompts)
+    sts = [co.prefill(W, cfg, x, 600) for x in prompts]
+    for _ in range(3):
+        emitted = ctx.step()
+        dl, vl = ctx.read("draft_logits"), ctx.read("verify_logits")
+        for b, st in enumerate(sts):
+            rec = co.step(W, cfg, st, tree)
+            assert rel_rows(dl[:, b], np.stack(rec["draft"]["logits"])) <= tol
+            assert rel_rows(vl[b], rec["verify"]["logits"]) <= tol
+            assert emitted[b] == rec["emitted"]
+    for b, st in enumerate(sts):
+        n = int(ctx.read("n")[b])
+        for layer in (0, -1):
+            k, v = ctx.read_kv(layer, b, 0, n)
+            rk, rv = (st.dK[:n], st.dV[:n]) if layer < 0 else (st.K[layer, :n], st.V[layer, :n])
+            assert rel_rows(k, rk) <= tol and rel_rows(v, rv) <= tol
+
+
 @pytest.mark.parametrize("name", ["tiny", "mini"])
 def test_prefill_again(name):
     # prompts of the same and of other lengths, batches and chunks on one context: the plans and
