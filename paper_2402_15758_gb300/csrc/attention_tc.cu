@@ -70,6 +70,10 @@ constexpr float RESCALE_LOG2 = 11.5f;        // raise the running max when it gr
 constexpr uint32_t TMEM_COLS = 512;          // S[2] (64 cols each), O[2] (128 cols each)
 constexpr uint32_t O_COL = 128;
 constexpr int MAX_PARTS = 16;                // partials of a row: one or two per split
+// The following linear's weights are requested into L2 by CTAs of at most this many tiles:
+// at 4 a step gains 0.2-1.1 % (4096 wide, one to four sequences), at 5-6 it is even or
+// loses 0.7 % and at 7-8 it loses 0.6-0.8 %, the requests competing with the KV loads.
+constexpr int NEXT_W_TILES = 4, NEXT_W_CHUNK = 4096;
 constexpr int MANY_NQ = 32;                  // more query rows than this take the MANY variant
 constexpr int PREC = HD + 4;                 // partial record (o[128], m, l, pad)
 constexpr int PART_FLOATS = (2 * MANY_NQ + 16) * PREC;  // the partial records of a CTA (<= NQ + 14 rows)
@@ -140,6 +144,11 @@ __device__ __forceinline__ float ex2_approx(float x) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Bulk request of `bytes` (a multiple of 16) at p into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes) : "memory");
+}
 
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
@@ -568,6 +577,14 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         slot = 0;
         phase ^= 1u;
       }
+    }
+    if (p.next_w && nt <= NEXT_W_TILES) {  // (all of this CTA's KV is requested)
+      const long long ctas = static_cast<long long>(gridDim.x) * gridDim.y * gridDim.z;
+      const long long cta = (static_cast<long long>(blockIdx.z) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+      const char* w = static_cast<const char*>(p.next_w);
+      for (long long o = (cta * 32 + lane) * NEXT_W_CHUNK; o < p.next_w_bytes; o += ctas * 32 * NEXT_W_CHUNK)
+        prefetch_l2(w + o, static_cast<uint32_t>(min(static_cast<long long>(NEXT_W_CHUNK), p.next_w_bytes - o)));
+      __syncwarp();
     }
     // copies still in flight when the CTA gives up: let them land before it exits
     if (*abort)

@@ -241,6 +241,10 @@ struct AttnParams {
   // own griddepcontrol.wait, so every kernel before it is complete and committed KV
   // rows (slots < n_ctx) may be read before this kernel's own wait
   int prewait_kv;
+  // weights of the linear that follows (optional, 16-byte aligned): with little KV to read the
+  // tensor-core kernel requests them into L2
+  const void* next_w;
+  long long next_w_bytes;
   int* err;
 };
 // dtype: 0 fp32 model (fp32 KV), 1 bf16 model (bf16 KV planes).

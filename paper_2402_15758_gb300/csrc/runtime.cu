@@ -471,6 +471,16 @@ cudaError_t run_attention(chimera_ctx* ctx, bool draft_pool, int layer, int nq, 
   p.counters = ctx->att_cnt;
   p.nq_max = nq_max;
   p.q_blocks = q_blocks;
+  // One wave of CTAs is bound by latency while the contexts are short and leaves DRAM idle:
+  // the kernel requests the O projection's weights into L2 once its own KV is requested.
+  // Step of a 64-node tree, 4096 wide, 512 rows, all 33.5 MB 3.920 ms, 24 MB 3.908, 16 MB
+  // 3.916, 8 MB 3.929, none 3.944 (more than the window holds delays the linear's own
+  // loads; all of it before the queries are read 3.983).
+  constexpr long long NEXT_W_BYTES = 24 << 20;
+  if (early && static_cast<long long>(splits) * ctx->H * ctx->batch <= ctx->num_sms) {
+    p.next_w = draft_pool ? ctx->draft.wo : ctx->layers[layer].wo;
+    p.next_w_bytes = std::min(NEXT_W_BYTES, static_cast<long long>(ctx->d) * ctx->d * static_cast<long long>(ctx->esz));
+  }
   if (attn_ws_floats(p.B, p.H, splits, nq_max, p.hd) > ctx->att_ws_floats) return cudaErrorInvalidValue;
   return attention(p, ctx->dtype, ctx->stream);
 }
