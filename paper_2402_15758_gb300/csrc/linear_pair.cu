@@ -38,6 +38,8 @@
 // 22016 x 4096: 72 rows 34.8 -> 31.9 us, 128 rows 41.1 -> 35.1, 256 rows 77.5 -> 60.6
 // (1.52 PFLOP/s), 512 rows 150.7 -> 108.7 (1.70);  4096 x 11008: 20.0 -> 18.8,
 // 23.8 -> 20.7, 41.7 -> 32.5, 76.7 -> 55.2.
+// Stored outputs, whose cut tiles go through the workspace (12288 x 4096, plain and SiLU to
+// bf16): 100 rows 40.2 and 47 -> 30.0 and 31 us, 256 rows 66.7 and 81 -> 44.1 and 47.
 // With the loads left out (wrong results) 256 rows of 22016 x 4096 take 45.7 us, without
 // the weights' alone 47.8: what is left is the L2's feed of the SMs.
 //
@@ -419,14 +421,41 @@ __device__ __forceinline__ void drain_tiles(const TcPairParams& p, int warp, int
     // ---- this pair's part of tile t is complete ----
     const int f = f0 + lane;
     const uint32_t c_first = pair_of_unit(t * w.KB, w.U, w.P), c_last = pair_of_unit(t * w.KB + w.KB - 1, w.U, w.P);
-    auto store = [&](int m, float x) {
-      if (m >= p.M || f >= p.N) return;
-      if (p.epi == EPI_SILU) x = silu_f(x);
-      const size_t idx = static_cast<size_t>(m) * p.ldy + f;
-      if (p.out_f32)
-        static_cast<float*>(p.Y)[idx] = x;
-      else
-        store_act(static_cast<bf16*>(p.Y), static_cast<bf16*>(p.Y2), idx, x);
+    // 8 tokens of this lane's feature
+    auto store8 = [&](int m, const float (&v)[8]) {
+      if (f >= p.N) return;
+      if (p.epi == EPI_RESID) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (m + j < p.M) red_add_f32(static_cast<float*>(p.Y) + static_cast<size_t>(m + j) * p.ldy + f, v[j]);
+        return;
+      }
+      if (p.epi == EPI_SILU) {
+        float e[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e[j] = 1.0f + expf(-v[j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (m + j >= p.M) break;
+          const float x = v[j] / e[j];
+          const size_t idx = static_cast<size_t>(m + j) * p.ldy + f;
+          if (p.out_f32)
+            static_cast<float*>(p.Y)[idx] = x;
+          else
+            store_act(static_cast<bf16*>(p.Y), static_cast<bf16*>(p.Y2), idx, x);
+        }
+        return;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const size_t idx = static_cast<size_t>(m + j) * p.ldy + f;
+        if (m + j < p.M) {
+          if (p.out_f32)
+            static_cast<float*>(p.Y)[idx] = v[j];
+          else
+            store_act(static_cast<bf16*>(p.Y), static_cast<bf16*>(p.Y2), idx, v[j]);
+        }
+      }
     };
     // slot of group c's partial of this token tile: [token][feature]
     auto slot = [&](uint32_t c) {
@@ -437,21 +466,16 @@ __device__ __forceinline__ void drain_tiles(const TcPairParams& p, int warp, int
     const bool parts = p.epi != EPI_RESID && c_first != c_last;
     float* wsp = parts ? slot(w.grp) : nullptr;
     int* counter = p.counters + 2 * (t * w.W + w.pair % w.W) + rank;
-#pragma unroll 1
-    for (int g = 0; g < gn; ++g) {
-      stage_group(g);
-#pragma unroll 1
-      for (int j = 0; j < 8; ++j) {
-        const float x = sw[j * RED_PITCH + lane];
-        const int m = m0 + g * 8 + j;
-        if (parts)
-          __stcg(wsp + (g * 8 + j) * BM, x);
-        else if (p.epi != EPI_RESID)
-          store(m, x);
-        else if (m < p.M && f < p.N)
-          red_add_f32(static_cast<float*>(p.Y) + static_cast<size_t>(m) * p.ldy + f, x);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      if (g < gn) {
+        if (parts) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) __stcg(wsp + (g * 8 + j) * BM, acc[g][j]);
+        } else {
+          store8(m0 + g * 8, acc[g]);
+        }
       }
-      __syncwarp();
     }
     if (parts) {  // the last pair to arrive sums the partials in pair order
       __threadfence();
@@ -460,25 +484,22 @@ __device__ __forceinline__ void drain_tiles(const TcPairParams& p, int warp, int
       named_bar(1, EPI_WARPS * 32);
       if (c->last) {
         __threadfence();
-#pragma unroll 1
-        for (int g = 0; g < gn; ++g) {
-          float v[8];
-          for (uint32_t c = c_first; c <= c_last; ++c) {
-            const float* src = slot(c) + g * 8 * BM;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float w = __ldcg(src + j * BM);
-              v[j] = c == c_first ? w : v[j] + w;
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
+        for (uint32_t c = c_first; c <= c_last; ++c) {  // a part's loads are all in flight at once
+          const float* src = slot(c);
+#pragma unroll
+          for (int g = 0; g < G; ++g)
+            if (g < gn) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) acc[g][j] += __ldcg(src + (g * 8 + j) * BM);
             }
-          }
-#pragma unroll 1
-          for (int j = 0; j < 8; ++j) {
-            float x = v[0];
-#pragma unroll
-            for (int i = 1; i < 8; ++i) x = j == i ? v[i] : x;
-            store(m0 + g * 8 + j, x);
-          }
         }
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+          if (g < gn) store8(m0 + g * 8, acc[g]);
         if (threadIdx.x == 64) *counter = 0;
       }
       named_bar(1, EPI_WARPS * 32);

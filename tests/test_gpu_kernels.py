@@ -78,6 +78,28 @@ def test_linear_bf16_split_operand(M, N, K):
     assert _rel_rows(Y.cpu().numpy(), ref) > 1e-4
 
 
+# stored outputs of tiles cut between CTAs: two to 71 parts per tile (a CTA
+# per stage when there are fewer stages than SMs), token tiles of 16, 32, 48 and 64 columns
+@pytest.mark.parametrize("M,N,K", [(1, 300, 1400), (24, 2050, 4104), (40, 12288, 520), (40, 300, 9000), (64, 1000, 4096)])
+@pytest.mark.parametrize("epi,out_f32", [(0, True), (1, True), (1, False)])
+def test_linear_stored_parts(M, N, K, epi, out_f32):
+    g = torch.Generator().manual_seed(M + N + K)
+    X32 = torch.randn(M, K, generator=g)
+    hi = X32.to(torch.bfloat16)
+    lo = (X32 - hi.float()).to(torch.bfloat16)
+    W = (torch.randn(N, K, generator=g) * 0.02).to(torch.bfloat16)
+    ref = ((hi.cuda().double() + lo.cuda().double()) @ W.cuda().double().T).cpu().numpy()
+    got = []
+    for _ in range(2):
+        Y = torch.full((M, N), float("nan"), dtype=torch.float32 if out_f32 else torch.bfloat16, device="cuda")
+        pkg.op_linear(hi.cuda(), W.cuda(), Y, epi=epi, out_f32=out_f32, X_lo=lo.cuda())
+        pkg.op_sync()
+        got.append(Y.float().cpu().numpy())
+    # chains of up to 563 truncated fp32 steps (2^-23 each, partly cancelling), or one rounding to bf16
+    assert _rel_rows(got[1], co.silu(ref) if epi else ref) <= (6e-5 if out_f32 else 8e-3)
+    assert np.array_equal(got[0], got[1])
+
+
 # the CTA-pair kernel: split activations of more than 64 rows with at least 1000 stages x
 # tokens per pair.  Ragged token tiles (1 of 80 and of 112 rows, 2 of 80, 3 of 96, 9 in two
 # rounds of 5), an odd number of 128-feature halves, columns that are no multiple of 4, a
