@@ -66,6 +66,9 @@ constexpr int MAX_TILES = 8192;
 // here, 20.6, 31.3, 18.4 there; at 65 rows (80 of a tile) 21.6, 34.7, 20.1 and 20.8, 31.8, 18.8.
 // One-term activations stay here: a token tile is 256 rows, its work half of a split's.
 constexpr int PAIR_ROWS = 64;
+// Tiles of at most CUT_COLS columns whose outputs are stored are summed from chains of p.cut
+// stages.
+constexpr int CUT_COLS = 64;
 
 
 // Stream-K partition in 32-bit arithmetic (the host checks units * grid < 2^32).
@@ -187,7 +190,7 @@ __device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
 // workspace path needs 70 more registers, and a CTA that holds them leaves the SM too
 // few for two CTAs of the row kernel that overlaps the launch (SwiGLU: 62 x 256; one
 // kernel for both made the linears 1 % faster and the step 1 % slower).
-template <bool RED>
+template <bool RED, bool CUT>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const __grid_constant__ TcLinearParams p) {
   if (p.skip) {
     // the flag is written by the previous kernel: read it after the dependency wait,
@@ -334,7 +337,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
     uint32_t aphase = 0;
     bool ok = true;
     for (uint32_t u = u_begin; ok && u < u_end;) {
-      const uint32_t seg_end = min(u_end, (u / KB + 1) * KB);
+      uint32_t seg_end = min(u_end, (u / KB + 1) * KB);
+      if (CUT) seg_end = min(seg_end, u + p.cut);
       ok = mbar_wait_warp(&tempty[buf], aphase ^ 1u, abort, p.wait_ns);
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + buf * p.acc_stride;
@@ -399,11 +403,42 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
     uint32_t aphase = 0;
     for (uint32_t u = u_begin; u < u_end;) {
       const int t = static_cast<int>(u / KB);
-      const uint32_t seg_end = min(u_end, static_cast<uint32_t>(t + 1) * KB);
-      u = seg_end;
-      const bool ok = mbar_wait(&tfull[buf], aphase, abort, p.wait_ns);
-      if (bar_any(1, 128, !ok)) break;
-      tc_fence_after();
+      const uint32_t part_end = min(u_end, static_cast<uint32_t>(t + 1) * KB);
+      // RED, and tiles of more than CUT_COLS columns: one chain.  Otherwise the pieces of
+      // the part are summed here, in registers.
+      float sum[CUT_COLS / 16][16];
+      bool ok = true;
+      if constexpr (CUT) {
+#pragma unroll
+        for (int b = 0; b < CUT_COLS / 16; ++b)
+#pragma unroll
+          for (int j = 0; j < 16; ++j) sum[b][j] = 0.f;
+        while (ok && u < part_end) {
+          u = min(part_end, u + p.cut);
+          ok = mbar_wait(&tfull[buf], aphase, abort, p.wait_ns);
+          ok = !bar_any(1, 128, !ok);
+          tc_fence_after();
+          const uint32_t ta = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * p.acc_stride;
+#pragma unroll
+          for (int b = 0; b < CUT_COLS / 16; ++b)
+            if (ok && 16 * b < p.BN) {
+              float v[16];
+              load16(ta + 16 * b, v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) sum[b][j] += v[j];
+            }
+          tc_fence_before();
+          mbar_arrive(&tempty[buf]);
+          buf ^= 1;
+          if (buf == 0) aphase ^= 1u;
+        }
+        if (!ok) break;
+      } else {
+        u = part_end;
+        ok = mbar_wait(&tfull[buf], aphase, abort, p.wait_ns);
+        if (bar_any(1, 128, !ok)) break;
+        tc_fence_after();
+      }
       const int ft = t / p.tok_tiles, tt = t % p.tok_tiles;
       const int m0 = tt * p.BN;
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * p.acc_stride;
@@ -424,24 +459,39 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       const int nparts = c_last - c_first + 1;
       const int f = ft * BM + row;
       if (nparts == 1 || p.epi == EPI_RESID) {
-        for (int c0 = 0; c0 < p.BN; c0 += 16) {
-          float v[16];
-          load16(tbase + c0, v);
-          epi_store16(p, m0 + c0, f, v);
+        if constexpr (CUT) {
+#pragma unroll
+          for (int b = 0; b < CUT_COLS / 16; ++b)
+            if (16 * b < p.BN) epi_store16(p, m0 + 16 * b, f, sum[b]);
+        } else {
+          for (int c0 = 0; c0 < p.BN; c0 += 16) {
+            float v[16];
+            load16(tbase + c0, v);
+            epi_store16(p, m0 + c0, f, v);
+          }
+          tc_fence_before();
+          mbar_arrive(&tempty[buf]);
         }
-        tc_fence_before();
-        mbar_arrive(&tempty[buf]);
       } else {
         const int my_slot = 2 * cta + ((u_begin / KB == static_cast<uint32_t>(t)) ? 0 : 1);
         float* wsp = p.ws + static_cast<size_t>(my_slot) * BM * p.BN;
-        for (int c0 = 0; c0 < p.BN; c0 += 16) {
-          float v[16];
-          load16(tbase + c0, v);
+        if constexpr (CUT) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) __stcg(&wsp[(c0 + j) * BM + row], v[j]);
+          for (int b = 0; b < CUT_COLS / 16; ++b)
+            if (16 * b < p.BN) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) __stcg(&wsp[(16 * b + j) * BM + row], sum[b][j]);
+            }
+        } else {
+          for (int c0 = 0; c0 < p.BN; c0 += 16) {
+            float v[16];
+            load16(tbase + c0, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) __stcg(&wsp[(c0 + j) * BM + row], v[j]);
+          }
+          tc_fence_before();
+          mbar_arrive(&tempty[buf]);
         }
-        tc_fence_before();
-        mbar_arrive(&tempty[buf]);
         __threadfence();
         named_bar(1, 128);
         if (threadIdx.x == 64) {
@@ -488,8 +538,10 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
         }
         named_bar(1, 128);
       }
-      buf ^= 1;
-      if (buf == 0) aphase ^= 1u;
+      if (!CUT) {
+        buf ^= 1;
+        if (buf == 0) aphase ^= 1u;
+      }
     }
   }
 
@@ -582,6 +634,43 @@ size_t tc_ws_floats(int max_bn) {
 int tc_max_tiles() { return MAX_TILES; }
 
 
+// CTAs of a linear that stores its output.  A tile cut between CTAs goes through the
+// workspace, which costs about 5 us and 0.011 us per part and token column; with every SM
+// taking the same number of stages two tiles are cut per CTA, one of them while stages are
+// left.  A stage takes 0.5 us, or what DRAM needs for one of every CTA.  So a tile goes to one CTA, or to as many as pay for themselves.  Equal stages / as
+// chosen here, us: 5 x 1000 x 520 6.2 / 4.8, 16 x 12288 x 4096 22.7 / 19.2, 64 x 1000 x 4096
+// 20.8 / 14.5, 64 x 4096 x 2560 22.1 / 15.7, 64 x 12288 x 4096 30.5 / 23.7.
+// Longer parts are longer chains of tensor-core sums, which round toward zero (2.4e-10 per
+// K: 4.4e-6 at 12288 x 4096).  So the epilogue sums the stages of a part in registers, one by
+// one, or two by two where a term more or the split had made the chains longer than that:
+// 1.3e-7 to 2.5e-7 everywhere, between 1.2e-7 and 2e-5 with equal stages.  That takes a
+// register per token column: wider tiles keep equal stages.
+static int stored_grid(int tiles, int kblocks, int bn, int sms) {
+  auto stages = [](double n, int ctas) { return n * std::max(0.5, 0.005 * ctas); };
+  const long long units = static_cast<long long>(tiles) * kblocks;
+  int best = static_cast<int>(std::min<long long>(units, sms));
+  double least = 1e30;
+  if (best > tiles || tiles > sms) {  // stream-K: parts of unequal size
+    const double n = static_cast<double>(units) / best;
+    least = stages(n, best) + 7.0 - std::min(2.0, 0.1 * n) + 0.011 * bn * (static_cast<double>(best) / tiles + 1);
+  }
+  for (int s = 1; s <= kblocks && static_cast<long long>(tiles) * s <= sms; ++s) {
+    const double t = stages((kblocks + s - 1) / s, tiles * s) + (s > 1 ? 5.0 + 0.011 * bn * s : 0.0);
+    if (t < least) {
+      least = t;
+      best = tiles * s;
+    }
+  }
+  for (int w = 2; w <= 8; ++w) {  // more tiles than SMs: w whole ones each, when that divides
+    const double t = tiles % w == 0 && tiles / w <= sms ? stages(static_cast<double>(w) * kblocks, tiles / w) : 1e30;
+    if (t < least) {
+      least = t;
+      best = tiles / w;
+    }
+  }
+  return best;
+}
+
 int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const void* X_lo, int ldx,
                    const void* W, void* Y, void* Y_lo, int ldy, int epi, int out_f32, float* ws,
                    int* counters, int* err, char* msg, size_t msg_len, const void* W2, int N2,
@@ -647,6 +736,8 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   if (X_lo && encode_2d_bf16(&p.tmB2, X_lo, K, M, ldx, ATOM, p.BN) != 0) return fail("tensor map of X_lo");
   const int sms = tc_num_sms() * CTAS_PER_SM;
   plan->grid = static_cast<int>(p.units < sms ? p.units : sms);
+  p.cut = p.has_lo || p.units >= 2ll * sms ? 2 : 1;
+  if (epi != EPI_RESID && p.BN <= CUT_COLS) plan->grid = stored_grid(p.feat_tiles * p.tok_tiles, p.kblocks, p.BN, sms);
   // float4 reductions need 16-byte aligned rows of Y and whole float4 runs of features
   p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && N % 4 == 0) ? 1 : 0;
   plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 32 * RED_PITCH * sizeof(float);
@@ -680,17 +771,17 @@ cudaError_t tc_linear_launch(const TcLinearPlan& plan, cudaStream_t s) {
   {
     std::lock_guard<std::mutex> lk(g_attr_mu);
     if (!g_attr_set[dev]) {
-      e = cudaFuncSetAttribute(tc_linear_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_linear_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e != cudaSuccess) return e;
+      for (auto k : {tc_linear_kernel<true, false>, tc_linear_kernel<false, true>, tc_linear_kernel<false, false>}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+      }
       g_attr_set[dev] = true;
     }
   }
-  if (plan.p.vec_red)
-    launch_pdl(tc_linear_kernel<true>, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
-  else
-    launch_pdl(tc_linear_kernel<false>, dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
+  launch_pdl(plan.p.vec_red             ? tc_linear_kernel<true, false>
+             : plan.p.BN <= CUT_COLS ? tc_linear_kernel<false, true>
+                                     : tc_linear_kernel<false, false>,
+             dim3(plan.grid), dim3(THREADS), plan.smem, s, plan.p);
   return cudaGetLastError();
 }
 
