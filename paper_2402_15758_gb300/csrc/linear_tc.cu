@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
           for (int j = 0; j < 16; ++j) sum[b][j] = 0.f;
         while (ok && u < part_end) {
           u = min(part_end, u + p.cut);
-          ok = mbar_wait(&tfull[buf], aphase, abort, p.wait_ns);
+          ok = mbar_wait_brief(&tfull[buf], aphase, abort, p.wait_ns);
           ok = !bar_any(1, 128, !ok);
           tc_fence_after();
           const uint32_t ta = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * p.acc_stride;
