@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   // memory from the projections (no round trip through the pool); the committed rows
   // are tiles of the pool.  The local tile is the last of the split's virtual tiles
   // (so it goes to the CTA with the fewest committed tiles) and that CTA's first tile
-  // (stage 0, free at start).  Otherwise the tiles cover slots [0, nctx + n_local).
+  // (its slots are free at start).  Otherwise the tiles cover slots [0, nctx + n_local).
   const bool lmode = p.qkv != nullptr && p.q_local0 == 0;
   // tiles of the pool (a block of prompt rows past its sequence's last row has none)
   const int ntiles = lmode              ? (nctx + KT - 1) / KT
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   // the P tiles' rows are all rewritten every tile; nothing else to clear
 
   // ---- local mode: the owner of the local tile rotates k, writes k and v of the fresh
-  // rows to the pool (for later steps) and into its stage-0 K and V tiles; rows past the
+  // rows to the pool (for later steps) and into the slots of its first K and V tile; rows past the
   // fresh ones are zero there ----
   if (hl) {
     for (int it = threadIdx.x; it < KT * 16; it += THREADS) {
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           }
         }
       }
-      // stage 0: row i, dims j .. j + 3 (half 0) and 64 + j .. (half 1): half of chunk j / 8
+      // row i, dims j .. j + 3 (half 0) and 64 + j .. (half 1): half of chunk j / 8
       const uint32_t o0 = (i >> 3) * ROW_STRIDE + swz(i & 7, j >> 3) + ((j & 7) << 1);
       const uint32_t o1 = GROUP + o0;
       uint8_t* kt = ring + k_pos(0) * HALF_BYTES;

@@ -15,11 +15,12 @@
 //
 // Work split: stream-K.  The (feature tile, token tile, K block) units are cut into
 // gridDim.x equal contiguous ranges (one persistent CTA per SM), so every SM streams
-// the same number of weight bytes whatever the matrix shape.  A tile whose K range
-// spans several CTAs is finished by the last CTA to arrive (an atomic counter per
-// tile): every contributor writes its fp32 partial to a workspace slot, and the last
-// one sums the partials in contributor order (deterministic) and runs the epilogue.
-// No CTA ever waits on another.
+// the same number of weight bytes whatever the matrix shape.  Accumulating outputs add
+// their part of a tile with reductions.  A stored tile whose K range spans several CTAs
+// is finished by the last CTA to arrive (an atomic counter per tile): every contributor
+// writes its fp32 partial to a workspace slot, and the last one sums the partials in
+// contributor order (deterministic) and runs the epilogue; stored_grid() below chooses
+// ranges that cut few tiles.  No CTA ever waits on another.
 //
 // Roles (192 threads): warp 0 issues TMA loads into an n-stage shared-memory ring,
 // warp 1 issues tcgen05.mma into one of two TMEM accumulators, warps 2..5 drain the
@@ -66,9 +67,7 @@ constexpr int MAX_TILES = 8192;
 // here, 20.6, 31.3, 18.4 there; at 65 rows (80 of a tile) 21.6, 34.7, 20.1 and 20.8, 31.8, 18.8.
 // One-term activations stay here: a token tile is 256 rows, its work half of a split's.
 constexpr int PAIR_ROWS = 64;
-// Tiles of at most CUT_COLS columns whose outputs are stored are summed from chains of p.cut
-// stages.
-constexpr int CUT_COLS = 64;
+constexpr int CUT_COLS = 64;  // token columns that the CUT variant holds in registers
 
 
 // Stream-K partition in 32-bit arithmetic (the host checks units * grid < 2^32).
@@ -77,8 +76,7 @@ __device__ __forceinline__ int cta_of_unit(uint32_t u, uint32_t U, uint32_t G) {
 }
 __device__ __forceinline__ uint32_t unit_begin(uint32_t c, uint32_t U, uint32_t G) { return c * U / G; }
 
-// Epilogue of 16 consecutive token columns (m0 .. m0+15) of feature row f.  All
-// loads are issued before the stores so they overlap.
+// Epilogue of 16 consecutive token columns (m0 .. m0+15) of feature row f.
 __device__ __forceinline__ void epi_store16(const TcLinearParams& p, int m0, int f, const float (&v)[16]) {
   if (f >= p.N) return;
   if (p.epi == EPI_RESID) {
@@ -190,6 +188,8 @@ __device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
 // workspace path needs 70 more registers, and a CTA that holds them leaves the SM too
 // few for two CTAs of the row kernel that overlaps the launch (SwiGLU: 62 x 256; one
 // kernel for both made the linears 1 % faster and the step 1 % slower).
+// CUT: stored tiles of at most CUT_COLS columns, summed in registers from chains of p.cut
+// stages (see stored_grid); wider ones, and unaligned accumulation, drain one chain.
 template <bool RED, bool CUT>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const __grid_constant__ TcLinearParams p) {
   if (p.skip) {
