@@ -277,7 +277,8 @@ chimera_status chimera_debug_read_kv(chimera_ctx* ctx, int layer, int seq, int p
  * dtype 1: X, X_lo (optional, NULL = none), W bf16 (K, ldx multiples of 8; 16-byte
  * aligned), tcgen05 kernel; dtype 0: everything fp32, X_lo ignored.  epi 0: Y = acc,
  * 1: Y = SiLU(acc), 2: Y(fp32) += acc.  out_f32 selects an fp32 Y for epi 0/1 with
- * dtype 1.  Device pointers.  Uses a workspace per device, allocated on the first call
+ * dtype 1.  Device pointers; X and W may be written by earlier work on the same stream,
+ * calls of this function among it.  Uses a workspace per device, allocated on the first call
  * made with that device current.  Asynchronous: the status covers the arguments and
  * the launch; what the kernel flags on the device (a bounded wait that gave up) is
  * reported by chimera_op_sync. */

@@ -277,6 +277,13 @@ __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorM
       : "memory");
 }
 
+// Request of a tile into L2 alone: no copy that a later write could leave stale.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0),
+               "r"(c1)
+               : "memory");
+}
+
 // Reductions into global memory that return nothing (red, not atom): the issuing thread
 // never waits for them.
 __device__ __forceinline__ void red_add_f32(float* addr, float v) {

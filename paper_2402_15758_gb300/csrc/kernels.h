@@ -36,6 +36,8 @@ struct TcLinearParams {
   int* err;          // device error word
   unsigned long long wait_ns;  // limit of every bounded wait of the launch (ns)
   const int* skip;   // optional device flag: nonzero at run time -> the launch does nothing
+  int early_w;       // 1: no kernel of the stream writes the weights, so they may be read
+                     // before the dependency wait (a context's; 0 unless the caller sets it)
   uint32_t tmem_cols;
   uint32_t acc_stride;  // TMEM column distance between the two accumulators
   // optional: [zero, zero + zero_floats) cleared by the epilogue warps after the
@@ -63,6 +65,7 @@ struct TcPairParams {
   int* err;
   unsigned long long wait_ns;
   const int* skip;
+  int early_w;            // as in TcLinearParams
   float* zero;
   long long zero_floats;
 };

@@ -1,8 +1,11 @@
 // Kernel launches with programmatic stream serialization: a kernel may begin launching
 // while its predecessor in the stream drains.  Every kernel calls pdl_wait() before it
-// touches memory written by earlier kernels, with one exception: the tensor-core tree
+// reads memory that earlier kernels write, with one exception: the tensor-core tree
 // attention with prewait_kv set reads n_ctx, the page table and committed KV rows
-// before its wait.  That is correct only because the launch directly before it is a
+// before its wait.  (A context's linears also read their weights before the wait, which no
+// kernel of its stream writes; the stateless entry points' weights may be the output of
+// the launch before, so these only request them into L2.)
+// The attention's early reads are correct only because the launch directly before it is a
 // tensor-core linear, which lets dependents launch only after its own pdl_wait (so
 // every earlier kernel is complete); the row kernels trigger before they wait, and the
 // runtime refuses to enqueue such an attention after anything but a tensor-core

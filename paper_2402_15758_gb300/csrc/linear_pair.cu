@@ -200,11 +200,22 @@ __device__ __forceinline__ void produce(const TcPairParams& p, int lane, uint32_
     const CUtensorMap* bmap = rank ? &p.tmB2 : &p.tmB;
     int sa = 0, sb = 0;
     uint32_t pa = 0, pb = 0;
-    auto load_a = [&](uint32_t u) {
-      const int half = w.ft(p, u) * 2 + static_cast<int>(rank), k = static_cast<int>(u % w.KB) * BK;
+    auto weight_tile = [&](uint32_t u, int& k, int& row) {
+      const int half = w.ft(p, u) * 2 + static_cast<int>(rank);
       const bool second = half >= p.half_split;
-      const CUtensorMap* map = second ? &p.tmA2 : &p.tmA;
-      const int row = (second ? half - p.half_split : half) * BM;
+      k = static_cast<int>(u % w.KB) * BK;
+      row = (second ? half - p.half_split : half) * BM;
+      return second ? &p.tmA2 : &p.tmA;
+    };
+    auto prefetch_a = [&](uint32_t u) {
+      int k, row;
+      const CUtensorMap* map = weight_tile(u, k, row);
+#pragma unroll
+      for (int a = 0; a < BKA; ++a) tma_prefetch_2d(map, k + a * ATOM, row);
+    };
+    auto load_a = [&](uint32_t u) {
+      int k, row;
+      const CUtensorMap* map = weight_tile(u, k, row);
       const uint32_t bar = dsmem_addr(smem_u32(&c->full_a[sa]), 0);
       if (!rank) mbar_arrive_expect_tx(&c->full_a[sa], static_cast<uint32_t>(2 * A_BYTES));
 #pragma unroll
@@ -235,12 +246,17 @@ __device__ __forceinline__ void produce(const TcPairParams& p, int lane, uint32_
         pb ^= 1u;
       }
     };
-    // the weights do not depend on earlier kernels: the first two units' (as in
-    // linear_tc.cu) are requested before the dependency wait
+    // the first two units' weights are requested before the dependency wait (as in
+    // linear_tc.cu), into L2 alone when an earlier kernel may still be writing them
     uint32_t ua = w.begin;
-    for (; ua < min(w.begin + 2, w.end); ++ua) load_a(ua);
+    const uint32_t pre = min(w.begin + 2, w.end);
+    if (p.early_w)
+      for (; ua < pre; ++ua) load_a(ua);
+    else
+      for (uint32_t u = ua; u < pre; ++u) prefetch_a(u);
     pdl_wait();
     pdl_trigger();
+    for (; ua < pre; ++ua) load_a(ua);
     bool ok = true;
     for (uint32_t u = w.begin; ok && u < w.end && !*abort; ++u) {
       if (u == ua) {

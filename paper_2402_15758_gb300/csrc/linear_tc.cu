@@ -266,14 +266,19 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued_mask = 0, issued_par = 0;
-      auto load_a = [&](uint32_t u, uint8_t* sa, uint64_t* bar) {
+      auto load_a = [&](uint32_t u, uint8_t* sa, uint64_t* bar, bool to_l2 = false) {
         const int t = static_cast<int>(u / KB), kb = static_cast<int>(u % KB);
         const int ft = t / p.tok_tiles;
         const bool second = ft >= p.ft_split;
         const CUtensorMap* map = second ? &p.tmA2 : &p.tmA;
         const int row = (second ? ft - p.ft_split : ft) * BM;
 #pragma unroll
-        for (int a = 0; a < BKA; ++a) tma_load_2d_hint(sa + a * a_atom, map, kb * BK + a * ATOM, row, bar, pol_w);
+        for (int a = 0; a < BKA; ++a) {
+          if (to_l2)
+            tma_prefetch_2d(map, kb * BK + a * ATOM, row);
+          else
+            tma_load_2d_hint(sa + a * a_atom, map, kb * BK + a * ATOM, row, bar, pol_w);
+        }
       };
       auto load_b = [&](uint32_t u, uint8_t* sb, uint64_t* bar) {
         const int t = static_cast<int>(u / KB), kb = static_cast<int>(u % KB);
@@ -289,15 +294,18 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       // stages, not the whole ring: the row kernel that usually runs meanwhile reads its
       // input from L2 behind these requests (measured: 1 stage 4.45, 2 stages 4.40, 3
       // stages 4.42 ms per 7B step).
+      // Weights that an earlier kernel of the stream may still be writing (early_w 0) are only
+      // requested into L2, which keeps no stale copy, and read after the wait (64 x 22016 x
+      // 4096 31.3 us either way, 256 x 4096 x 11008 36.1 -> 36.5).
       const uint32_t npre = min(static_cast<uint32_t>(min(p.stages, CHIMERA_LIN_PRE_STAGES)), u_end - u_begin);
       for (uint32_t i = 0; i < npre; ++i) {
-        uint8_t* sa = smem + i * stage_bytes;
         mbar_arrive_expect_tx(&full[i], static_cast<uint32_t>(stage_bytes));
-        load_a(u_begin + i, sa, &full[i]);
+        load_a(u_begin + i, smem + i * stage_bytes, &full[i], !p.early_w);
         issued_mask |= 1u << i;
       }
       pdl_wait();
       pdl_trigger();
+      for (uint32_t i = 0; i < npre && !p.early_w; ++i) load_a(u_begin + i, smem + i * stage_bytes, &full[i]);
       for (uint32_t i = 0; i < npre; ++i) load_b(u_begin + i, smem + i * stage_bytes + a_atom * BKA, &full[i]);
       stage = static_cast<int>(npre % p.stages);
       phase = (npre == static_cast<uint32_t>(p.stages)) ? 1u : 0u;

@@ -382,6 +382,7 @@ bool make_lin(chimera_ctx* ctx, Lin* l, int M, int N, int K, const void* X, cons
   }
   l->tp.p.wait_ns = l->tp.pair.p.wait_ns = kDefaultWaitNs;  // the timeout hook applies to the stateless entry points only
   l->tp.p.skip = l->tp.pair.p.skip = skip;
+  l->tp.p.early_w = l->tp.pair.p.early_w = 1;  // the weights do not change while the context lives
   return true;
 }
 

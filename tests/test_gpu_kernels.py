@@ -129,6 +129,29 @@ def test_linear_pair_kernel(M, N, K, epi, out_f32):
         assert np.array_equal(got[0], got[1])
 
 
+# W written by the launch just before on the stream: 16 rows and 64 rows (linear_tc.cu), 100 rows
+# (the CTA-pair kernel), and the allocation-free entry point
+@pytest.mark.parametrize("M,split,noalloc", [(16, False, False), (64, True, False), (100, True, False), (16, True, True)])
+def test_linear_weights_from_the_launch_before(M, split, noalloc):
+    g = torch.Generator().manual_seed(M)
+    D = 4096
+    A = torch.randn(D, 2048, generator=g).to(torch.bfloat16).cuda()
+    B = (torch.randn(D, 2048, generator=g) * 0.02).to(torch.bfloat16).cuda()
+    X32 = torch.randn(M, D, generator=g)
+    hi = X32.to(torch.bfloat16).cuda()
+    lo = (X32 - hi.cpu().float()).to(torch.bfloat16).cuda() if split else None
+    op = pkg.op_linear_noalloc if noalloc else pkg.op_linear
+    for _ in range(3):
+        W = torch.full((D, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        Y = torch.empty(M, D, device="cuda")
+        pkg.op_linear(A, B, W, epi=0)
+        op(hi, W, Y, epi=0, out_f32=True, X_lo=lo)
+        pkg.op_sync()
+        ref = (hi.double() + (lo.double() if split else 0.0)) @ W.double().T
+        # fp32 sums of 4096 products, truncated at most every 16 K: 256 * 2^-23 at most
+        assert _rel_rows(Y.cpu().numpy(), ref.cpu().numpy()) <= 3e-5
+
+
 def test_linear_deterministic():
     g = torch.Generator().manual_seed(5)
     X = torch.randn(64, 4096, generator=g).to(torch.bfloat16).cuda()
