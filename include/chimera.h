@@ -278,10 +278,13 @@ chimera_status chimera_debug_read_kv(chimera_ctx* ctx, int layer, int seq, int p
  * aligned), tcgen05 kernel; dtype 0: everything fp32, X_lo ignored.  epi 0: Y = acc,
  * 1: Y = SiLU(acc), 2: Y(fp32) += acc.  out_f32 selects an fp32 Y for epi 0/1 with
  * dtype 1.  Device pointers; X and W may be written by earlier work on the same stream,
- * calls of this function among it.  Uses a workspace per device, allocated on the first call
- * made with that device current.  Asynchronous: the status covers the arguments and
- * the launch; what the kernel flags on the device (a bounded wait that gave up) is
- * reported by chimera_op_sync. */
+ * calls of this function among it.  Calls on different streams may overlap: each of the
+ * first eight streams of a device has a workspace of its own (107 MB, allocated on its first
+ * call and kept), further streams share one and their calls run one after the other.
+ * Calls captured into graphs share one more: replays that overlap on the GPU must be ordered
+ * by the caller.  The same holds for chimera_op_attention.  Asynchronous: the status
+ * covers the arguments and the launch; what the kernel flags on the device (a bounded wait
+ * that gave up) is reported by chimera_op_sync. */
 chimera_status chimera_op_linear(int dtype, int epi, int out_f32, int M, int N, int K,
                                  const void* X, const void* X_lo, int ldx, const void* W, void* Y,
                                  int ldy, void* cuda_stream);

@@ -1926,51 +1926,87 @@ chimera_status chimera_debug_read_kv(chimera_ctx* ctx, int layer, int seq, int p
 // stateless kernel-level entry points
 // ---------------------------------------------------------------------------
 namespace {
-// Scratch of the stateless entry points, one set per device (allocated on the first
-// call made with that device current and kept until exit).
+// Scratch of the stateless entry points.  Two launches that run at the same time must not
+// share a set (partial tiles, arrival counters), so each stream of a device has its own, up
+// to OP_STREAM_SETS of them; the streams after those share one, and each of their calls
+// waits on the device for the one before.  Calls under capture take a set that no eager call
+// uses (the graph may be replayed at any time).  107 MB a set, allocated when a stream first needs
+// one and kept until exit.
 struct OpScratch {
   bool ready = false;
+  unsigned long long stream = 0;  // cudaStreamGetId of the owner (never reused, unlike handles)
   float* lin_ws = nullptr;
   int* lin_cnt = nullptr;
   int* err = nullptr;
   float* att_ws = nullptr;
-  size_t att_floats = 0;
   int* att_cnt = nullptr;
+  cudaEvent_t done = nullptr;  // the shared set: the end of its last call
 };
 constexpr int OP_MAX_DEVICES = 64;
+constexpr int OP_STREAM_SETS = 8;
+constexpr int OP_SHARED = OP_STREAM_SETS, OP_CAPTURED = OP_STREAM_SETS + 1, OP_SETS = OP_STREAM_SETS + 2;
 constexpr int OP_ATT_COUNTERS = 64 * 256;
+constexpr size_t OP_ATT_FLOATS = static_cast<size_t>(16) << 20;
 std::mutex g_op_mu;
-OpScratch g_op_dev[OP_MAX_DEVICES];
+OpScratch g_op_dev[OP_MAX_DEVICES][OP_SETS];
 
-// The current device's scratch (nullptr on failure).  Caller holds g_op_mu.
-OpScratch* op_scratch() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= OP_MAX_DEVICES) return nullptr;
-  OpScratch& s = g_op_dev[dev];
-  if (s.ready) return &s;
+bool op_alloc(OpScratch* out, bool shared) {
+  // this stream, or another thread's, may be capturing: allocations are no part of a graph
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
   OpScratch n;
-  n.att_floats = static_cast<size_t>(16) << 20;
-  bool ok = cudaMalloc(&n.lin_ws, tc_ws_floats(256) * sizeof(float)) == cudaSuccess;
+  cudaStream_t zs = nullptr;
+  bool ok = cudaStreamCreateWithFlags(&zs, cudaStreamNonBlocking) == cudaSuccess;
+  ok = ok && cudaMalloc(&n.lin_ws, tc_ws_floats(256) * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&n.lin_cnt, tc_max_tiles() * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMalloc(&n.err, sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMalloc(&n.att_ws, n.att_floats * sizeof(float)) == cudaSuccess;
+  ok = ok && cudaMalloc(&n.att_ws, OP_ATT_FLOATS * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&n.att_cnt, OP_ATT_COUNTERS * sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMemset(n.lin_cnt, 0, tc_max_tiles() * sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMemset(n.err, 0, sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMemset(n.att_cnt, 0, OP_ATT_COUNTERS * sizeof(int)) == cudaSuccess;
-  ok = ok && cudaDeviceSynchronize() == cudaSuccess;
+  ok = ok && (!shared || cudaEventCreateWithFlags(&n.done, cudaEventDisableTiming) == cudaSuccess);
+  ok = ok && cudaMemsetAsync(n.lin_cnt, 0, tc_max_tiles() * sizeof(int), zs) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(n.err, 0, sizeof(int), zs) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(n.att_cnt, 0, OP_ATT_COUNTERS * sizeof(int), zs) == cudaSuccess;
+  ok = ok && cudaStreamSynchronize(zs) == cudaSuccess;
   if (!ok) {
     cudaFree(n.lin_ws);
     cudaFree(n.lin_cnt);
     cudaFree(n.err);
     cudaFree(n.att_ws);
     cudaFree(n.att_cnt);
-    return nullptr;
+    if (n.done) cudaEventDestroy(n.done);
+    cudaGetLastError();
   }
-  n.ready = true;
-  s = n;
-  return &s;
+  if (zs) cudaStreamDestroy(zs);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  n.ready = ok;
+  if (ok) *out = n;
+  return ok;
 }
+
+// The set for a call on stream s (nullptr on failure); op_done(set, s) follows the launch.
+// Caller holds g_op_mu.
+OpScratch* op_scratch(cudaStream_t s) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= OP_MAX_DEVICES) return nullptr;
+  OpScratch* sets = g_op_dev[dev];
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long id = ~0ull;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+    return sets[OP_CAPTURED].ready || op_alloc(&sets[OP_CAPTURED], false) ? &sets[OP_CAPTURED] : nullptr;
+  cudaStreamGetId(s, &id);
+  cudaGetLastError();  // (an unusable stream: the launch reports it)
+  for (int i = 0; i < OP_STREAM_SETS; ++i) {
+    if (sets[i].ready && sets[i].stream == id) return &sets[i];
+    if (sets[i].ready) continue;
+    if (!op_alloc(&sets[i], false)) break;
+    sets[i].stream = id;
+    return &sets[i];
+  }
+  OpScratch& sh = sets[OP_SHARED];
+  if (!sh.ready && !op_alloc(&sh, true)) return nullptr;
+  return cudaStreamWaitEvent(s, sh.done, 0) == cudaSuccess ? &sh : nullptr;
+}
+bool op_done(const OpScratch* sc, cudaStream_t s) { return !sc->done || cudaEventRecord(sc->done, s) == cudaSuccess; }
 }  // namespace
 
 chimera_status chimera_op_linear(int dtype, int epi, int out_f32, int M, int N, int K, const void* X,
@@ -1984,14 +2020,15 @@ chimera_status chimera_op_linear(int dtype, int epi, int out_f32, int M, int N, 
                              ? CHIMERA_OK
                              : CHIMERA_ECUDA;
   std::lock_guard<std::mutex> lk(g_op_mu);
-  OpScratch* sc = op_scratch();
+  OpScratch* sc = op_scratch(s);
   if (!sc) return CHIMERA_ENOMEM;
   TcLinearPlan plan;
   char msg[256];
   if (tc_linear_plan(&plan, M, N, K, X, X_lo, ldx, W, Y, nullptr, ldy, epi, epi == EPI_RESID ? 1 : out_f32, sc->lin_ws,
                      sc->lin_cnt, sc->err, msg, sizeof(msg)) != 0)
     return CHIMERA_EINVAL;
-  return tc_linear_launch(plan, s) == cudaSuccess ? CHIMERA_OK : CHIMERA_ECUDA;
+  const cudaError_t e = tc_linear_launch(plan, s);
+  return op_done(sc, s) && e == cudaSuccess ? CHIMERA_OK : CHIMERA_ECUDA;
 }
 
 chimera_status chimera_op_attention(int dtype, int kv_split, int batch, int n_heads, int head_dim, int nq, int q_local0,
@@ -2003,8 +2040,10 @@ chimera_status chimera_op_attention(int dtype, int kv_split, int batch, int n_he
       splits < 1 || splits > 16 || (dtype == 1 && head_dim == 128 && splits > 8) || batch * n_heads > 64 * 256 ||
       n_blocks < 1)
     return CHIMERA_EINVAL;
+  if (attn_ws_floats(batch, n_heads, splits, nq, head_dim) > OP_ATT_FLOATS) return CHIMERA_EINVAL;
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   std::lock_guard<std::mutex> lk(g_op_mu);
-  OpScratch* sc = op_scratch();
+  OpScratch* sc = op_scratch(s);
   if (!sc) return CHIMERA_ENOMEM;
   AttnParams p{};
   p.q = q;
@@ -2032,10 +2071,8 @@ chimera_status chimera_op_attention(int dtype, int kv_split, int batch, int n_he
   p.counters = sc->att_cnt;
   p.err = sc->err;
   p.nq_max = nq;
-  if (attn_ws_floats(batch, n_heads, splits, nq, head_dim) > sc->att_floats) return CHIMERA_EINVAL;
-  return attention(p, dtype, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
-             ? CHIMERA_OK
-             : CHIMERA_ECUDA;
+  const cudaError_t e = attention(p, dtype, s);
+  return op_done(sc, s) && e == cudaSuccess ? CHIMERA_OK : CHIMERA_ECUDA;
 }
 
 chimera_status chimera_op_sync(void* cuda_stream) {
@@ -2046,13 +2083,14 @@ chimera_status chimera_op_sync(void* cuda_stream) {
     std::lock_guard<std::mutex> lk(g_op_mu);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= OP_MAX_DEVICES) return CHIMERA_ECUDA;
-    OpScratch& sc = g_op_dev[dev];
-    if (sc.ready) {
+    for (const OpScratch& sc : g_op_dev[dev]) {
+      if (!sc.ready) continue;
       int e = 0;
       if (cudaMemcpy(&e, sc.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return CHIMERA_ECUDA;
       if (e) {
-        // a launch that gave up can leave split-K or split-merge counters raised
-        if (cudaMemset(sc.err, 0, sizeof(int)) != cudaSuccess ||
+        // a launch that gave up can leave split-K or split-merge counters raised; the set may be
+        // another stream's, with calls still running
+        if (cudaDeviceSynchronize() != cudaSuccess || cudaMemset(sc.err, 0, sizeof(int)) != cudaSuccess ||
             cudaMemset(sc.lin_cnt, 0, tc_max_tiles() * sizeof(int)) != cudaSuccess ||
             cudaMemset(sc.att_cnt, 0, OP_ATT_COUNTERS * sizeof(int)) != cudaSuccess ||
             cudaDeviceSynchronize() != cudaSuccess)

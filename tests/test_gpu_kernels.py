@@ -152,6 +152,50 @@ def test_linear_weights_from_the_launch_before(M, split, noalloc):
         assert _rel_rows(Y.cpu().numpy(), ref.cpu().numpy()) <= 3e-5
 
 
+# launches that overlap: tiles cut between CTAs (fp32 output, summed in a fixed order) and a
+# split fp32 attention, on more streams than have a workspace of their own, beside a graph
+# captured on a stream without an earlier call
+@pytest.mark.parametrize("n_streams", [2, 11])
+def test_ops_on_several_streams(n_streams):
+    g = torch.Generator().manual_seed(8)
+    X = torch.randn(5, 9000, generator=g).to(torch.bfloat16).cuda()
+    W = (torch.randn(300, 9000, generator=g) * 0.02).to(torch.bfloat16).cuda()
+    kv = torch.randn(70, 2, 2, 16, 64, generator=g).cuda()
+    q = torch.randn(1, 128, generator=g).cuda()
+    pages = torch.arange(70, dtype=torch.int32, device="cuda").view(1, 70)
+    n_ctx = torch.tensor([1100], dtype=torch.int32, device="cuda")
+    anc = torch.ones(1, dtype=torch.int64, device="cuda")
+
+    def call(y, o, stream):
+        pkg.op_linear(X, W, y, epi=0, out_f32=True, stream=stream)
+        pkg.op_attention(q, kv, pages, n_ctx, anc, o, 1, 0, 1, 1, 2, 64, splits=4, stream=stream)
+
+    outs = [(torch.zeros(5, 300, device="cuda"), torch.zeros(1, 128, device="cuda")) for _ in range(n_streams + 2)]
+    call(*outs[0], None)
+    graph = torch.cuda.CUDAGraph()
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        call(*outs[1], torch.cuda.current_stream())
+        call(*outs[2], streams[0])  # an eager call beside the capture
+    ref = tuple(t.clone() for t in outs[0])
+    assert _rel_rows(ref[0].cpu().numpy(), (X.double() @ W.double().T).cpu().numpy()) <= 2e-6
+    torch.cuda.synchronize()
+    for rep in range(100):
+        for st, out in zip(streams, outs[2:]):
+            call(*out, st)
+        graph.replay()
+        if rep % 10 == 9:
+            torch.cuda.synchronize()
+            for y, o in outs:
+                assert torch.equal(y, ref[0]) and torch.equal(o, ref[1])
+                if rep < 90:
+                    y.zero_(), o.zero_()
+            call(*outs[0], None)
+            torch.cuda.synchronize()
+    pkg.op_sync()
+
+
 def test_linear_deterministic():
     g = torch.Generator().manual_seed(5)
     X = torch.randn(64, 4096, generator=g).to(torch.bfloat16).cuda()
