@@ -224,21 +224,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // The same for a wait that is usually over within the time for which try_wait may suspend a
-// thread: suspended for no longer than the limit, so that a short limit (a test's) is kept.
+// thread (which no hint keeps below a microsecond or so): with a short limit (a test's) the
+// barrier is polled instead, until the limit has passed.
 __device__ __forceinline__ bool mbar_wait_brief(uint64_t* bar, uint32_t parity, volatile int* abort, uint64_t limit_ns) {
-  const uint32_t hint = limit_ns < 1000000ull ? static_cast<uint32_t>(limit_ns) : 1000000u;
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(hint)
-      : "memory");
-  if (ok) return true;
   if (limit_ns >= 1000000ull) return mbar_wait(bar, parity, abort, limit_ns);
-  *abort = 1;
-  return false;
+  const uint64_t t0 = global_timer_ns();
+  while (!mbar_test(bar, parity)) {
+    if (*abort) return false;
+    if (global_timer_ns() - t0 >= limit_ns) {
+      *abort = 1;
+      return false;
+    }
+  }
+  return true;
 }
 
 // The same wait by a whole warp, with one answer for all lanes.

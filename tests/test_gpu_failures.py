@@ -110,3 +110,24 @@ def test_bounded_wait_timeout_is_reported_and_recovered():
         pkg.op_sync()
         got = Y.cpu().double().numpy()
         assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) <= 1e-2
+
+
+# the sums of short chains are waited for within a microsecond or so: a limit of a few ns still
+# runs out, with the weights in L2 too, and one that is longer than the work never does
+@pytest.mark.parametrize("ns,status", [(2, ETIMEDOUT), (900000, 0)])
+def test_short_wait_limit_is_kept(ns, status):
+    g = torch.Generator().manual_seed(6)
+    X = torch.randn(64, 4096, generator=g).to(torch.bfloat16).cuda()
+    W = (torch.randn(4096, 4096, generator=g) * 0.02).to(torch.bfloat16).cuda()
+    Y = torch.zeros(64, 4096, device="cuda")
+    pkg.op_sync()
+    for _ in range(20):
+        try:
+            pkg.set_wait_limit(ns)
+            pkg.op_linear(X, W, Y, epi=0, out_f32=True)
+        finally:
+            pkg.set_wait_limit(0)
+        if status:
+            assert _status(pkg.op_sync) == status
+        else:
+            pkg.op_sync()
