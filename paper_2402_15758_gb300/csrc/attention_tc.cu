@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   uint64_t* o_done = bars + 20;      // count 2: tcgen05.commit of the QK and of the PV warp
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 21);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
+  int* s_next = s_abort + 1;         // ring position after the last one requested
   int* s_pages = s_abort + 2;        // [PAGE_CACHE]
   int* s_lpages = s_pages + PAGE_CACHE;  // [8] pages of the local rows
   volatile int* abort = s_abort;
@@ -586,10 +587,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         prefetch_l2(w + o, static_cast<uint32_t>(min(static_cast<long long>(NEXT_W_CHUNK), p.next_w_bytes - o)));
       __syncwarp();
     }
-    // copies still in flight when the CTA gives up: let them land before it exits
-    if (*abort)
-      for (int j = next_pos - 1; j >= 0 && j >= next_pos - SLOTS; --j)
-        if (wanted(j)) mbar_wait_plain(&full[j % SLOTS], (j / SLOTS) & 1, 200000000ull);
+    if (lane == 0) *s_next = next_pos;
     __syncwarp();
   } else if (warp == QK_WARP || warp == PV_WARP) {
     // ---------------- MMA issuers (a warp for each product, one elected lane issues) ----------------
@@ -801,6 +799,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     __syncwarp();
   }
   __syncthreads();  // this CTA's tiles are idle: every load landed and every MMA completed
+  if (*abort) {     // (but if some wait gave up: copies may still be in flight)
+    if (warp == LOAD_WARP)
+      for (int n = *s_next, j = max(0, n - SLOTS); j < n; ++j)
+        if (wanted(j)) mbar_wait_plain(&full[j % SLOTS], (j / SLOTS) & 1, 200000000ull);
+    __syncthreads();
+  }
   __syncwarp();
   if (S > 1) cluster_arrive();
   const int rpc = (nq + S - 1) / S;

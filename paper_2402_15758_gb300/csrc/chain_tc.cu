@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
   uint64_t* drain = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
+  uint32_t* s_issued = reinterpret_cast<uint32_t*>(s_abort + 1);                   // stages requested
   float* s_sum = reinterpret_cast<float*>(s_abort + 4);                            // [4] norm partials
   float* s_red = reinterpret_cast<float*>(smem + p.stages * stage_bytes + 1024);  // [4][16][33]
 
@@ -268,16 +269,15 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
       if (*abort) {
         // every started stage must land before the CTA exits: request the activation
         // half of the units whose weights are in flight too (in-bounds reads of
-        // whatever the buffer holds), then wait for the last `stages` units
+        // whatever the buffer holds)
         while (xq < wq) {
           issue_x(xq, xg, xu);
           ++xq;
           ++xu;
           norm_cursor(xg, xu);
         }
-        for (uint32_t q = (wq > static_cast<uint32_t>(p.stages) ? wq - p.stages : 0u); q < wq; ++q)
-          mbar_wait_plain(&full[q % p.stages], (q / p.stages) & 1u, 200000000ull);
       }
+      *s_issued = wq;
     } else {
       pdl_wait();
       pdl_trigger();
@@ -323,10 +323,6 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
           buf ^= 1;
           if (buf == 0) aphase ^= 1u;
         }
-      }
-      if (*abort) {
-        tc_commit(drain);
-        mbar_wait_plain(drain, 0, 200000000ull);
       }
     }
   } else {
@@ -463,6 +459,21 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
 
   tc_fence_before();
   __syncthreads();
+  // Some role gave up (whichever: the others may have been done before): the copies in flight
+  // land before the CTA exits, and the MMAs end before tensor memory is released.
+  if (*abort) {
+    if (threadIdx.x == 0) {
+      const uint32_t n = *s_issued;
+      for (uint32_t q = (n > static_cast<uint32_t>(p.stages) ? n - p.stages : 0u); q < n; ++q)
+        mbar_wait_plain(&full[q % p.stages], (q / p.stages) & 1u, 200000000ull);
+    } else if (warp == 1) {
+      if (lane == 0) {
+        tc_commit(drain);
+        mbar_wait_plain(drain, 0, 200000000ull);
+      }
+      __syncwarp();
+    }
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, p.tmem_cols);

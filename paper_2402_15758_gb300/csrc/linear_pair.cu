@@ -155,6 +155,7 @@ struct Ctrl {  // at the start of the aligned dynamic shared memory
   uint64_t tfull[2], tempty[2], drain;
   uint32_t tmem;
   int abort, last;
+  uint32_t issued, issued_par;  // stages requested, their parities; bits 0..: weight tiles, 8..: token tiles
 };
 constexpr int CTRL_BYTES = 1024;
 static_assert(sizeof(Ctrl) <= CTRL_BYTES, "control block");
@@ -196,7 +197,7 @@ __device__ __forceinline__ void produce(const TcPairParams& p, int lane, uint32_
     volatile int* abort = &c->abort;
     // ---------------- TMA producer (each CTA: its features, its rows of B) ----------------
     const uint64_t pol_w = policy_evict_first();
-    uint32_t issued = 0, issued_par = 0;  // bits 0..: weight tiles, bits 8..: token tiles
+    uint32_t issued = 0, issued_par = 0;
     const CUtensorMap* bmap = rank ? &p.tmB2 : &p.tmB;
     int sa = 0, sb = 0;
     uint32_t pa = 0, pb = 0;
@@ -266,21 +267,32 @@ __device__ __forceinline__ void produce(const TcPairParams& p, int lane, uint32_
       ok = ok && mbar_wait(&c->empty_b[sb], pb ^ 1u, abort, p.wait_ns);
       if (ok) load_b(u);
     }
-    // After a timeout copies may still be in flight, and a CTA must not end before its
-    // own have landed.  They signal CTA 0's barriers, which CTA 1 cannot wait on and
-    // which stay short of bytes when only one CTA requested a stage: CTA 0 waits for
-    // its stages within a limit, and both let 10 ms pass (a copy takes microseconds).
-    if (*abort) {
-      if (!rank)
-        for (int i = 0; i < 8 + p.b_stages; ++i)
-          if (issued >> i & 1u)
-            mbar_wait_plain(i < 8 ? &c->full_a[i] : &c->full_b[i - 8], issued_par >> i & 1u, 20000000ull);
-      for (const uint64_t t0 = global_timer_ns(); global_timer_ns() - t0 < 10000000ull;) {
-      }
-    }
+    c->issued = issued;
+    c->issued_par = issued_par;
   } else {
     pdl_wait();
     pdl_trigger();
+  }
+}
+
+// Some role gave up (whichever: the others may have been done before).  A CTA must not end
+// before its copies have landed.  They signal CTA 0's barriers, which CTA 1 cannot wait on and
+// which stay short of bytes when only one CTA requested a stage: CTA 0 waits for its stages
+// within a limit, and both let 10 ms pass (a copy takes microseconds).  The MMAs end before
+// tensor memory is released.
+__device__ __forceinline__ void settle(const TcPairParams& p) {
+  Ctrl* c = reinterpret_cast<Ctrl*>(smem_base());
+  const uint32_t rank = cluster_rank();
+  if (threadIdx.x == 0) {
+    if (!rank)
+      for (int i = 0; i < 8 + p.b_stages; ++i)
+        if (c->issued >> i & 1u)
+          mbar_wait_plain(i < 8 ? &c->full_a[i] : &c->full_b[i - 8], c->issued_par >> i & 1u, 20000000ull);
+    for (const uint64_t t0 = global_timer_ns(); global_timer_ns() - t0 < 10000000ull;) {
+    }
+  } else if (threadIdx.x >> 5 == 1 && !rank) {
+    tc_commit_pair(&c->drain, elect_one());  // (the lane that issued them: the election is deterministic)
+    mbar_wait_plain(&c->drain, 0, 200000000ull);
   }
 }
 
@@ -340,10 +352,6 @@ __device__ __forceinline__ void multiply(const TcPairParams& p, uint32_t rank) {
       if (ok) tc_commit_pair(&c->tfull[buf], elected);
       buf ^= 1;
       if (buf == 0) aphase ^= 1u;
-    }
-    if (!ok) {  // every MMA issued so far must complete before tensor memory is released
-      tc_commit_pair(&c->drain, elected);
-      mbar_wait_plain(&c->drain, 0, 200000000ull);
     }
   }
   __syncwarp();
@@ -582,6 +590,7 @@ __global__ void __launch_bounds__(THREADS, 1) __cluster_dims__(2, 1, 1)
 
   tc_fence_before();
   __syncthreads();
+  if (*const_cast<volatile int*>(&c->abort)) settle(p);
   __syncwarp();
   cluster_sync();  // both CTAs are done with each other's shared and tensor memory
   if (warp == 1) {

@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   int* s_abort = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_last = s_abort + 1;
+  uint32_t* s_issued = reinterpret_cast<uint32_t*>(s_last + 1);  // [2] stages requested, their parities
   float* s_red = reinterpret_cast<float*>(smem + p.stages * stage_bytes + 1024);  // [4 warps][32][RED_PITCH]
 
   const int warp = threadIdx.x >> 5;
@@ -322,11 +323,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
           phase ^= 1u;
         }
       }
-      if (*abort) {
-        // let copies that are still in flight land before the CTA exits
-        for (int s = 0; s < p.stages; ++s)
-          if (issued_mask >> s & 1u) mbar_wait_plain(&full[s], issued_par >> s & 1u, 200000000ull);
-      }
+      s_issued[0] = issued_mask;
+      s_issued[1] = issued_par;
     } else {
       pdl_wait();
       pdl_trigger();
@@ -375,11 +373,6 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
       if (ok) tc_commit(&tfull[buf], elected);
       buf ^= 1;
       if (buf == 0) aphase ^= 1u;
-    }
-    if (!ok) {
-      // every MMA issued so far must complete before TMEM is released
-      tc_commit(drain, elected);
-      mbar_wait_plain(drain, 0, 200000000ull);
     }
     __syncwarp();
   } else {
@@ -555,6 +548,18 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const _
 
   tc_fence_before();
   __syncthreads();
+  // Some role gave up (whichever: the others may have been done before): the copies in flight
+  // land before the CTA exits, and the MMAs end before tensor memory is released.
+  if (*abort) {
+    if (threadIdx.x == 0) {
+      for (int s = 0; s < p.stages; ++s)
+        if (s_issued[0] >> s & 1u) mbar_wait_plain(&full[s], s_issued[1] >> s & 1u, 200000000ull);
+    } else if (warp == 1) {
+      tc_commit(drain, elect_one());  // (the lane that issued them: the election is deterministic)
+      mbar_wait_plain(drain, 0, 200000000ull);
+      __syncwarp();
+    }
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, p.tmem_cols);

@@ -131,3 +131,29 @@ def test_short_wait_limit_is_kept(ns, status):
             assert _status(pkg.op_sync) == status
         else:
             pkg.op_sync()
+
+
+# every variant of the linear: accumulating, wide stored tiles, and the CTA-pair kernel (split
+# activations of more than 64 rows), stored and accumulating
+@pytest.mark.parametrize("M,N,K,split,epi", [(64, 8192, 4096, True, 2), (100, 8192, 4096, False, 0),
+                                             (128, 8192, 4096, True, 0), (200, 8200, 4096, True, 2)])
+def test_bounded_wait_timeout_of_each_linear_kernel(M, N, K, split, epi):
+    g = torch.Generator().manual_seed(M)
+    X = torch.randn(M, K, generator=g)
+    hi = X.to(torch.bfloat16).cuda()
+    lo = (X.cuda() - hi.float()).to(torch.bfloat16) if split else None
+    W = (torch.randn(N, K, generator=g) * 0.02).to(torch.bfloat16).cuda()
+    ref = (hi.double() + (lo.double() if split else 0.0)) @ W.double().T
+    Y = torch.zeros(M, N, device="cuda")
+    pkg.op_sync()  # nothing pending
+    for _ in range(3):
+        try:
+            pkg.set_wait_limit(2)
+            pkg.op_linear(hi, W, Y, epi=epi, out_f32=True, X_lo=lo)
+        finally:
+            pkg.set_wait_limit(0)
+        assert _status(pkg.op_sync) == ETIMEDOUT
+        Y.zero_()
+        pkg.op_linear(hi, W, Y, epi=epi, out_f32=True, X_lo=lo)
+        pkg.op_sync()
+        assert float((Y.double() - ref).abs().max() / ref.abs().max()) <= 1e-4
