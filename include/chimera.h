@@ -51,7 +51,8 @@ typedef enum {
   CHIMERA_ENOMEM = -2,     /* device allocation failed */
   CHIMERA_ECAPACITY = -3,  /* a sequence would exceed max_seq_len KV slots */
   CHIMERA_ECUDA = -4,      /* a CUDA call or kernel failed */
-  CHIMERA_ETIMEDOUT = -5,  /* a bounded device-side wait gave up */
+  CHIMERA_ETIMEDOUT = -5,  /* a bounded device-side wait gave up; a context clears its caches
+                              and needs a new prefill (its steps return ESTATE until then) */
   CHIMERA_ESTATE = -6      /* call out of order (e.g. step before prefill) */
 } chimera_status;
 
@@ -240,6 +241,11 @@ chimera_status chimera_debug_override_tree(chimera_ctx* ctx, const int32_t* node
 
 /* Replace the root token x[n] of every sequence (host int32 [batch]). */
 chimera_status chimera_debug_set_root(chimera_ctx* ctx, const int32_t* roots);
+
+/* Leave the context as a launch whose bounded wait gave up may leave it: the error flagged on
+ * the device, arrival counters raised by one, KV rows and cached trigram rows that are no
+ * numbers.  The next call that waits for the device returns CHIMERA_ETIMEDOUT. */
+chimera_status chimera_debug_inject_timeout(chimera_ctx* ctx);
 
 enum {
   CHIMERA_DBG_NODE_TOKENS = 1,    /* int32 [batch][N] tree tokens of the last step */

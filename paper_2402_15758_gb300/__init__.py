@@ -74,6 +74,7 @@ _SIGS = {
     "chimera_profile_kind": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int] + [ctypes.c_void_p] * 3),
     "chimera_debug_override_tree": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "chimera_debug_set_root": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
+    "chimera_debug_inject_timeout": (ctypes.c_int, [ctypes.c_void_p]),
     "chimera_debug_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t]),
     "chimera_debug_read_kv": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                              ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
@@ -279,6 +280,10 @@ class Chimera:
     def set_root(self, roots):
         a = np.ascontiguousarray(np.asarray(roots, np.int32))
         self._check(self.lib.chimera_debug_set_root(self.h, a.ctypes.data))
+
+    def inject_timeout(self):
+        """The state that a launch which gave up may leave; the next sync raises ETIMEDOUT."""
+        self._check(self.lib.chimera_debug_inject_timeout(self.h))
 
     def read(self, what: str):
         """Copy a debug buffer to the host (numpy; bf16 buffers come back as float32)."""

@@ -8,6 +8,7 @@
 #include <functional>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/chimera.h"
@@ -1129,6 +1130,29 @@ chimera_status flush_page_table(chimera_ctx* ctx) {
   return CHIMERA_OK;
 }
 
+// Zero what a context keeps from one call to the next and from one prompt to the next: the KV
+// pools (rows past a sequence's last one are read, masked, and must be finite), the arrival
+// counters, which every launch leaves at zero, and the trigram cache.
+cudaError_t clear_kept_state(chimera_ctx* ctx) {
+  const size_t pool = static_cast<size_t>(ctx->kv_layer_stride) * ctx->kv_esz, entries = ctx->tc_entries;
+  const std::pair<void*, size_t> kept[] = {
+      {ctx->kv, pool * ctx->L},
+      {ctx->dkv, pool},
+      {ctx->att_cnt, static_cast<size_t>(ctx->Bmax) * ctx->H * sizeof(int)},
+      {ctx->topk_cnt, ctx->Bmax * sizeof(int)},
+      {ctx->lin_cnt, tc_max_tiles() * sizeof(int)},
+      {ctx->chain_bars, static_cast<size_t>(CHAIN_BAR_BLOCKS) * CHAIN_BAR_INTS * sizeof(int)},
+      {ctx->tc_keys, entries * sizeof(unsigned long long)},
+      {ctx->tc_stamp, entries * sizeof(int)},
+      {ctx->tc_clock, sizeof(int)},
+  };
+  for (const auto& [ptr, bytes] : kept) {
+    const cudaError_t e = ptr ? cudaMemsetAsync(ptr, 0, bytes, ctx->stream) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 chimera_status check_err(chimera_ctx* ctx) {
   int e = 0;
   CK(cudaMemcpyAsync(&ctx->h_stage[0], ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1136,10 +1160,13 @@ chimera_status check_err(chimera_ctx* ctx) {
   e = ctx->h_stage[0];
   if (e == 0) return CHIMERA_OK;
   CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
-  if ((e & ERR_TIMEOUT) && ctx->chain_bars)  // an aborted chain can leave step counters raised
-    CK(cudaMemsetAsync(ctx->chain_bars, 0, static_cast<size_t>(CHAIN_BAR_BLOCKS) * CHAIN_BAR_INTS * sizeof(int),
-                       ctx->stream));
-  if (e & ERR_TIMEOUT) return fail(ctx, CHIMERA_ETIMEDOUT, "a bounded device wait timed out");
+  if (e & ERR_TIMEOUT) {
+    // a launch that gave up leaves counters raised, and rows of unfinished sums in the caches;
+    // the plans and step graphs hold neither
+    ctx->prefilled = false;
+    CK(clear_kept_state(ctx));
+    return fail(ctx, CHIMERA_ETIMEDOUT, "a bounded device wait timed out: prefill again");
+  }
   if (e & ERR_CAPACITY) return fail(ctx, CHIMERA_ECAPACITY, "a kernel hit the KV capacity bound");
   return fail(ctx, CHIMERA_EINVAL, "a kernel saw an out-of-range token id or index");
 }
@@ -1436,16 +1463,8 @@ chimera_status chimera_init(const chimera_config* cfg, const chimera_weights* w,
   // zero-initialised state and scratch
   cudaStream_t s = ctx->stream;
   bool zok = true;
-  zok = zok && cudaMemsetAsync(ctx->kv, 0, static_cast<size_t>(ctx->kv_layer_stride) * ctx->L * ctx->kv_esz, s) == cudaSuccess;
-  zok = zok && cudaMemsetAsync(ctx->dkv, 0, static_cast<size_t>(ctx->kv_layer_stride) * ctx->kv_esz, s) == cudaSuccess;
-  zok = zok && cudaMemsetAsync(ctx->att_cnt, 0, static_cast<size_t>(B) * ctx->H * sizeof(int), s) == cudaSuccess;
-  zok = zok && cudaMemsetAsync(ctx->topk_cnt, 0, static_cast<size_t>(B) * sizeof(int), s) == cudaSuccess;
-  if (ctx->lin_cnt)
-    zok = zok && cudaMemsetAsync(ctx->lin_cnt, 0, static_cast<size_t>(tc_max_tiles()) * sizeof(int), s) == cudaSuccess;
+  zok = zok && clear_kept_state(ctx) == cudaSuccess;
   zok = zok && cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s) == cudaSuccess;
-  if (ctx->chain_bars)
-    zok = zok && cudaMemsetAsync(ctx->chain_bars, 0, static_cast<size_t>(CHAIN_BAR_BLOCKS) * CHAIN_BAR_INTS * sizeof(int),
-                                 s) == cudaSuccess;
   zok = zok && cudaMemsetAsync(ctx->d_ovr_flag, 0, sizeof(int), s) == cudaSuccess;
   zok = zok && cudaMemsetAsync(ctx->d_step, 0, sizeof(int), s) == cudaSuccess;
   zok = zok && cudaMemsetAsync(ctx->d_topk, 0, static_cast<size_t>(B) * K * ctx->KMAX * sizeof(int), s) == cudaSuccess;
@@ -1479,12 +1498,8 @@ chimera_status chimera_init(const chimera_config* cfg, const chimera_weights* w,
   zok = zok && cudaMemsetAsync(ctx->d_child_start1, 0, 2 * sizeof(int), s) == cudaSuccess;
   zok = zok && cudaMemsetAsync(ctx->d_child1, 0, sizeof(int), s) == cudaSuccess;
   zok = zok && cudaMemcpyAsync(ctx->d_parent, t.parent.data(), N * sizeof(int), cudaMemcpyHostToDevice, s) == cudaSuccess;
-  if (ctx->tc_entries) {
-    zok = zok && cudaMemsetAsync(ctx->tc_keys, 0, ctx->tc_entries * sizeof(unsigned long long), s) == cudaSuccess;
-    zok = zok && cudaMemsetAsync(ctx->tc_stamp, 0, ctx->tc_entries * sizeof(int), s) == cudaSuccess;
-    zok = zok && cudaMemsetAsync(ctx->tc_clock, 0, sizeof(int), s) == cudaSuccess;
+  if (ctx->tc_entries)
     zok = zok && cudaMemsetAsync(ctx->tc_hit_log, 0, static_cast<size_t>(K) * B * sizeof(int), s) == cudaSuccess;
-  }
   zok = zok && cudaStreamSynchronize(s) == cudaSuccess;
   if (!zok) {
     free_ctx(ctx);
@@ -1846,6 +1861,22 @@ chimera_status chimera_debug_set_root(chimera_ctx* ctx, const int32_t* roots) {
     CK(cudaMemcpy(ctx->d_tok + static_cast<size_t>(b) * ctx->tok_stride + ctx->host_n[b], &roots[b], sizeof(int),
                   cudaMemcpyHostToDevice));
   }
+  return CHIMERA_OK;
+}
+
+chimera_status chimera_debug_inject_timeout(chimera_ctx* ctx) {
+  if (!ctx) return CHIMERA_EINVAL;
+  CK(cudaStreamSynchronize(ctx->stream));
+  const std::vector<int> ones(std::max(tc_max_tiles(), ctx->Bmax * ctx->H), 1);
+  const int err = ERR_TIMEOUT;
+  const auto kv_bytes = static_cast<size_t>(ctx->kv_layer_stride) * ctx->kv_esz;
+  CK(cudaMemset(ctx->kv, 0xff, kv_bytes * ctx->L));
+  CK(cudaMemset(ctx->dkv, 0xff, kv_bytes));
+  if (ctx->tc_vals) CK(cudaMemset(ctx->tc_vals, 0xff, static_cast<size_t>(ctx->tc_entries) * ctx->d * sizeof(float)));
+  if (ctx->lin_cnt) CK(cudaMemcpy(ctx->lin_cnt, ones.data(), tc_max_tiles() * sizeof(int), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(ctx->att_cnt, ones.data(), static_cast<size_t>(ctx->Bmax) * ctx->H * sizeof(int), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(ctx->d_err, &err, sizeof(int), cudaMemcpyHostToDevice));
+  CK(cudaDeviceSynchronize());
   return CHIMERA_OK;
 }
 

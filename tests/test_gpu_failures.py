@@ -157,3 +157,33 @@ def test_bounded_wait_timeout_of_each_linear_kernel(M, N, K, split, epi):
         pkg.op_linear(hi, W, Y, epi=epi, out_f32=True, X_lo=lo)
         pkg.op_sync()
         assert float((Y.double() - ref).abs().max() / ref.abs().max()) <= 1e-4
+
+
+# after a timeout a prompt runs as in a new context: arrival counters at zero (the trigram
+# linears' tiles are cut between CTAs), no cached trigram row or KV row of unfinished sums
+@pytest.mark.parametrize("cache", [0, 256])
+def test_context_recovers_from_a_timeout(cache):
+    cfg = dict(synth.get_config("mini"), n_layers=1, d_model=1024, n_heads=8, vocab=1024, tree_nodes=16,
+               trigram_cache=cache)
+    w = {k: v.cuda() for k, v in synth.make_weights(cfg).items()}
+    prompt = synth.make_prompts(cfg)[0]
+    ctx = pkg.Chimera(cfg, w, max_batch=1, max_seq_len=256)
+
+    def run():
+        ctx.prefill([prompt])
+        out = []
+        for _ in range(3):
+            tokens = ctx.step()[0]
+            out.append((tokens, ctx.read("draft_logits").copy(), ctx.read("verify_logits").copy()))
+        return out
+
+    ref = run()
+    ctx.inject_timeout()
+    assert _status(ctx.sync) == ETIMEDOUT
+    assert _status(ctx.step) == ESTATE
+    for (tok, dl, vl), (rtok, rdl, rvl) in zip(run(), ref):
+        assert tok == rtok
+        # the order of the sums' reductions alone differs
+        assert np.max(np.abs(dl - rdl)) <= 1e-4 * np.max(np.abs(rdl))
+        assert np.max(np.abs(vl - rvl)) <= 1e-4 * np.max(np.abs(rvl))
+    ctx.close()
