@@ -104,10 +104,13 @@ int tc_max_tiles();
 // Returns 0 on success, otherwise a negative code and a message in `msg`.
 // W2 (optional, N2 rows): a second weight matrix whose outputs follow W's in Y (one
 // launch for two projections of the same input, e.g. SwiGLU gate and up); needs N % 128 == 0.
+// A stored output of up to 64 rows is cut into parts that depend on the rows' token tile;
+// with cut_rows set they are those of cut_rows rows, so that a row has the same bits in
+// every batch.
 int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const void* X_lo, int ldx,
                    const void* W, void* Y, void* Y_lo, int ldy, int epi, int out_f32, float* ws,
                    int* counters, int* err, char* msg, size_t msg_len, const void* W2 = nullptr, int N2 = 0,
-                   float* zero = nullptr, long long zero_floats = 0);
+                   float* zero = nullptr, long long zero_floats = 0, int cut_rows = 0);
 cudaError_t tc_linear_launch(const TcLinearPlan& plan, cudaStream_t s);
 
 // Error word of the allocation-free linear's static scratch on the current device:

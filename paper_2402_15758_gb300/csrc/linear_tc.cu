@@ -687,7 +687,7 @@ static int stored_grid(int tiles, int kblocks, int bn, int sms) {
 int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const void* X_lo, int ldx,
                    const void* W, void* Y, void* Y_lo, int ldy, int epi, int out_f32, float* ws,
                    int* counters, int* err, char* msg, size_t msg_len, const void* W2, int N2,
-                   float* zero, long long zero_floats) {
+                   float* zero, long long zero_floats, int cut_rows) {
   auto fail = [&](const char* m) {
     if (msg && msg_len) snprintf(msg, msg_len, "linear(M=%d,N=%d,K=%d): %s", M, N, K, m);
     return -1;
@@ -750,7 +750,8 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   const int sms = tc_num_sms() * CTAS_PER_SM;
   plan->grid = static_cast<int>(p.units < sms ? p.units : sms);
   p.cut = p.has_lo || p.units >= 2ll * sms ? 2 : 1;
-  if (epi != EPI_RESID && p.BN <= CUT_COLS) plan->grid = stored_grid(p.feat_tiles * p.tok_tiles, p.kblocks, p.BN, sms);
+  if (epi != EPI_RESID && p.BN <= CUT_COLS)
+    plan->grid = stored_grid(p.feat_tiles * p.tok_tiles, p.kblocks, cut_rows ? (cut_rows + 15) / 16 * 16 : p.BN, sms);
   // float4 reductions need 16-byte aligned rows of Y and whole float4 runs of features
   p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && N % 4 == 0) ? 1 : 0;
   plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 32 * RED_PITCH * sizeof(float);

@@ -106,6 +106,23 @@ def test_mini_trigram_cache_rows_match():
     ctx.close()
 
 
+def test_trigram_rows_are_the_same_in_every_batch():
+    # the cache is kept from one prompt to the next, also when the batch changes
+    cfg, _, w_dev = _setup("mini", trigram_cache=64, n_layers=1, d_model=1024, n_heads=8, tree_nodes=16, batch=1)
+    prompt = synth.make_prompts(cfg)[0]
+    rows = []
+    for batch in (1, 16, 20, 40, 64):
+        prompts = [prompt] + [prompt[i:] + prompt[:i] for i in range(1, batch)]
+        ctx = pkg.Chimera(cfg, w_dev, max_batch=64, max_seq_len=192)  # an empty cache
+        ctx.prefill(prompts)
+        ctx.set_root([7 + i for i in range(batch)])
+        ctx.step()
+        rows.append(ctx.read("htri")[0, 0].copy())
+        ctx.close()
+    for r in rows[1:]:
+        np.testing.assert_array_equal(r, rows[0])
+
+
 # ----------------------------------------------------------------------------
 # typical acceptance
 # ----------------------------------------------------------------------------
