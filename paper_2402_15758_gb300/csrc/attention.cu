@@ -108,27 +108,35 @@ __device__ void combine_splits(const AttnParams& p, const float* wsb, int nq, in
   }
 }
 
-// Four consecutive elements of a KV row as fp32 (split planes: hi + lo); one element at a
-// time when the pool is not aligned for vectors.
-__device__ __forceinline__ float4 load_row4(const float* p, bool vec) {
-  return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
-}
-__device__ __forceinline__ float4 load_row4(const bf16* p, bool vec) {
-  if (!vec) return make_float4(to_f(p[0]), to_f(p[1]), to_f(p[2]), to_f(p[3]));
-  const uint2 u = *reinterpret_cast<const uint2*>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
+// Four consecutive elements of a KV row as loaded, one element at a time when the pool is not
+// aligned for vectors, and their values.
 template <typename TKV>
-__device__ __forceinline__ float4 load_kv4(const TKV* p, int lo_ofs, bool vec) {
-  float4 v = load_row4(p, vec);
-  if (lo_ofs) {
-    const float4 w = load_row4(p + lo_ofs, vec);
-    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+struct Raw4;
+template <>
+struct Raw4<float> {
+  float4 v;
+  __device__ __forceinline__ void load(const float* p, bool vec) {
+    v = vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
   }
-  return v;
-}
+  __device__ __forceinline__ float4 value() const { return v; }
+};
+template <>
+struct Raw4<bf16> {
+  uint2 v;
+  __device__ __forceinline__ void load(const bf16* p, bool vec) {
+    if (vec) {
+      v = *reinterpret_cast<const uint2*>(p);
+    } else {
+      const unsigned short* u = reinterpret_cast<const unsigned short*>(p);
+      v = make_uint2(u[0] | static_cast<uint32_t>(u[1]) << 16, u[2] | static_cast<uint32_t>(u[3]) << 16);
+    }
+  }
+  __device__ __forceinline__ float4 value() const {
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+};
 
 // Sum v[0..NV) over each half-warp (NV <= 16): lane l returns the total of value
 // (l % 16) / (16 / NV); every step halves the values a lane still holds.
@@ -155,7 +163,11 @@ __device__ __forceinline__ float half_sum_many(float (&v)[NV], int lane) {
 // lanes per row, with the K and V of all four in flight at once, and scores them against
 // QG queries from shared memory; the 16 partial sums of a query group are reduced
 // together, and a lane keeps the running max and sum of one query.  No tile is staged and
-// the warps meet once, at the end.  More queries than QG are further CTAs.  Measured (GB300,
+// the warps meet once, at the end.  A CTA takes one query, up to 8, or up to 16 (8 at 128 dims);
+// more queries are further CTAs.  (Every query of the group costs its products: 8 queries at 200
+// rows, fp32, 15.5 us in a group of 16, 12.6 in one of 8.  bf16 pools took 18.6 and at 4000 rows, 8
+// sequences of 16 heads, 378 with a branch on the pool's form around each load, which kept
+// the next ones waiting; now 12.6 and 140.  16 queries: 18.9 -> 15.7.)  Measured (GB300,
 // fp32, 4 heads of 64, an event pair around every launch): one query at 70 rows 19 -> 9 us,
 // 16 tree rows 17 -> 13; a 64-token prompt and eight steps 2.70 -> 2.26 ms.  The kernel
 // before staged 32-key tiles for all queries, kept seven of eight warps idle for one
@@ -171,6 +183,7 @@ __global__ void __launch_bounds__(THREADS) attn_kernel(const AttnParams p, int g
   pdl_wait();     // inputs of this kernel are complete
   constexpr int DV = HD / 64;        // float4 of a row per lane
   constexpr int LPQ = 16 / QG;       // lanes that hold the same query's state
+  constexpr bool LO = !std::is_same_v<TKV, float>;  // the pool may hold lo planes
   __shared__ __align__(16) float qs[QG * HD];
   __shared__ __align__(16) float s_acc[WARPS * 1024];  // [WARPS][QG][HD], later combine_splits' weights
   __shared__ float s_m[WARPS * QG], s_l[WARPS * QG];
@@ -258,17 +271,56 @@ __global__ void __launch_bounds__(THREADS) attn_kernel(const AttnParams p, int g
 
   for (int base = k0; base < k1; base += KEYS) {
     // key base + 16 u + hw: row hw of page base / 16 + u
-    float4 kk[4][DV], vv[4][DV];
+    // (the branches on the pool's form surround all loads of a pass, and nothing is converted
+    // before the last one is on its way)
+    const TKV* row[4];
+    bool in[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const bool in = base + 16 * u + hw < k1;
-      const int page = in ? p.page_table[b * p.max_pages + base / 16 + u] : 0;
-      const TKV* row = pool + (static_cast<size_t>(page) * p.H + h) * p.planes * 16 * HD + hw * HD + hl * 4;
+      in[u] = base + 16 * u + hw < k1;
+      const int page = in[u] ? p.page_table[b * p.max_pages + base / 16 + u] : 0;
+      row[u] = pool + (static_cast<size_t>(page) * p.H + h) * p.planes * 16 * HD + hw * HD + hl * 4;
+    }
+    auto load_rows = [&](Raw4<TKV>(&kr)[4][DV], Raw4<TKV>(&vr)[4][DV], int ofs, bool as_vec) {
 #pragma unroll
-      for (int d = 0; d < DV; ++d) {
-        kk[u][d] = in ? load_kv4(row + 64 * d, lo_ofs, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-        vv[u][d] = in ? load_kv4(row + v_ofs + 64 * d, lo_ofs, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+          kr[u][d] = vr[u][d] = Raw4<TKV>{};
+          if (in[u]) {
+            kr[u][d].load(row[u] + ofs + 64 * d, as_vec);
+            vr[u][d].load(row[u] + ofs + v_ofs + 64 * d, as_vec);
+          }
+        }
+    };
+    Raw4<TKV> kr[4][DV], vr[4][DV];
+    if (vec)
+      load_rows(kr, vr, 0, true);
+    else
+      load_rows(kr, vr, 0, false);
+    float4 kk[4][DV], vv[4][DV];
+    auto add4 = [](float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); };
+    if (LO && lo_ofs) {
+      Raw4<TKV> kl[4][DV], vl[4][DV];
+      if (vec)
+        load_rows(kl, vl, lo_ofs, true);
+      else
+        load_rows(kl, vl, lo_ofs, false);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+          kk[u][d] = add4(kr[u][d].value(), kl[u][d].value());
+          vv[u][d] = add4(vr[u][d].value(), vl[u][d].value());
+        }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+          kk[u][d] = kr[u][d].value();
+          vv[u][d] = vr[u][d].value();
+        }
     }
     float part[4][QG];
 #pragma unroll
@@ -410,15 +462,16 @@ cudaError_t launch(AttnParams p, cudaStream_t s) {
   p.splits = std::max(1, std::min(p.splits, (p.max_pages * 16 + SPLIT_KEYS - 1) / SPLIT_KEYS));
   const int groups = p.nq_max == 1 ? 1 : (p.nq_max + QG - 1) / QG;
   const dim3 grid(p.splits, p.H, p.B * std::max(1, p.q_blocks) * groups);
+  auto* kernel = p.nq_max == 1   ? attn_kernel<TKV, T, HD, 1, false>
+                 : p.nq_max <= 8 ? attn_kernel<TKV, T, HD, 8, false>
+                                 : attn_kernel<TKV, T, HD, QG, false>;
   if constexpr (std::is_same_v<TKV, float>) {
-    if (p.qkv) {
-      launch_pdl(p.nq_max == 1 ? attn_kernel<TKV, T, HD, 1, true> : attn_kernel<TKV, T, HD, QG, true>, grid, dim3(THREADS),
-                 0, s, p, groups);
-      return cudaGetLastError();
-    }
+    if (p.qkv)
+      kernel = p.nq_max == 1   ? attn_kernel<TKV, T, HD, 1, true>
+               : p.nq_max <= 8 ? attn_kernel<TKV, T, HD, 8, true>
+                               : attn_kernel<TKV, T, HD, QG, true>;
   }
-  launch_pdl(p.nq_max == 1 ? attn_kernel<TKV, T, HD, 1, false> : attn_kernel<TKV, T, HD, QG, false>, grid, dim3(THREADS),
-             0, s, p, groups);
+  launch_pdl(kernel, grid, dim3(THREADS), 0, s, p, groups);
   return cudaGetLastError();
 }
 

@@ -330,6 +330,18 @@ def test_attention_tree_masked_paged(dtype, case):
 @pytest.mark.parametrize("nctx,nq,splits", [([0], 1, 1), ([64, 63], 1, 16), ([700, 5], 1, 3), ([130], 9, 2), ([300, 0], 64, 16)])
 @pytest.mark.parametrize("offset", [0, 1])
 def test_attention_simt(dtype, hd, nctx, nq, splits, offset):
+    _attention_simt(dtype, hd, nctx, nq, splits, offset)
+
+
+# groups of 8 queries, partly filled and full
+@pytest.mark.parametrize("dtype,hd", [("fp32", 64), ("bf16", 64), ("bf16_split", 64)])
+@pytest.mark.parametrize("nctx,nq,splits", [([0, 130], 2, 1), ([700, 5], 7, 3), ([300], 8, 16)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_attention_simt_few_queries(dtype, hd, nctx, nq, splits, offset):
+    _attention_simt(dtype, hd, nctx, nq, splits, offset)
+
+
+def _attention_simt(dtype, hd, nctx, nq, splits, offset):
     B, H, n_local = len(nctx), 3, max(nq, 2)
     rng = np.random.default_rng(nq + splits)
     max_pages = (max(nctx) + n_local + 15) // 16
