@@ -658,7 +658,7 @@ int tc_max_tiles() { return MAX_TILES; }
 // one, or two by two where a term more or the split had made the chains longer than that:
 // 1.3e-7 to 2.5e-7 everywhere, between 1.2e-7 and 2e-5 with equal stages.  That takes a
 // register per token column: wider tiles keep equal stages.
-static int stored_grid(int tiles, int kblocks, int bn, int sms) {
+static int stored_grid(int tiles, int kblocks, int bn, bool split, int sms) {
   auto stages = [](double n, int ctas) { return n * std::max(0.5, 0.005 * ctas); };
   const long long units = static_cast<long long>(tiles) * kblocks;
   int best = static_cast<int>(std::min<long long>(units, sms));
@@ -674,8 +674,11 @@ static int stored_grid(int tiles, int kblocks, int bn, int sms) {
       best = tiles * s;
     }
   }
-  for (int w = 2; w <= 8; ++w) {  // more tiles than SMs: w whole ones each, when that divides
-    const double t = tiles % w == 0 && tiles / w <= sms ? stages(static_cast<double>(w) * kblocks, tiles / w) : 1e30;
+  // More tiles than SMs: w whole ones each, when that divides.  (A split's stage takes 0.55 us:
+  // 1 and 64 x 22016 x 4096 35.3 and 46.1 us as 86 x 2 tiles, 32.3 and 42.1 as equal stages; 27648
+  // columns, 108 x 2, 36.7 and 48.3, 38.5 and 48.8.)
+  for (int w = 2; w <= 8; ++w) {
+    const double t = tiles % w == 0 && tiles / w <= sms ? w * kblocks * std::max(split ? 0.55 : 0.5, 0.005 * (tiles / w)) : 1e30;
     if (t < least) {
       least = t;
       best = tiles / w;
@@ -751,7 +754,7 @@ int tc_linear_plan(TcLinearPlan* plan, int M, int N, int K, const void* X, const
   plan->grid = static_cast<int>(p.units < sms ? p.units : sms);
   p.cut = p.has_lo || p.units >= 2ll * sms ? 2 : 1;
   if (epi != EPI_RESID && p.BN <= CUT_COLS)
-    plan->grid = stored_grid(p.feat_tiles * p.tok_tiles, p.kblocks, cut_rows ? (cut_rows + 15) / 16 * 16 : p.BN, sms);
+    plan->grid = stored_grid(p.feat_tiles * p.tok_tiles, p.kblocks, cut_rows ? (cut_rows + 15) / 16 * 16 : p.BN, p.has_lo, sms);
   // float4 reductions need 16-byte aligned rows of Y and whole float4 runs of features
   p.vec_red = (epi == EPI_RESID && (reinterpret_cast<uintptr_t>(Y) & 15) == 0 && ldy % 4 == 0 && N % 4 == 0) ? 1 : 0;
   plan->smem = 1024 + static_cast<size_t>(p.stages) * stage_bytes + 1024 + 4 * 32 * RED_PITCH * sizeof(float);
