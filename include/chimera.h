@@ -130,7 +130,10 @@ typedef struct {
 
 /* Create a context.  `cuda_stream` is a cudaStream_t (NULL: the context creates its
  * own non-blocking stream).  Validates shapes, records the weight pointers and
- * allocates the KV pools (max_batch * max_seq_len slots), scratch and the tree.
+ * allocates the KV pools (max_batch * max_seq_len slots), scratch and the tree.  The scratch
+ * holds one prefill pass: up to 1024 prompt rows (no more than max_batch * max_seq_len, at
+ * least 64 per sequence) of 44 d_model + 12 ffn_dim bytes each with precision 1, 320 MB for
+ * the 4096-wide model, besides 40 MB of partial sums and the logits.
  * It synchronizes the device first, so weights written by earlier work on any stream
  * are complete before the context reads them; the weights must not change while the
  * context lives.  EINVAL on bad shapes or a NULL weight, ENOMEM on allocation failure,
@@ -283,12 +286,13 @@ chimera_status chimera_debug_read_kv(chimera_ctx* ctx, int layer, int seq, int p
  * dtype 1: X, X_lo (optional, NULL = none), W bf16 (K, ldx multiples of 8; 16-byte
  * aligned), tcgen05 kernel; dtype 0: everything fp32, X_lo ignored.  epi 0: Y = acc,
  * 1: Y = SiLU(acc), 2: Y(fp32) += acc.  out_f32 selects an fp32 Y for epi 0/1 with
- * dtype 1.  Device pointers; X and W may be written by earlier work on the same stream,
- * calls of this function among it.  Calls on different streams may overlap: each of the
- * first eight streams of a device has a workspace of its own (107 MB, allocated on its first
- * call and kept), further streams share one and their calls run one after the other.
- * Calls captured into graphs share one more: replays that overlap on the GPU must be ordered
- * by the caller.  The same holds for chimera_op_attention.  Asynchronous: the status
+ * dtype 1.  A row's last bits may depend on M.  Device pointers; X and W may be written by
+ * earlier work on the same stream, calls of this function among it.  Calls on different
+ * streams may overlap: each of the first eight streams of a device has a workspace of its
+ * own (107 MB, allocated on its first call and kept), further streams share one and their
+ * calls run one after the other.  Calls captured into graphs share one more: replays that
+ * overlap on the GPU must be ordered by the caller.  The same holds for
+ * chimera_op_attention.  Asynchronous: the status
  * covers the arguments and the launch; what the kernel flags on the device (a bounded wait
  * that gave up) is reported by chimera_op_sync. */
 chimera_status chimera_op_linear(int dtype, int epi, int out_f32, int M, int N, int K,

@@ -198,8 +198,6 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: gives up after `limit_ns` (or as soon as *abort is set by another
-// role of the same CTA) and returns false; the caller records the error.
 // Bounded wait that ignores the abort flag (draining copies / MMAs in flight).
 __device__ __forceinline__ bool mbar_wait_plain(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
   const uint64_t t0 = global_timer_ns();
@@ -209,6 +207,8 @@ __device__ __forceinline__ bool mbar_wait_plain(uint64_t* bar, uint32_t parity, 
   return true;
 }
 
+// Bounded wait: gives up after `limit_ns` (or as soon as *abort is set by another
+// role of the same CTA) and returns false; the caller records the error.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           uint64_t limit_ns = 2000000000ull) {
   if (mbar_try_wait(bar, parity)) return true;

@@ -188,8 +188,10 @@ __device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
 // workspace path needs 70 more registers, and a CTA that holds them leaves the SM too
 // few for two CTAs of the row kernel that overlaps the launch (SwiGLU: 62 x 256; one
 // kernel for both made the linears 1 % faster and the step 1 % slower).
-// CUT: stored tiles of at most CUT_COLS columns, summed in registers from chains of p.cut
-// stages (see stored_grid); wider ones, and unaligned accumulation, drain one chain.
+// CUT: tiles of at most CUT_COLS columns, summed in registers from chains of p.cut stages (see
+// stored_grid); wider ones drain one chain.  Either way accumulation into rows that are not
+// aligned for vectors is one reduction per value.  (64 x 2050 x 4104 takes 10.0 us in short
+// chains, 8.9 in one, whose error is 2-4 times as large.)
 template <bool RED, bool CUT>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) tc_linear_kernel(const __grid_constant__ TcLinearParams p) {
   if (p.skip) {
@@ -650,9 +652,10 @@ int tc_max_tiles() { return MAX_TILES; }
 // CTAs of a linear that stores its output.  A tile cut between CTAs goes through the
 // workspace, which costs about 5 us and 0.011 us per part and token column; with every SM
 // taking the same number of stages two tiles are cut per CTA, one of them while stages are
-// left.  A stage takes 0.5 us, or what DRAM needs for one of every CTA.  So a tile goes to one CTA, or to as many as pay for themselves.  Equal stages / as
-// chosen here, us: 5 x 1000 x 520 6.2 / 4.8, 16 x 12288 x 4096 22.7 / 19.2, 64 x 1000 x 4096
-// 20.8 / 14.5, 64 x 4096 x 2560 22.1 / 15.7, 64 x 12288 x 4096 30.5 / 23.7.
+// left.  A stage takes 0.5 us, or what DRAM needs for one of every CTA.  So a tile goes to
+// one CTA, or to as many as pay for themselves.  Equal stages / as chosen here, us:
+// 5 x 1000 x 520 6.2 / 4.8, 16 x 12288 x 4096 22.7 / 19.2, 64 x 1000 x 4096 20.8 / 14.5,
+// 64 x 4096 x 2560 22.1 / 15.7, 64 x 12288 x 4096 30.5 / 23.7.
 // Longer parts are longer chains of tensor-core sums, which round toward zero (2.4e-10 per
 // K: 4.4e-6 at 12288 x 4096).  So the epilogue sums the stages of a part in registers, one by
 // one, or two by two where a term more or the split had made the chains longer than that:

@@ -223,7 +223,6 @@ struct chimera_ctx {
   void *tbuf = nullptr, *ubuf = nullptr, *ubuf_lo = nullptr, *headin = nullptr, *headin_lo = nullptr;
   float *hfull_log = nullptr, *hsel = nullptr, *kvtmp = nullptr;
   float *dres = nullptr, *hlog = nullptr;
-  bool tc_zero = false;  // tensor-core linears clear the next accumulators (see enqueue_layer)
 
   // scratch of the split kernels
   float* lin_ws = nullptr;
@@ -615,10 +614,9 @@ cudaError_t enqueue_layer(chimera_ctx* ctx, int l, const Lin* lin, int rows, int
                           const int* pos_off, const unsigned long long* anc, int splits, double kv_bytes) {
   const chimera_block_weights& w = ctx->layers[l];
   const int d = ctx->d;
-  // the accumulators of the QKV and gate|up linears are cleared by the norms, or (tensor-
-  // core linears) by the previous layer's down linear and this layer's O linear
-  const bool z = !ctx->tc_zero;
-  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.attn_norm, rows, (z || l == 0) ? ctx->qkv : nullptr, 3 * d));
+  // the accumulators of the QKV and gate|up linears are cleared by the previous layer's down
+  // linear (the first layer's by its norm) and by this layer's O linear
+  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.attn_norm, rows, l == 0 ? ctx->qkv : nullptr, 3 * d));
   RUN(run_lin(ctx, lin[0]));
   const int blocks = (rows_per_seq + CHUNK - 1) / CHUNK, nq = std::min(rows_per_seq, CHUNK);
   if (blocks == 1 && attn_fuses_rope(ctx->dtype, ctx->hd)) {
@@ -630,7 +628,7 @@ cudaError_t enqueue_layer(chimera_ctx* ctx, int l, const Lin* lin, int rows, int
                       nullptr, blocks));
   }
   RUN(run_lin(ctx, lin[1]));
-  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.ffn_norm, rows, z ? ctx->gu : nullptr, 2 * ctx->F));
+  if (!folds(ctx)) RUN(run_norm(ctx, ctx->x, w.ffn_norm, rows, nullptr, 0));
   RUN(run_lin(ctx, lin[2]));
   RUN(run_lin(ctx, lin[3]));
   if (!folds_swiglu(ctx, rows))
@@ -1024,7 +1022,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
       // the O linear clears the gate|up accumulator of this layer, the down linear the
       // QKV accumulator of the next one (their epilogue warps, off the critical path)
       if (!make_lin(ctx, &p[1], M, d, d, ao, al, d, w.wo, ctx->x, nullptr, d, ACC, f32, nullptr, 0,
-                    ctx->tc_zero ? ctx->gu : nullptr, static_cast<long long>(M) * 2 * F))
+                    ctx->gu, static_cast<long long>(M) * 2 * F))
         return false;
       // gate and up: one launch writing gu[:, 0:F] and gu[:, F:2F]
       if (!make_lin(ctx, &p[2], M, F, d, xn, xl, d, w.w_gate, ctx->gu, nullptr, 2 * F, OUT, f32, w.w_up, F))
@@ -1032,7 +1030,7 @@ bool build_plans(chimera_ctx* ctx, int B) {
       fold_norm(ctx, &p[2], ctx->x, w.ffn_norm);
       p[3] = Lin();  // N = 0: nothing to launch
       if (!make_lin(ctx, &p[4], M, d, F, hf, hl, F, w.w_down, ctx->x, nullptr, d, ACC, f32, nullptr, 0,
-                    ctx->tc_zero ? ctx->qkv : nullptr, static_cast<long long>(M) * 3 * d))
+                    ctx->qkv, static_cast<long long>(M) * 3 * d))
         return false;
       fold_swiglu(ctx, &p[4]);
     }
@@ -1381,7 +1379,6 @@ chimera_status chimera_init(const chimera_config* cfg, const chimera_weights* w,
   ok = ok && dalloc_bytes(ctx, &ctx->xn, Rx * d * ctx->esz);
   if (sp) ok = ok && dalloc_bytes(ctx, &ctx->xn_lo, Rx * d * ctx->esz);
   ok = ok && dalloc(ctx, &ctx->qkv, static_cast<size_t>(ctx->R) * 3 * d);
-  ctx->tc_zero = ctx->dtype == 1;
   ok = ok && dalloc(ctx, &ctx->qr, static_cast<size_t>(ctx->R) * d);
   ok = ok && dalloc_bytes(ctx, &ctx->ao, static_cast<size_t>(ctx->R) * d * ctx->esz);
   if (sp) ok = ok && dalloc_bytes(ctx, &ctx->ao_lo, static_cast<size_t>(ctx->R) * d * ctx->esz);
